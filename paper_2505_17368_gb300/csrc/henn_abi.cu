@@ -495,8 +495,7 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
   const int32_t dpad = ix->dpad, M = ix->M;
   Scratch sc(st);
   // insertion order and centred operand
-  int64_t chunks = (s + 4095) / 4096;
-  float* partial = sc.get<float>((size_t)chunks * dpad);
+  float* partial = sc.get<float>((size_t)mean_chunks(s) * dpad);
   float* mean = sc.get<float>(dpad);
   launch_layer_mean(ix->xw, Ly.ids, s, dpad, partial, mean, st);
   int32_t* inv = sc.get<int32_t>(s);
@@ -1112,7 +1111,7 @@ const henn_index::EntryOps& entry_ops(const henn_index* idx, int32_t li, cudaStr
   float* rows = sc.get<float>((size_t)s * dpad);
   CK(launch_layer_rows_f32(Ly.vec, Ly.vscale, s, idx->storage, dpad, rows, st));
   e.mean = static_cast<float*>(get(sizeof(float) * dpad));
-  float* partial = sc.get<float>((size_t)((s + 4095) / 4096) * dpad);
+  float* partial = sc.get<float>((size_t)mean_chunks(s) * dpad);
   launch_layer_mean(rows, nullptr, s, dpad, partial, e.mean, st);
   int32_t* inv = sc.get<int32_t>(s);
   float* xo = sc.get<float>((size_t)s * dpad);

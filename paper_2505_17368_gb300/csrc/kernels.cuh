@@ -50,7 +50,8 @@ void launch_inv_norms(const float* x32, int64_t n, int32_t dpad, float* inv_norm
 void launch_normalise(const float* x32, const float* inv_norm, int64_t n, int32_t dpad, float* xn,
                       cudaStream_t st);
 // mean over the rows listed in ids (or rows 0..s-1): partial buffer of
-// ceil(s/4096) * dpad floats
+// mean_chunks(s) * dpad floats (16-byte aligned, as are the rows)
+int64_t mean_chunks(int64_t s);
 void launch_layer_mean(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, float* partial,
                        float* mean, cudaStream_t st);
 // insertion order: rank[j] = perm(j), inv[rank] = j; xo[rank] = xw[ids[j]] - mean; norms
