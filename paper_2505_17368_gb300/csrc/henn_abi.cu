@@ -363,7 +363,7 @@ int32_t build_layer_membership(henn_index* ix, const henn_build_params& p, int32
   float* lo = sc.get<float>(r);
   float* hi = sc.get<float>(r);
   int32_t* status = sc.get<int32_t>(r);
-  float* D = (w <= s) ? sc.get<float>((size_t)r * s) : nullptr;
+  float* D = (w <= s) ? sc.get<float>((size_t)r * ring_ld(s)) : nullptr;
   double* D64 = nullptr;
   double* bounds = sc.get<double>(2);
   // certified FP32 error model of the ring distances (see layers.cu)

@@ -7,7 +7,6 @@
 
 namespace henn {
 
-constexpr int kMaxDimPerLane = 32;  // dpad <= 1024 (dpad = d rounded up to 32)
 constexpr int kMaxD = 1024;
 
 enum RingStatus : int32_t { kRingPass = 1, kRingFail = 2, kRingAmbiguous = 3 };
@@ -28,6 +27,9 @@ void launch_offsets(const int32_t* counts, int64_t s, int64_t* tile_buf, int64_t
                     cudaStream_t st);
 void launch_ring_params(uint64_t bc, uint64_t bs, int32_t r, int64_t s, int64_t span, int32_t* centre,
                         int64_t* start, cudaStream_t st);
+// D: r rows of ring_ld(s) floats (16-byte aligned), the distances of ring
+// centre q to the layer's s points in row q
+int64_t ring_ld(int64_t s);
 void launch_ring_dist(const float* x32, int32_t dpad, const int32_t* prev_ids, int64_t s,
                       const int32_t* centre, int32_t r, int32_t metric, const float* inv_norm, float* D,
                       cudaStream_t st);
