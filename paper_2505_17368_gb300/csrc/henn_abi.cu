@@ -488,6 +488,53 @@ void build_membership(henn_index* ix, const henn_build_params& p, int32_t first_
   CK(cudaStreamSynchronize(st));
 }
 
+// Columns that a CTA of the collecting tile pass keeps for one row; a row
+// with more goes to the exact scan.
+constexpr int32_t kCollectCap = 256;
+
+// Forward lists of the rows that their candidate lists left open (nflagged of
+// them, listed in f): a second tile pass over those rows alone collects every
+// column that can belong to a list (its tile distance is at or under the
+// row's f.thr), and the exact FP32 rerank of these gives the list.  Rows with
+// too many such columns (massive ties) are scanned exactly.  Without this
+// pass the scan took them all: 52.9 of 74 ms of a 100,000 x 960 build.
+// hi / lo / norms: planes of the rows f refers to (nb: the columns, their
+// planes and norms b_*); row r may take columns below row0 + r (causal) or
+// all but itself.
+void settle_flagged(henn_index* ix, const LayerDev& Ly, int64_t s, const FlaggedRows& f, int32_t nflagged, int64_t row0,
+                    int32_t mode, const int32_t* ids, const int32_t* inv, const void* hi, const void* lo,
+                    const float* norms, const void* b_hi, const void* b_lo, const float* b_norms, int32_t dk,
+                    Scratch& sc, cudaStream_t st) {
+  const int64_t nf = nflagged;
+  void* fhi = sc.get<uint16_t>((size_t)nf * dk);
+  void* flo = sc.get<uint16_t>((size_t)nf * dk);
+  float* fnorms = sc.get<float>(nf);
+  int32_t* lim = sc.get<int32_t>(nf);
+  int32_t* self = sc.get<int32_t>(nf);
+  const unsigned grid = tile_collect_grid(nf);
+  uint32_t* cols = sc.get<uint32_t>((size_t)grid * kTileRows * kCollectCap);
+  int32_t* ncols = sc.get<int32_t>((size_t)grid * kTileRows);
+  int32_t* over = sc.get<int32_t>((size_t)nf + 2);  // their number, the rows, and the tile launch's error flag
+  int32_t* err = over + nf + 1;
+  CK(cudaMemsetAsync(over, 0, sizeof(int32_t), st));
+  CK(cudaMemsetAsync(err, 0, sizeof(int32_t), st));
+  launch_gather_flagged(f, nf, row0, mode == 0, mode == 1, s, hi, lo, norms, dk, fhi, flo, fnorms, lim, self, st);
+  CK(launch_tile_collect_tc(fhi, flo, fnorms, nf, b_hi, b_lo, b_norms, s, dk, lim, self, f.thr, f.count, grid, cols,
+                            ncols, kCollectCap, err, st));
+  launch_rerank_collected_fwd(ix->xw, ids, f, nf, row0, ix->dpad, ix->metric, inv, s, grid, cols, ncols, kCollectCap,
+                              ix->M, Ly.fwd, Ly.fwd_d, over, err, st);
+  CKL("collected rows");
+  int32_t nover = 0, herr = 0;
+  CK(cudaMemcpyAsync(&nover, over, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  if (herr) throw Failure(HENN_ERR_TIMEOUT, "tensor-core tile pipeline wait timed out (code " + std::to_string(herr) + ")");
+  if (nover > 0) {
+    launch_exact_rows(ix->xw, ids, s, ix->dpad, ix->metric, inv, mode, over + 1, nover, ix->M, Ly.fwd, Ly.fwd_d, st);
+    CKL("exact rows");
+  }
+}
+
 void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, CapturedGraph& graph, cudaStream_t st,
                        BuildTrace& tr) {
   LayerDev& Ly = ix->layers[li];
@@ -499,40 +546,50 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
   float* mean = sc.get<float>(dpad);
   launch_layer_mean(ix->xw, Ly.ids, s, dpad, partial, mean, st);
   int32_t* inv = sc.get<int32_t>(s);
-  float* xo = sc.get<float>((size_t)s * dpad);
   float* norms = sc.get<float>(s);
-  launch_order_gather(ix->xw, Ly.ids, s, dpad, ix->seed, li, ix->graph, mean, inv, xo, norms, st);
-  CKL("order/gather");
   float* nmax = sc.get<float>(1);
-  launch_max_nonneg(norms, s, nmax, st);
-  tr.mark("mean/order/norms", li);
-  // tiles + top-KP
   const int32_t KP = M <= 16 ? 32 : (M <= 48 ? 64 : 128);
-  uint64_t* cand = sc.get<uint64_t>((size_t)s * KP);
   const int32_t mode = ix->graph == HENN_GRAPH_KNN ? 1 : 0;
   const bool tc_ok = tc_tiles_supported(dpad, KP);
   if (p.tiles == HENN_TILES_TCGEN05 && !tc_ok)
     throw Failure(HENN_ERR_UNSUPPORTED, "tcgen05 tiles need M <= 16");
   const bool use_tc = tc_ok && p.tiles != HENN_TILES_SIMT;
+  const int32_t dk = round_up(dpad, 64);
+  float* xo = nullptr;
+  void* hi = nullptr;
+  void* lo = nullptr;
+  if (use_tc) {
+    hi = sc.get<uint16_t>((size_t)s * dk);
+    lo = sc.get<uint16_t>((size_t)s * dk);
+    launch_order_split(ix->xw, Ly.ids, s, dpad, ix->seed, li, mode == 1, mean, dk, hi, lo, inv, norms, nullptr, nmax, st);
+  } else {
+    xo = sc.get<float>((size_t)s * dpad);
+    launch_order_gather(ix->xw, Ly.ids, s, dpad, ix->seed, li, ix->graph, mean, inv, xo, norms, st);
+    launch_max_nonneg(norms, s, nmax, st);
+  }
+  CKL("order/gather");
+  tr.mark("mean/order/norms", li);
+  // tiles + top-KP
+  uint64_t* cand = sc.get<uint64_t>((size_t)s * KP);
   double tile_u;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   CK(cudaEventCreate(&ev0));
   CK(cudaEventCreate(&ev1));
   CK(cudaEventRecord(ev0, st));
   if (use_tc) {
-    const int32_t dk = (dpad + 63) / 64 * 64;
-    void* hi = sc.get<uint16_t>((size_t)s * dk);
-    void* lo = sc.get<uint16_t>((size_t)s * dk);
     int32_t* err = sc.get<int32_t>(1);
     CK(cudaMemsetAsync(err, 0, sizeof(int32_t), st));
-    CK(launch_tile_topk_tc(xo, norms, s, dpad, mode, cand, hi, lo, err, st));
+    const int32_t splits = tile_list_splits(s, s, mode == 0);
+    uint64_t* lists = splits > 1 ? sc.get<uint64_t>((size_t)splits * s * KP) : cand;
+    CK(launch_tile_lists_tc(hi, lo, norms, s, hi, lo, norms, s, dk, mode, nullptr, splits, lists, err, st));
+    if (splits > 1) launch_merge_lists(lists, s, splits, KP, cand, sc.get<float>(s), st);
     int32_t herr = 0;
     CK(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (herr) throw Failure(HENN_ERR_TIMEOUT, "tensor-core tile pipeline wait timed out (code " + std::to_string(herr) + ")");
     tile_u = tc_tile_unit_error(dk);
   } else {
-    launch_tile_topk_simt(xo, norms, s, xo, norms, s, dpad, mode, KP, 1, cand, st);
+    launch_tile_topk_simt(xo, norms, s, xo, norms, s, dpad, mode, KP, 1, cand, nullptr, nullptr, st);
     CKL("distance tiles");
     tile_u = (dpad + 8.0) * std::ldexp(1.0, -24);
   }
@@ -547,17 +604,24 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
   ix->tile_flops += pairs * 2.0 * ix->d;
   if (li == 0) ix->tile_engine = use_tc ? HENN_TILES_TCGEN05 : HENN_TILES_SIMT;
   tr.mark("tiles + top-k", li);
-  int32_t* unc = sc.get<int32_t>((size_t)s + 1);
-  CK(cudaMemsetAsync(unc, 0, sizeof(int32_t), st));
-  launch_rerank_fwd(ix->xw, Ly.ids, s, dpad, ix->metric, inv, cand, KP, M, norms, nmax, tile_u, Ly.fwd, Ly.fwd_d, unc,
-                    st);
+  FlaggedRows flagged;
+  flagged.count = sc.get<int32_t>(1);
+  flagged.rows = sc.get<int32_t>(s);
+  flagged.thr = sc.get<float>(s);
+  CK(cudaMemsetAsync(flagged.count, 0, sizeof(int32_t), st));
+  launch_rerank_fwd(ix->xw, Ly.ids, s, 0, dpad, ix->metric, inv, cand, KP, M, norms, nmax, tile_u, Ly.fwd, Ly.fwd_d,
+                    flagged, st);
   CKL("rerank");
   int32_t nunc = 0;
-  CK(cudaMemcpyAsync(&nunc, unc, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(&nunc, flagged.count, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   if (nunc > 0) {
-    launch_exact_rows(ix->xw, Ly.ids, s, dpad, ix->metric, inv, mode, unc + 1, nunc, M, Ly.fwd, Ly.fwd_d, st);
-    CKL("exact rows");
+    if (use_tc) {
+      settle_flagged(ix, Ly, s, flagged, nunc, 0, mode, Ly.ids, inv, hi, lo, norms, hi, lo, norms, dk, sc, st);
+    } else {
+      launch_exact_rows(ix->xw, Ly.ids, s, dpad, ix->metric, inv, mode, flagged.rows, nunc, M, Ly.fwd, Ly.fwd_d, st);
+      CKL("exact rows");
+    }
     ix->uncertified += nunc;
   }
   tr.mark("rerank/certify", li, nunc);
@@ -1019,8 +1083,48 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       for (int64_t j = 0; j < c; ++j) rows[j] = (int32_t)(s0 + j);
       int32_t* drows = sc.get<int32_t>(c);
       CK(cudaMemcpyAsync(drows, rows.data(), sizeof(int32_t) * c, cudaMemcpyHostToDevice, st));
-      launch_exact_rows(ix->xw, li >= 1 ? Ly.ids : nullptr, s1, dpad, ix->metric, nullptr, 0, drows, (int32_t)c, M,
-                        Ly.fwd, Ly.fwd_d, st);
+      const int32_t* lids = li >= 1 ? Ly.ids : nullptr;
+      const int32_t KP = M <= 16 ? 32 : 64;
+      if (tc_tiles_supported(dpad, KP)) {
+        // tiles of the new rows against the whole layer (row j takes the
+        // columns before position s0 + j), reranked and settled as a build's.
+        // The exact scan of every row that this replaces took 61.9 of the
+        // 72.9 ms that a 100,000 x 128 build and 20,000 insertions ran.
+        const int32_t dk = round_up(dpad, 64);
+        float* partial = sc.get<float>((size_t)mean_chunks(s1) * dpad);
+        float* mean = sc.get<float>(dpad);
+        launch_layer_mean(ix->xw, lids, s1, dpad, partial, mean, st);
+        uint16_t* hi = sc.get<uint16_t>((size_t)s1 * dk);
+        uint16_t* lo = sc.get<uint16_t>((size_t)s1 * dk);
+        float* norms = sc.get<float>(s1);
+        float* nmax = sc.get<float>(1);
+        launch_order_split(ix->xw, lids, s1, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, norms, nullptr, nmax, st);
+        const int32_t splits = tile_list_splits(c, s1, false);
+        uint64_t* lists = sc.get<uint64_t>((size_t)splits * c * KP);
+        uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)c * KP) : lists;
+        int32_t* err = sc.get<int32_t>(2);  // the tile launch's error flag, the flagged rows' number
+        CK(cudaMemsetAsync(err, 0, 2 * sizeof(int32_t), st));
+        CK(launch_tile_lists_tc(hi + (size_t)s0 * dk, lo + (size_t)s0 * dk, norms + s0, c, hi, lo, norms, s1, dk, 2,
+                                drows, splits, lists, err, st));
+        if (splits > 1) launch_merge_lists(lists, c, splits, KP, cand, sc.get<float>(c), st);
+        FlaggedRows flagged;
+        flagged.count = err + 1;
+        flagged.rows = sc.get<int32_t>(c);
+        flagged.thr = sc.get<float>(c);
+        launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, KP, M, norms + s0, nmax,
+                          tc_tile_unit_error(dk), Ly.fwd, Ly.fwd_d, flagged, st);
+        CKL("rerank");
+        int32_t host[2] = {0, 0};
+        CK(cudaMemcpyAsync(host, err, sizeof(host), cudaMemcpyDeviceToHost, st));
+        CK(cudaStreamSynchronize(st));
+        if (host[0])
+          throw Failure(HENN_ERR_TIMEOUT, "tensor-core tile pipeline wait timed out (code " + std::to_string(host[0]) + ")");
+        if (host[1] > 0)
+          settle_flagged(ix, Ly, s1, flagged, host[1], s0, 0, lids, nullptr, hi + (size_t)s0 * dk, lo + (size_t)s0 * dk,
+                         norms + s0, hi, lo, norms, dk, sc, st);
+      } else {
+        launch_exact_rows(ix->xw, lids, s1, dpad, ix->metric, nullptr, 0, drows, (int32_t)c, M, Ly.fwd, Ly.fwd_d, st);
+      }
       CKL("forward lists");
       // edge rule over the layer's updated forward lists
       int32_t* cnt = sc.get<int32_t>(s1);
@@ -1393,8 +1497,8 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
         const int32_t splits =
             (int32_t)std::max<int64_t>(1, std::min<int64_t>((2 * 152 + rb - 1) / rb, (s + 4095) / 4096));
         uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)splits * nq * 32) : pkeys;
-        launch_tile_topk_simt(qo, qn, nq, eo.xo, eo.norms, s, dpad, 2, 32, splits, cand, st);
-        if (splits > 1) launch_merge_splits(cand, nq, 32, splits, pkeys, st);
+        launch_tile_topk_simt(qo, qn, nq, eo.xo, eo.norms, s, dpad, 2, 32, splits, cand, nullptr, nullptr, st);
+        if (splits > 1) launch_merge_splits(cand, nq, 32, splits, pkeys, nullptr, st);
         a.pre_tile_u = (dpad + 8.0) * std::ldexp(1.0, -24);
         launches += splits > 1 ? 3 : 2;
       }
@@ -1610,6 +1714,123 @@ extern "C" henn_status henn_index_get_layer(const henn_index* idx, int32_t layer
 
 // ------------------------------------------------- standalone kernels
 
+namespace {
+
+// Pool width of the SIMT engine's candidates for k results.
+int32_t knn_pool(int32_t k) {
+  int32_t KP = 32;
+  while (KP < k + 16) KP <<= 1;
+  return KP;
+}
+
+// Exact k-NN by the SIMT FP32 tiles: a pool of at least k + 16 candidates,
+// reranked.  xp / qp: rows of dpad floats.
+void knn_simt(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t dpad, int32_t k, int32_t metric,
+              int64_t* out_ids, float* out_dists, Scratch& sc, cudaStream_t st) {
+  float* xn = sc.get<float>(n);
+  float* qn = sc.get<float>(nq);
+  launch_sq_norms(xp, n, dpad, xn, st);
+  launch_sq_norms(qp, nq, dpad, qn, st);
+  const int32_t KP = knn_pool(k);
+  const int64_t rb = (nq + 63) / 64;
+  const int32_t splits = (int32_t)std::max<int64_t>(1, std::min<int64_t>((2 * 152 + rb - 1) / rb, (n + 4095) / 4096));
+  uint64_t* cand = sc.get<uint64_t>((size_t)splits * nq * KP);
+  launch_tile_topk_simt(qp, qn, nq, xp, xn, n, dpad, 2, KP, splits, cand, nullptr, nullptr, st);
+  uint64_t* merged = cand;
+  if (splits > 1) {
+    merged = sc.get<uint64_t>((size_t)nq * KP);
+    launch_merge_splits(cand, nq, KP, splits, merged, nullptr, st);
+  }
+  launch_rerank_queries(qp, nq, xp, dpad, metric, merged, KP, k, out_ids, out_dists, nullptr, nullptr, st);
+}
+
+// From this many (query, point) pairs on, the tensor-core path.  It takes
+// about 170 us at the least (14 launches); the SIMT path as long for one
+// query against 2,000 x 32 points (159 us) and more beyond: 8 queries 278 us,
+// 1 against 20,000 x 128 511 us, 1,000 against 1,000,000 x 128 11.9 ms (1.8
+// ms on the tensor cores).
+constexpr int64_t kKnnTilesMin = 4096;
+// Queries that go through it together (its buffers are sized for them).
+constexpr int64_t kKnnBatch = 65536;
+
+// Exact k-NN on the tensor cores: split-BF16 tiles keep lists of each query's
+// nearest columns, the merged pool is reranked in FP32 and certified (every
+// column outside it is provably farther than the k-th), queries that fail
+// the certificate collect all columns that can matter in a second tile pass
+// over those queries alone, and those with too many (massive ties, values
+// that are no numbers) take the SIMT path.  Everything is enqueued without
+// a wait: the later passes read how many queries they have on the device.
+void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t dpad, int32_t k, int32_t metric,
+               int64_t* out_ids, float* out_dists, Scratch& sc, cudaStream_t st) {
+  const int32_t dk = round_up(dpad, 64);
+  float* partial = sc.get<float>((size_t)mean_chunks(n) * dpad);
+  float* mean = sc.get<float>(dpad);
+  launch_layer_mean(xp, nullptr, n, dpad, partial, mean, st);
+  void* hi = sc.get<uint16_t>((size_t)n * dk);
+  void* lo = sc.get<uint16_t>((size_t)n * dk);
+  float* xn = sc.get<float>(n);
+  float* xraw = sc.get<float>(n);
+  float* nmax = sc.get<float>(2);  // of the points; of the queries (not used)
+  launch_order_split(xp, nullptr, n, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, xn, xraw, nmax, st);
+  const int64_t nb = std::min(nq, kKnnBatch);
+  uint16_t* qhi = sc.get<uint16_t>((size_t)nb * dk);
+  uint16_t* qlo = sc.get<uint16_t>((size_t)nb * dk);
+  float* qn = sc.get<float>(nb);
+  float* qraw = sc.get<float>(nb);
+  // the pool: 32, 64 or 128 candidates, at least 16 more than k; wider than a
+  // list, it takes lists enough that one seldom holds more than 8 of the k
+  const int32_t KP = k <= 16 ? 32 : (k <= 48 ? 64 : 128);
+  const int64_t tiles = (n + kTileCols - 1) / kTileCols;
+  int32_t splits = tile_list_splits(nb, n, false);
+  if (k > 16) splits = (int32_t)std::min<int64_t>(tiles, std::max(splits, (k + 7) / 8));
+  uint64_t* lists = sc.get<uint64_t>((size_t)splits * nb * 32);
+  uint64_t* cand = sc.get<uint64_t>((size_t)nb * KP);
+  float* thr = sc.get<float>(nb);
+  void* fhi = sc.get<uint16_t>((size_t)nb * dk);
+  void* flo = sc.get<uint16_t>((size_t)nb * dk);
+  float* fnorms = sc.get<float>(nb);
+  int32_t* lim = sc.get<int32_t>(nb);
+  int32_t* self = sc.get<int32_t>(nb);
+  FlaggedRows flagged;
+  flagged.rows = sc.get<int32_t>(nb);
+  flagged.thr = sc.get<float>(nb);
+  const unsigned grid = tile_collect_grid(nb);
+  uint32_t* cols = sc.get<uint32_t>((size_t)grid * kTileRows * kCollectCap);
+  int32_t* ncols = sc.get<int32_t>((size_t)grid * kTileRows);
+  int32_t* over = sc.get<int32_t>((size_t)nb + 3);  // number, rows, flagged rows' number, tile error flag
+  flagged.count = over + nb + 1;
+  int32_t* err = over + nb + 2;
+  const int32_t KS = knn_pool(k);
+  // the SIMT path's lists: split over the points as far as 64 MB allow
+  const int32_t ssplits = (int32_t)std::max<int64_t>(
+      1, std::min<int64_t>({(int64_t)64, (n + 4095) / 4096, (int64_t)(64 << 20) / (nb * KS * 8)}));
+  uint64_t* scand = sc.get<uint64_t>((size_t)ssplits * nb * KS);
+  uint64_t* smerged = ssplits > 1 ? sc.get<uint64_t>((size_t)nb * KS) : scand;
+  const double tile_u = tc_tile_unit_error(dk);
+  for (int64_t q0 = 0; q0 < nq; q0 += nb) {
+    const int64_t c = std::min(nb, nq - q0);
+    const float* q = qp + q0 * dpad;
+    int64_t* oi = out_ids + q0 * k;
+    float* od = out_dists + q0 * k;
+    CK(cudaMemsetAsync(over, 0, sizeof(int32_t), st));
+    CK(cudaMemsetAsync(flagged.count, 0, 2 * sizeof(int32_t), st));
+    launch_order_split(q, nullptr, c, dpad, 0, 0, true, mean, dk, qhi, qlo, nullptr, qn, qraw, nmax + 1, st);
+    CK(launch_tile_lists_tc(qhi, qlo, qn, c, hi, lo, xn, n, dk, 2, nullptr, splits, lists, err, st));
+    launch_merge_lists(lists, c, splits, KP, cand, thr, st);
+    launch_rerank_knn(q, c, xp, n, dpad, metric, cand, thr, KP, k, qn, nmax, tile_u, err, oi, od, flagged, st);
+    launch_gather_flagged(flagged, c, 0, false, false, n, qhi, qlo, qn, dk, fhi, flo, fnorms, lim, self, st);
+    CK(launch_tile_collect_tc(fhi, flo, fnorms, c, hi, lo, xn, n, dk, lim, self, flagged.thr, flagged.count, grid, cols,
+                              ncols, kCollectCap, err, st));
+    launch_rerank_collected_knn(q, xp, flagged, c, dpad, metric, n, grid, cols, ncols, kCollectCap, k, oi, od, over,
+                                err, st);
+    launch_tile_topk_simt(q, qraw, c, xp, xraw, n, dpad, 2, KS, ssplits, scand, over + 1, over, st);
+    if (ssplits > 1) launch_merge_splits(scand, c, KS, ssplits, smerged, over, st);
+    launch_rerank_queries(q, c, xp, dpad, metric, smerged, KS, k, oi, od, over + 1, over, st);
+  }
+}
+
+}  // namespace
+
 extern "C" henn_status henn_exact_knn(const float* X, int64_t n, int32_t d, const float* Q, int64_t nq, int32_t k,
                                       int32_t metric, int64_t* out_ids, float* out_dists, void* stream) {
   g_error.clear();
@@ -1623,42 +1844,25 @@ extern "C" henn_status henn_exact_knn(const float* X, int64_t n, int32_t d, cons
     cudaStream_t st = (cudaStream_t)stream;
     const int32_t dpad = round_up(d, 32);
     Scratch sc(st);
-    float* xp = sc.get<float>((size_t)n * dpad);
-    float* qp = sc.get<float>((size_t)nq * dpad);
-    CK(cudaMemsetAsync(xp, 0, sizeof(float) * n * dpad, st));
-    CK(cudaMemsetAsync(qp, 0, sizeof(float) * nq * dpad, st));
-    CK(cudaMemcpy2DAsync(xp, sizeof(float) * dpad, X, sizeof(float) * d, sizeof(float) * d, n, cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpy2DAsync(qp, sizeof(float) * dpad, Q, sizeof(float) * d, sizeof(float) * d, nq, cudaMemcpyDeviceToDevice, st));
-    float* xn = sc.get<float>(n);
-    float* qn = sc.get<float>(nq);
-    if (metric == HENN_ANGULAR) {
-      launch_inv_norms(xp, n, dpad, xn, st);
-      launch_normalise(xp, xn, n, dpad, xp, st);
-      launch_inv_norms(qp, nq, dpad, qn, st);
-      launch_normalise(qp, qn, nq, dpad, qp, st);
-    }
-    // squared norms of the (possibly normalised) rows
-    float* mean0 = sc.get<float>(dpad);
-    CK(cudaMemsetAsync(mean0, 0, sizeof(float) * dpad, st));
-    int32_t* invx = sc.get<int32_t>(n);
-    int32_t* invq = sc.get<int32_t>(nq);
-    float* xo = sc.get<float>((size_t)n * dpad);
-    float* qo = sc.get<float>((size_t)nq * dpad);
-    launch_order_gather(xp, nullptr, n, dpad, 0, 0, HENN_GRAPH_KNN, mean0, invx, xo, xn, st);
-    launch_order_gather(qp, nullptr, nq, dpad, 0, 0, HENN_GRAPH_KNN, mean0, invq, qo, qn, st);
-    int32_t KP = 32;
-    while (KP < k + 16) KP <<= 1;
-    int sms = 152;
-    int64_t rb = (nq + 63) / 64;
-    int32_t splits = (int32_t)std::max<int64_t>(1, std::min<int64_t>((2 * sms + rb - 1) / rb, (n + 4095) / 4096));
-    uint64_t* cand = sc.get<uint64_t>((size_t)splits * nq * KP);
-    launch_tile_topk_simt(qo, qn, nq, xo, xn, n, dpad, 2, KP, splits, cand, st);
-    uint64_t* merged = cand;
-    if (splits > 1) {
-      merged = sc.get<uint64_t>((size_t)nq * KP);
-      launch_merge_splits(cand, nq, KP, splits, merged, st);
-    }
-    launch_rerank_queries(qo, nq, xo, dpad, metric, merged, KP, k, out_ids, out_dists, st);
+    // rows of dpad floats (unit length for angular); used as they are where
+    // they already are that
+    auto rows_of = [&](const float* v, int64_t rows) -> const float* {
+      if (metric == HENN_L2 && d == dpad && (reinterpret_cast<uintptr_t>(v) & 15) == 0) return v;
+      float* p = sc.get<float>((size_t)rows * dpad);
+      launch_pad_copy(v, rows, d, dpad, p, st);
+      if (metric == HENN_ANGULAR) {
+        float* inv = sc.get<float>(rows);
+        launch_inv_norms(p, rows, dpad, inv, st);
+        launch_normalise(p, inv, rows, dpad, p, st);
+      }
+      return p;
+    };
+    const float* xp = rows_of(X, n);
+    const float* qp = rows_of(Q, nq);
+    if (nq * n >= kKnnTilesMin)
+      knn_tiles(xp, n, qp, nq, dpad, k, metric, out_ids, out_dists, sc, st);
+    else
+      knn_simt(xp, n, qp, nq, dpad, k, metric, out_ids, out_dists, sc, st);
     CKL("exact knn");
     return HENN_OK;
   } catch (const Failure& f) {

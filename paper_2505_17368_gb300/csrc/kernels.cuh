@@ -60,6 +60,16 @@ void launch_layer_mean(const float* xw, const int32_t* ids, int64_t s, int32_t d
 void launch_order_gather(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, uint64_t seed,
                          int32_t layer, int32_t graph, const float* mean, int32_t* inv, float* xo,
                          float* norms, cudaStream_t st);
+// The operand of the tensor-core tiles in one pass: row j of the layer minus
+// its mean at rank perm(j) (identity: j), as BF16 planes hi = bf16(x), lo =
+// bf16(x - hi), dk wide, with its squared norm; inv (nullable) as above;
+// *norm_max the largest norm (NaN if one is)
+// (raw_norms, nullable: the rows' squared norms without the mean taken off)
+void launch_order_split(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, uint64_t seed, int32_t layer,
+                        bool identity, const float* mean, int32_t dk, void* hi, void* lo, int32_t* inv, float* norms,
+                        float* raw_norms, float* norm_max, cudaStream_t st);
+// squared norms of rows of dpad floats
+void launch_sq_norms(const float* x, int64_t s, int32_t dpad, float* norms, cudaStream_t st);
 void launch_gather_rows32(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, float* out,
                           cudaStream_t st);
 void launch_quantize(const float* x, int64_t n, int32_t d, int32_t dpad_in, int32_t dpad_out,
@@ -69,16 +79,50 @@ void launch_quantize(const float* x, int64_t n, int32_t d, int32_t dpad_in, int3
 //   mode 0: causal (column c valid iff c < row), A == B
 //   mode 1: all other rows (c != row), A == B
 //   mode 2: rows of A against all rows of B
+// rowsel / count (nullable): only the rows rowsel[0 .. *count - 1] of A; list
+// i is then row rowsel[i]'s
 void launch_tile_topk_simt(const float* A, const float* An, int64_t na, const float* B, const float* Bn,
                            int64_t nb, int32_t dpad, int32_t mode, int32_t KP, int32_t splits,
-                           uint64_t* out, cudaStream_t st);
+                           uint64_t* out, const int32_t* rowsel, const int32_t* count, cudaStream_t st);
 void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t KP, int32_t splits, uint64_t* out,
-                         cudaStream_t st);
-// knn_tc.cu: the same tiles on tcgen05 tensor cores (split BF16, KP = 32,
-// dpad <= 128); scratch_hi / scratch_lo hold s * roundup(dpad, 64) BF16
+                         const int32_t* count, cudaStream_t st);
+// Sorted lists of 32 keys per row and split (splits x rows x 32) -> the KP
+// (32, 64 or 128) smallest of each row, and a bound on what they leave out:
+// every column of the row that is not among them has a tile distance of at
+// least thr[row] (+inf: every column that the lists were offered is there).
+void launch_merge_lists(const uint64_t* in, int64_t rows, int32_t splits, int32_t KP, uint64_t* out, float* thr,
+                        cudaStream_t st);
+// knn_tc.cu: the same tiles on tcgen05 tensor cores (split BF16, lists of
+// KP = 32, dpad <= 1024) from BF16 planes of rows and columns, dk =
+// roundup(dpad, 64) wide
 bool tc_tiles_supported(int32_t dpad, int32_t KP);
-cudaError_t launch_tile_topk_tc(const float* xo, const float* norms, int64_t s, int32_t dpad, int32_t mode,
-                                uint64_t* out, void* scratch_hi, void* scratch_lo, int32_t* err, cudaStream_t st);
+// CTAs per row block, each with its own lists, for na rows against nb columns
+int32_t tile_list_splits(int64_t na, int64_t nb, bool causal);
+// modes 0 - 2; out: splits x na x 32 keys, each list sorted; lim (nullable):
+// row r takes columns 0 .. lim[r] - 1 only
+cudaError_t launch_tile_lists_tc(const void* a_hi, const void* a_lo, const float* a_norms, int64_t na,
+                                 const void* b_hi, const void* b_lo, const float* b_norms, int64_t nb, int32_t dk,
+                                 int32_t mode, const int32_t* lim, int32_t splits, uint64_t* out, int32_t* err,
+                                 cudaStream_t st);
+// Every column of a row whose tile distance is at or under the row's
+// threshold.  The number of rows is *count (device, at most max_rows); the
+// grid's CTAs are shared out over the 128-row blocks there are
+// (collect_splits); CTA b of a block writes row r's columns, at most cap of
+// them, at cols + (b * 128 + r) * cap and their number (over cap: some were
+// dropped) to ncols[b * 128 + r].
+constexpr int kTileRows = 128, kTileCols = 256;
+__host__ __device__ inline int32_t collect_splits(unsigned grid, int64_t rows, int64_t nb) {
+  const int64_t blocks = (rows + kTileRows - 1) / kTileRows;
+  const int64_t most = (nb + 2 * kTileCols - 1) / (2 * kTileCols);  // at least two tiles each
+  const int64_t k = (int64_t)grid / blocks;
+  return (int32_t)(k < 1 ? 1 : (k > most ? most : k));
+}
+unsigned tile_collect_grid(int64_t max_rows);
+cudaError_t launch_tile_collect_tc(const void* a_hi, const void* a_lo, const float* a_norms, int64_t max_rows,
+                                   const void* b_hi, const void* b_lo, const float* b_norms, int64_t nb, int32_t dk,
+                                   const int32_t* lim, const int32_t* self, const float* thr, const int32_t* count,
+                                   unsigned grid, uint32_t* cols, int32_t* ncols, int32_t cap, int32_t* err,
+                                   cudaStream_t st);
 // FP32 rows (dpad wide) -> BF16 planes hi = bf16(x), lo = bf16(x - hi), dk wide (zero padded)
 void launch_split_bf16(const float* x, int64_t s, int32_t dpad, int32_t dk, void* hi, void* lo, cudaStream_t st);
 // mode 2 on tensor cores from pre-split planes: na rows (queries) against nb
@@ -100,11 +144,52 @@ cudaError_t launch_tile_cross_tc(const void* a_hi, const void* a_lo, const float
 // launch_tile_cross_tc -- hi and lo for tiles of 256 columns, then for 128 --
 // written to maps (4 x 128 bytes); false if not encodable.
 bool make_column_maps(const void* b_hi, const void* b_lo, int64_t nb, int32_t dk, void* maps);
-// exact FP32 rerank of layer candidates -> forward lists (layer-local ids)
-void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, int32_t metric,
+// Rows that a candidate list could not settle: their number, the rows, and
+// for each the tile distance that every column of its answer lies under.
+struct FlaggedRows {
+  int32_t* count;
+  int32_t* rows;
+  float* thr;
+};
+// exact FP32 rerank of layer candidates -> forward lists (layer-local ids).
+// Row r is layer position inv[r], or row0 + r with inv == nullptr (columns
+// are then positions too).
+void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
                        const int32_t* inv, const uint64_t* cand, int32_t KP, int32_t M, const float* norms,
-                       const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d, int32_t* uncertified,
+                       const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d, const FlaggedRows& flagged,
                        cudaStream_t st);
+// The flagged rows' BF16 planes and norms, compact; lim[i]: causal the row's
+// own rank row0 + r, else nb; self[i]: r with skip_self, else -1.
+void launch_gather_flagged(const FlaggedRows& f, int64_t max_rows, int64_t row0, bool causal, bool skip_self,
+                           int64_t nb, const void* hi, const void* lo, const float* norms, int32_t dk, void* hi_out,
+                           void* lo_out, float* norms_out, int32_t* lim, int32_t* self, cudaStream_t st);
+// exact FP32 rerank of collected columns -> forward lists of the flagged
+// rows; rows with more than cap columns in one CTA (or any, with *err set)
+// go to over (over[0]: their number, then the rows, plus row0)
+void launch_rerank_collected_fwd(const float* xw, const int32_t* ids, const FlaggedRows& f, int64_t max_rows,
+                                 int64_t row0, int32_t dpad, int32_t metric, const int32_t* inv, int64_t nb,
+                                 unsigned grid, const uint32_t* cols, const int32_t* ncols, int32_t cap, int32_t M,
+                                 int32_t* fwd, float* fwd_d, int32_t* over, const int32_t* err, cudaStream_t st);
+// the same for queries (rows of Q): k results (int64 ids, reported distances)
+void launch_rerank_collected_knn(const float* Q, const float* X, const FlaggedRows& f, int64_t max_rows, int32_t dpad,
+                                 int32_t metric, int64_t nb, unsigned grid, const uint32_t* cols,
+                                 const int32_t* ncols, int32_t cap, int32_t k, int64_t* out_ids, float* out_d,
+                                 int32_t* over, const int32_t* err, cudaStream_t st);
+// queries' merged tile lists -> k results, and the queries whose list does
+// not prove them (thr: launch_merge_lists; err: the tile launch's flag)
+void launch_rerank_knn(const float* Q, int64_t nq, const float* X, int64_t n, int32_t dpad, int32_t metric,
+                       const uint64_t* cand, const float* thr, int32_t KP, int32_t k, const float* qnorms,
+                       const float* norm_max, double tile_u, const int32_t* err, int64_t* out_ids, float* out_d,
+                       const FlaggedRows& flagged, cudaStream_t st);
+// exact recompute of the forward list of uncertified rows
+void launch_exact_rows(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, int32_t metric,
+                       const int32_t* inv, int32_t mode, const int32_t* rows, int32_t nrows, int32_t M,
+                       int32_t* fwd, float* fwd_d, cudaStream_t st);
+// exact rerank of query candidates -> k results (rowsel / count as for the
+// SIMT tiles: list i is query rowsel[i]'s)
+void launch_rerank_queries(const float* Q, int64_t nq, const float* X, int32_t dpad, int32_t metric,
+                           const uint64_t* cand, int32_t KP, int32_t k, int64_t* out_ids, float* out_d,
+                           const int32_t* rowsel, const int32_t* count, cudaStream_t st);
 void launch_max_nonneg(const float* v, int64_t n, float* out, cudaStream_t st);
 // exact recompute of the forward list of uncertified rows
 void launch_exact_rows(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, int32_t metric,

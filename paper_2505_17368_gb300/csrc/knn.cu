@@ -21,7 +21,9 @@ template <int KP>
 __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict__ A, const float* __restrict__ An,
                                                         int64_t na, const float* __restrict__ B,
                                                         const float* __restrict__ Bn, int64_t nb, int32_t dpad,
-                                                        int32_t mode, int32_t splits, uint64_t* __restrict__ out) {
+                                                        int32_t mode, int32_t splits, uint64_t* __restrict__ out,
+                                                        const int32_t* __restrict__ rowsel,
+                                                        const int32_t* __restrict__ count) {
   __shared__ __align__(16) float As[kBK][kBM + 4];
   __shared__ __align__(16) float Bs[kBK][kBN + 4];
   __shared__ float S[kBM][kBN + 1];
@@ -29,6 +31,11 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   const int warp = tid >> 5;
+  const int64_t stride = na;  // rows between two splits' lists
+  if (count) {
+    na = min(na, (int64_t)*count);
+    if ((int64_t)blockIdx.x * kBM >= na) return;
+  }
   const int64_t nblocks = (na + kBM - 1) / kBM;
   // causal rows: heaviest row blocks first
   const int64_t rb = (mode == 0) ? (nblocks - 1 - blockIdx.x) : blockIdx.x;
@@ -61,7 +68,7 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
         int row = idx >> 3, kq = (idx & 7) * 4;
         int64_t gr = r0 + row;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (gr < na) v = *reinterpret_cast<const float4*>(A + gr * dpad + k0 + kq);
+        if (gr < na) v = *reinterpret_cast<const float4*>(A + (rowsel ? (int64_t)rowsel[gr] : gr) * dpad + k0 + kq);
         As[kq + 0][row] = v.x;
         As[kq + 1][row] = v.y;
         As[kq + 2][row] = v.z;
@@ -91,7 +98,7 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       int64_t gr = r0 + ty * 4 + i;
-      float an = gr < na ? An[gr] : 0.f;
+      float an = gr < na ? An[rowsel ? (int64_t)rowsel[gr] : gr] : 0.f;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         int64_t gc = c0 + tx * 4 + j;
@@ -138,7 +145,7 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
   for (int i = 0; i < 8; ++i) {
     int64_t gr = r0 + warp * 8 + i;
     if (gr < na) {
-      uint64_t* dst = out + ((int64_t)split * na + gr) * KP;
+      uint64_t* dst = out + ((int64_t)split * stride + gr) * KP;
 #pragma unroll
       for (int r = 0; r < KP / 32; ++r) dst[r * 32 + (tid & 31)] = lists[i].v[r];
     }
@@ -146,21 +153,24 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
 }
 
 void launch_tile_topk_simt(const float* A, const float* An, int64_t na, const float* B, const float* Bn, int64_t nb,
-                           int32_t dpad, int32_t mode, int32_t KP, int32_t splits, uint64_t* out, cudaStream_t st) {
+                           int32_t dpad, int32_t mode, int32_t KP, int32_t splits, uint64_t* out,
+                           const int32_t* rowsel, const int32_t* count, cudaStream_t st) {
   dim3 grid((unsigned)((na + kBM - 1) / kBM), (unsigned)splits);
   switch (KP) {
-    case 32: k_tile_topk_simt<32><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out); break;
-    case 64: k_tile_topk_simt<64><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out); break;
-    case 128: k_tile_topk_simt<128><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out); break;
-    default: k_tile_topk_simt<256><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out); break;
+    case 32: k_tile_topk_simt<32><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
+    case 64: k_tile_topk_simt<64><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
+    case 128: k_tile_topk_simt<128><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
+    default: k_tile_topk_simt<256><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
   }
 }
 
 // merge per-split lists of one row into one list of KP
 template <int KP>
-__global__ void k_merge_splits(const uint64_t* __restrict__ in, int64_t rows, int32_t splits, uint64_t* __restrict__ out) {
+__global__ void k_merge_splits(const uint64_t* __restrict__ in, int64_t rows, int32_t splits, uint64_t* __restrict__ out,
+                               const int32_t* __restrict__ count) {
   const int lane = threadIdx.x & 31;
-  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < rows;
+  const int64_t nr = count ? min(rows, (int64_t)*count) : rows;
+  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < nr;
        r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
     WarpList<KP> list;
     list.clear();
@@ -183,14 +193,15 @@ __global__ void k_merge_splits(const uint64_t* __restrict__ in, int64_t rows, in
   }
 }
 
-void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t KP, int32_t splits, uint64_t* out, cudaStream_t st) {
+void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t KP, int32_t splits, uint64_t* out,
+                         const int32_t* count, cudaStream_t st) {
   int grid = (int)((rows + 7) / 8);
   if (grid > 152 * 16) grid = 152 * 16;
   switch (KP) {
-    case 32: k_merge_splits<32><<<grid, 256, 0, st>>>(in, rows, splits, out); break;
-    case 64: k_merge_splits<64><<<grid, 256, 0, st>>>(in, rows, splits, out); break;
-    case 128: k_merge_splits<128><<<grid, 256, 0, st>>>(in, rows, splits, out); break;
-    default: k_merge_splits<256><<<grid, 256, 0, st>>>(in, rows, splits, out); break;
+    case 32: k_merge_splits<32><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
+    case 64: k_merge_splits<64><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
+    case 128: k_merge_splits<128><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
+    default: k_merge_splits<256><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
   }
 }
 
@@ -211,97 +222,458 @@ __device__ __forceinline__ float warp_exact_dist(const float* __restrict__ a, co
   return metric == HENN_ANGULAR ? 0.5f * acc : acc;
 }
 
-// Forward lists from the KP tile candidates of each row (rank space).
-// Certification: the tile distance of any non-candidate column is >= the
-// row's KP-th tile distance thr; its true distance is >= thr - beta where
-// beta bounds the tile error for this row.  If thr - beta exceeds the M-th
-// exact distance, no column outside the pool can enter the forward list;
-// otherwise the row is flagged for an exact recompute.
-template <int KP>
-__global__ void k_rerank_fwd(const float* __restrict__ xw, const int32_t* __restrict__ ids, int64_t s, int32_t dpad,
-                             int32_t metric, const int32_t* __restrict__ inv, const uint64_t* __restrict__ cand,
-                             int32_t M, const float* __restrict__ norms, const float* __restrict__ norm_max, double tile_u,
-                             int32_t* __restrict__ fwd, float* __restrict__ fwd_d, int32_t* __restrict__ uncertified) {
+// The same distance from row `a` to 32 rows at once: lane c gives row c's
+// index (count of them, lanes 0 .. count - 1) and gets its distance.  Eight
+// rows' loads are in flight together, and the 32 sums over the lanes are
+// formed by exchanging halves (31 shuffles for 32 rows instead of 160): lane
+// l ends with row l's sum, added up in the tree of the butterfly above
+// (offsets 16, 8, 4, 2, 1; addition commutes), so every distance has the bits
+// that warp_exact_dist gives it.  The rows come from L2 or HBM at random; one
+// row at a time left one load in flight per lane and a butterfly per row (the
+// rerank of 10,000 x 32 points' 32 candidates: 104 us, now 64 us).
+__device__ __forceinline__ float warp_exact_dist32(const float* __restrict__ a, const float* __restrict__ X,
+                                                   int64_t row, int count, int32_t dpad, int32_t metric) {
   const int lane = threadIdx.x & 31;
-  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < s;
-       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t j = inv[r];
-    const int64_t gj = ids ? ids[j] : j;
-    const float* xj = xw + gj * dpad;
-    WarpList<KP> list;
-    list.clear();
-    const uint64_t* row = cand + r * KP;
-    uint64_t thr_key = kEmpty;
-    int count = 0;
-    for (int c = 0; c < KP; ++c) {
-      uint64_t key = row[c];  // warp-uniform broadcast load
-      if (key == kEmpty) break;
-      ++count;
-      thr_key = key;
-      int64_t qj = inv[key_index(key)];
-      int64_t gq = ids ? ids[qj] : qj;
-      float dv = warp_exact_dist(xj, xw + gq * dpad, dpad, metric);
-      list.insert(pack(dv, (uint32_t)qj));
-    }
-    // certification (every lane evaluates it; lane 0 records)
-    uint64_t mkey = shfl64(list.v[(M - 1) >> 5], (M - 1) & 31);
-    if (count == KP && uncertified) {
-      double thr = (double)key_dist(thr_key);
-      double dm = (mkey == kEmpty) ? 1e300 : (double)key_dist(mkey);
-      // exact distances here are of raw vectors; tile distances of centred
-      // ones: identical in exact arithmetic.  Angular: tile values are 2x.
-      if (metric == HENN_ANGULAR) dm *= 2.0;
-      // relative error bound of the exact FP32 distances (dpad / 32 FMA
-      // steps per lane, five butterfly additions), doubled
-      const double slack = (dpad / 32 + 8) * 0x1p-23;
-      // Only columns whose true distance can reach dm matter, and those lie
-      // within sqrt(dm) of this row, so their centred norm is at most
-      // (|x_r| + sqrt(dm))^2 (widened for the centring rounding); the tile
-      // error bound needs the column norm only up to that cap.
-      const double nr = (double)norms[r];
-      const double rad = sqrt(nr) * (1.0 + 1e-3) + sqrt(dm * (1.0 + 2.0 * slack)) * (1.0 + 1e-3);
-      const double nc = fmin((double)*norm_max, rad * rad);
-      const double beta = tile_u * 4.0 * (nr + nc) + 1e-30;
-      if (!(thr - beta > dm * (1.0 + slack))) {
-        if (lane == 0) {
-          int at = atomicAdd(uncertified, 1);
-          uncertified[1 + at] = (int32_t)r;
+  float acc[32];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) acc[c] = 0.f;
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    if (8 * g < count) {  // warp-uniform
+      const float* p[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        // past the last row: the last one again (its sum is not used)
+        const int64_t r = __shfl_sync(0xffffffffu, row, min(8 * g + i, count - 1));
+        p[i] = X + r * dpad + lane;
+      }
+#pragma unroll 2
+      for (int k = 0; k < dpad; k += 32) {
+        const float x = a[k + lane];
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = __ldg(p[i] + k);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float t = x - v[i];
+          acc[8 * g + i] = fmaf(t, t, acc[8 * g + i]);
         }
       }
     }
-    // output first M of the list, layer-local ids
+  }
 #pragma unroll
-    for (int q = 0; q < KP / 32; ++q) {
-      int g = q * 32 + lane;
-      if (g < M) {
-        uint64_t key = list.v[q];
-        fwd[j * M + g] = key == kEmpty ? -1 : (int32_t)key_index(key);
-        fwd_d[j * M + g] = key == kEmpty ? __int_as_float(0x7f800000) : key_dist(key);
-      }
+  for (int o = 16; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float keep = up ? acc[i + o] : acc[i];
+      const float send = up ? acc[i] : acc[i + o];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return metric == HENN_ANGULAR ? 0.5f * acc[0] : acc[0];
+}
+
+// ascending sort of a bitonic sequence, one key per lane
+__device__ __forceinline__ uint64_t warp_bitonic_clean(uint64_t v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t x = shfl_xor64(v, o);
+    v = (lane & o) == 0 ? (x < v ? x : v) : (x > v ? x : v);
+  }
+  return v;
+}
+
+// The 32 R smallest of a sorted list (element 32 r + lane in v[r]) and 32
+// sorted keys: the keys' smaller half against the list's last 32, then down
+// through the list, 32 and 32 merged into 64 at a time.
+template <int R>
+__device__ __forceinline__ void merge_sorted32(uint64_t (&v)[R], uint64_t keys) {
+  if (!__any_sync(0xffffffffu, keys < shfl64(v[R - 1], 31))) return;
+  uint64_t b = shfl64(keys, 31 - (threadIdx.x & 31));
+  b = warp_bitonic_clean(b < v[R - 1] ? b : v[R - 1]);
+#pragma unroll
+  for (int r = R - 2; r >= 0; --r) {
+    const uint64_t x = shfl64(b, 31 - (threadIdx.x & 31));
+    const uint64_t lo = x < v[r] ? x : v[r], hi = x < v[r] ? v[r] : x;
+    v[r + 1] = warp_bitonic_clean(hi);
+    b = warp_bitonic_clean(lo);
+  }
+  v[0] = b;
+}
+
+template <int KP>
+__global__ void __launch_bounds__(256) k_merge_lists(const uint64_t* __restrict__ in, int64_t rows, int32_t splits,
+                                                     uint64_t* __restrict__ out, float* __restrict__ thr) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < rows;
+       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    uint64_t v[KP / 32];
+#pragma unroll
+    for (int i = 0; i < KP / 32; ++i) v[i] = kEmpty;
+    uint64_t bound = kEmpty;  // smallest last key of a full list
+    for (int s = 0; s < splits; ++s) {
+      const uint64_t b = __ldg(in + ((int64_t)s * rows + r) * 32 + lane);
+      const uint64_t last = shfl64(b, 31);
+      bound = last < bound ? last : bound;
+      merge_sorted32(v, b);
+    }
+    const uint64_t last = shfl64(v[KP / 32 - 1], 31);
+    bound = last < bound ? last : bound;
+#pragma unroll
+    for (int i = 0; i < KP / 32; ++i) out[r * KP + 32 * i + lane] = v[i];
+    if (lane == 0) thr[r] = bound == kEmpty ? __int_as_float(0x7f800000) : key_dist(bound);
+  }
+}
+
+void launch_merge_lists(const uint64_t* in, int64_t rows, int32_t splits, int32_t KP, uint64_t* out, float* thr,
+                        cudaStream_t st) {
+  int grid = (int)((rows + 7) / 8);
+  if (grid > 152 * 16) grid = 152 * 16;
+  if (KP == 32)
+    k_merge_lists<32><<<grid, 256, 0, st>>>(in, rows, splits, out, thr);
+  else if (KP == 64)
+    k_merge_lists<64><<<grid, 256, 0, st>>>(in, rows, splits, out, thr);
+  else
+    k_merge_lists<128><<<grid, 256, 0, st>>>(in, rows, splits, out, thr);
+}
+
+// The certificate of a candidate pool.  The tile distance of any column
+// outside the pool is >= thr, so its true distance is >= thr - beta, beta
+// bounding the tile error for this row; if that exceeds the wanted list's
+// last exact distance dm, no outside column belongs to the list.  Else
+// *collect is the tile distance at or under which every column of the list
+// lies: their true distances are at most dm (the pool holds that many), so
+// their tile distances at most dm + beta.
+__device__ __forceinline__ bool pool_certified(double thr, double dm, float norm_row, float norm_max, double tile_u,
+                                               int32_t dpad, float* collect) {
+  // relative error bound of the exact FP32 distances (dpad / 32 FMA
+  // steps per lane, five butterfly additions), doubled
+  const double slack = (dpad / 32 + 8) * 0x1p-23;
+  // Only columns whose true distance can reach dm matter, and those lie
+  // within sqrt(dm) of this row, so their centred norm is at most
+  // (|x_r| + sqrt(dm))^2 (widened for the centring rounding); the tile
+  // error bound needs the column norm only up to that cap.
+  const double nr = (double)norm_row;
+  const double rad = sqrt(nr) * (1.0 + 1e-3) + sqrt(dm * (1.0 + 2.0 * slack)) * (1.0 + 1e-3);
+  // a NaN among the columns' norms stays one (fmin would drop it)
+  const double nc = norm_max != norm_max ? (double)norm_max : fmin((double)norm_max, rad * rad);
+  const double beta = tile_u * 4.0 * (nr + nc) + 1e-30;
+  *collect = __double2float_ru(dm * (1.0 + slack) + beta);
+  return thr - beta > dm * (1.0 + slack);
+}
+
+__device__ __forceinline__ void flag_row(const FlaggedRows& f, int32_t row, float thr) {
+  if ((threadIdx.x & 31) == 0) {
+    const int at = atomicAdd(f.count, 1);
+    f.rows[at] = row;
+    // not a number (a distance or a norm that is none): every column
+    f.thr[at] = thr != thr ? __int_as_float(0x7f800000) : thr;
+  }
+}
+
+// key g of a sorted list
+template <int R>
+__device__ __forceinline__ uint64_t list_key(const uint64_t (&v)[R], int g) {
+  uint64_t x = v[0];
+#pragma unroll
+  for (int r = 1; r < R; ++r)
+    if (r == g >> 5) x = v[r];
+  return shfl64(x, g & 31);
+}
+
+template <int R>
+__device__ __forceinline__ void write_fwd(const uint64_t (&v)[R], int64_t j, int32_t M, int32_t* __restrict__ fwd,
+                                          float* __restrict__ fwd_d) {
+#pragma unroll
+  for (int q = 0; q < R; ++q) {
+    const int g = q * 32 + (threadIdx.x & 31);
+    if (g < M) {
+      fwd[j * M + g] = v[q] == kEmpty ? -1 : (int32_t)key_index(v[q]);
+      fwd_d[j * M + g] = v[q] == kEmpty ? __int_as_float(0x7f800000) : key_dist(v[q]);
     }
   }
 }
 
-void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, int32_t metric, const int32_t* inv,
-                       const uint64_t* cand, int32_t KP, int32_t M, const float* norms, const float* norm_max, double tile_u,
-                       int32_t* fwd, float* fwd_d, int32_t* uncertified, cudaStream_t st) {
-  int grid = (int)((s + 7) / 8);
+template <int R>
+__device__ __forceinline__ void write_knn(const uint64_t (&v)[R], int64_t q, int32_t k, int32_t metric,
+                                          int64_t* __restrict__ out_ids, float* __restrict__ out_d) {
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int g = r * 32 + (threadIdx.x & 31);
+    if (g < k) {
+      const bool e = v[r] == kEmpty;
+      const float dv = e ? __int_as_float(0x7f800000) : key_dist(v[r]);
+      out_ids[q * k + g] = e ? -1 : (int64_t)key_index(v[r]);
+      out_d[q * k + g] = e ? dv : (metric == HENN_ANGULAR ? dv : sqrtf(dv));
+    }
+  }
+}
+
+// Forward lists from the KP tile candidates of each row (rank space), with
+// the certificate above; a row that fails it is flagged.
+template <int KP>
+__global__ void __launch_bounds__(256) k_rerank_fwd(const float* __restrict__ xw, const int32_t* __restrict__ ids,
+                                                    int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
+                                                    const int32_t* __restrict__ inv, const uint64_t* __restrict__ cand,
+                                                    int32_t M, const float* __restrict__ norms,
+                                                    const float* __restrict__ norm_max, double tile_u,
+                                                    int32_t* __restrict__ fwd, float* __restrict__ fwd_d,
+                                                    FlaggedRows flagged) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < nr;
+       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t j = inv ? (int64_t)inv[r] : row0 + r;
+    const float* xj = xw + (ids ? (int64_t)ids[j] : j) * dpad;
+    uint64_t v[KP / 32];
+#pragma unroll
+    for (int i = 0; i < KP / 32; ++i) v[i] = kEmpty;
+    uint64_t last = kEmpty;  // the pool's last key, if it is full
+#pragma unroll 1
+    for (int b = 0; b < KP; b += 32) {
+      const uint64_t key = __ldg(cand + r * KP + b + lane);
+      const int cnt = __popc(__ballot_sync(0xffffffffu, key != kEmpty));  // the pool is sorted: empty keys last
+      last = shfl64(key, 31);
+      if (cnt == 0) break;
+      int64_t qj = 0, gq = 0;
+      if (lane < cnt) {
+        qj = inv ? (int64_t)inv[key_index(key)] : (int64_t)key_index(key);
+        gq = ids ? (int64_t)ids[qj] : qj;
+      }
+      const float dv = warp_exact_dist32(xj, xw, gq, cnt, dpad, metric);
+      merge_sorted32(v, warp_sort_asc(lane < cnt ? pack(dv, (uint32_t)qj) : kEmpty));
+    }
+    if (last != kEmpty) {
+      const uint64_t mkey = list_key(v, M - 1);
+      double dm = (mkey == kEmpty) ? 1e300 : (double)key_dist(mkey);
+      // exact distances here are of raw vectors; tile distances of centred
+      // ones: identical in exact arithmetic.  Angular: tile values are 2x.
+      if (metric == HENN_ANGULAR) dm *= 2.0;
+      float collect;
+      if (!pool_certified((double)key_dist(last), dm, norms[r], *norm_max, tile_u, dpad, &collect))
+        flag_row(flagged, (int32_t)r, collect);
+    }
+    write_fwd(v, j, M, fwd, fwd_d);
+  }
+}
+
+void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
+                       const int32_t* inv, const uint64_t* cand, int32_t KP, int32_t M, const float* norms,
+                       const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d, const FlaggedRows& flagged,
+                       cudaStream_t st) {
+  int grid = (int)((nr + 7) / 8);
   if (grid > 152 * 32) grid = 152 * 32;
   if (grid < 1) grid = 1;
   switch (KP) {
     case 32:
-      k_rerank_fwd<32><<<grid, 256, 0, st>>>(xw, ids, s, dpad, metric, inv, cand, M, norms, norm_max, tile_u, fwd,
-                                             fwd_d, uncertified);
+      k_rerank_fwd<32><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, M, norms, norm_max, tile_u, fwd,
+                                             fwd_d, flagged);
       break;
     case 64:
-      k_rerank_fwd<64><<<grid, 256, 0, st>>>(xw, ids, s, dpad, metric, inv, cand, M, norms, norm_max, tile_u, fwd,
-                                             fwd_d, uncertified);
+      k_rerank_fwd<64><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, M, norms, norm_max, tile_u, fwd,
+                                             fwd_d, flagged);
       break;
     default:
-      k_rerank_fwd<128><<<grid, 256, 0, st>>>(xw, ids, s, dpad, metric, inv, cand, M, norms, norm_max, tile_u, fwd,
-                                              fwd_d, uncertified);
+      k_rerank_fwd<128><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, M, norms, norm_max, tile_u,
+                                              fwd, fwd_d, flagged);
       break;
   }
+}
+
+template <int KP>
+__global__ void __launch_bounds__(256) k_rerank_knn(const float* __restrict__ Q, int64_t nq, const float* __restrict__ X,
+                                                    int64_t n, int32_t dpad, int32_t metric,
+                                                    const uint64_t* __restrict__ cand, const float* __restrict__ thr,
+                                                    int32_t k, const float* __restrict__ qnorms,
+                                                    const float* __restrict__ norm_max, double tile_u,
+                                                    const int32_t* __restrict__ err, int64_t* __restrict__ out_ids,
+                                                    float* __restrict__ out_d, FlaggedRows flagged) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < nq;
+       q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    uint64_t v[KP / 32];
+#pragma unroll
+    for (int i = 0; i < KP / 32; ++i) v[i] = kEmpty;
+    int64_t total = 0;
+#pragma unroll 1
+    for (int b = 0; b < KP; b += 32) {
+      const uint64_t key = __ldg(cand + q * KP + b + lane);
+      const int cnt = __popc(__ballot_sync(0xffffffffu, key != kEmpty));
+      if (cnt == 0) break;
+      total += cnt;
+      const int64_t col = lane < cnt ? (int64_t)key_index(key) : 0;
+      const float dv = warp_exact_dist32(Q + q * dpad, X, col, cnt, dpad, metric);
+      merge_sorted32(v, warp_sort_asc(lane < cnt ? pack(dv, (uint32_t)col) : kEmpty));
+    }
+    if (total < n || *err != 0) {
+      const uint64_t mkey = list_key(v, k - 1);
+      double dm = mkey == kEmpty ? 1e300 : (double)key_dist(mkey);
+      if (metric == HENN_ANGULAR) dm *= 2.0;
+      float collect;
+      const bool ok = pool_certified((double)thr[q], dm, qnorms[q], *norm_max, tile_u, dpad, &collect);
+      if (!ok || *err != 0) flag_row(flagged, (int32_t)q, collect);
+    }
+    write_knn(v, q, k, metric, out_ids, out_d);
+  }
+}
+
+void launch_rerank_knn(const float* Q, int64_t nq, const float* X, int64_t n, int32_t dpad, int32_t metric,
+                       const uint64_t* cand, const float* thr, int32_t KP, int32_t k, const float* qnorms,
+                       const float* norm_max, double tile_u, const int32_t* err, int64_t* out_ids, float* out_d,
+                       const FlaggedRows& flagged, cudaStream_t st) {
+  int grid = (int)((nq + 7) / 8);
+  if (grid > 152 * 32) grid = 152 * 32;
+  if (KP == 32)
+    k_rerank_knn<32><<<grid, 256, 0, st>>>(Q, nq, X, n, dpad, metric, cand, thr, k, qnorms, norm_max, tile_u, err,
+                                           out_ids, out_d, flagged);
+  else if (KP == 64)
+    k_rerank_knn<64><<<grid, 256, 0, st>>>(Q, nq, X, n, dpad, metric, cand, thr, k, qnorms, norm_max, tile_u, err,
+                                           out_ids, out_d, flagged);
+  else
+    k_rerank_knn<128><<<grid, 256, 0, st>>>(Q, nq, X, n, dpad, metric, cand, thr, k, qnorms, norm_max, tile_u, err,
+                                            out_ids, out_d, flagged);
+}
+
+// ------------------------------------------ rows the pool did not settle
+
+__global__ void __launch_bounds__(256) k_gather_flagged(FlaggedRows f, int64_t max_rows, int64_t row0, int32_t causal,
+                                                        int32_t skip_self, int64_t nb, const uint4* __restrict__ hi,
+                                                        const uint4* __restrict__ lo, const float* __restrict__ norms,
+                                                        int32_t quads, uint4* __restrict__ hi_out,
+                                                        uint4* __restrict__ lo_out, float* __restrict__ norms_out,
+                                                        int32_t* __restrict__ lim, int32_t* __restrict__ self) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nf = min((int64_t)*f.count, max_rows);
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < nf;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t r = f.rows[i];
+    for (int c = lane; c < quads; c += 32) {
+      hi_out[i * quads + c] = __ldg(hi + r * quads + c);
+      lo_out[i * quads + c] = __ldg(lo + r * quads + c);
+    }
+    if (lane == 0) {
+      norms_out[i] = norms[r];
+      lim[i] = (int32_t)(causal ? row0 + r : nb);
+      self[i] = skip_self ? (int32_t)r : -1;
+    }
+  }
+}
+
+void launch_gather_flagged(const FlaggedRows& f, int64_t max_rows, int64_t row0, bool causal, bool skip_self,
+                           int64_t nb, const void* hi, const void* lo, const float* norms, int32_t dk, void* hi_out,
+                           void* lo_out, float* norms_out, int32_t* lim, int32_t* self, cudaStream_t st) {
+  int grid = (int)((max_rows + 7) / 8);
+  if (grid > 152 * 8) grid = 152 * 8;
+  k_gather_flagged<<<grid, 256, 0, st>>>(f, max_rows, row0, causal ? 1 : 0, skip_self ? 1 : 0, nb,
+                                         static_cast<const uint4*>(hi), static_cast<const uint4*>(lo), norms, dk / 8,
+                                         static_cast<uint4*>(hi_out), static_cast<uint4*>(lo_out), norms_out, lim,
+                                         self);
+}
+
+// One warp per flagged row: its collected columns' exact distances into a
+// sorted list.  `row` gives the column's row in X, `to_key` its key index.
+template <int R, class RowOf, class KeyOf>
+__device__ __forceinline__ bool rerank_collected(const float* __restrict__ a, const float* __restrict__ X, int64_t i,
+                                                 int32_t ns, const uint32_t* __restrict__ cols,
+                                                 const int32_t* __restrict__ ncols, int32_t cap, int32_t dpad,
+                                                 int32_t metric, RowOf row_of, KeyOf key_of, uint64_t (&v)[R]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < R; ++q) v[q] = kEmpty;
+  const int64_t seg0 = (i / kTileRows) * ns * kTileRows + i % kTileRows;
+  bool over = false;
+  for (int s = lane; s < ns; s += 32) over |= ncols[seg0 + (int64_t)s * kTileRows] > cap;
+  if (__any_sync(0xffffffffu, over)) return false;
+  for (int s = 0; s < ns; ++s) {
+    const int64_t seg = seg0 + (int64_t)s * kTileRows;
+    const int c = ncols[seg];
+    for (int b = 0; b < c; b += 32) {
+      const int cnt = min(32, c - b);
+      const uint32_t col = lane < cnt ? cols[seg * cap + b + lane] : 0u;
+      const int64_t key = lane < cnt ? (int64_t)key_of(col) : 0;
+      const int64_t row = lane < cnt ? (int64_t)row_of(key) : 0;
+      const float dv = warp_exact_dist32(a, X, row, cnt, dpad, metric);
+      merge_sorted32(v, warp_sort_asc(lane < cnt ? pack(dv, (uint32_t)key) : kEmpty));
+    }
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(256) k_rerank_collected_fwd(const float* __restrict__ xw,
+                                                              const int32_t* __restrict__ ids, FlaggedRows f,
+                                                              int64_t max_rows, int64_t row0, int32_t dpad,
+                                                              int32_t metric, const int32_t* __restrict__ inv,
+                                                              int64_t nb, unsigned grid,
+                                                              const uint32_t* __restrict__ cols,
+                                                              const int32_t* __restrict__ ncols, int32_t cap,
+                                                              int32_t M, int32_t* __restrict__ fwd,
+                                                              float* __restrict__ fwd_d, int32_t* __restrict__ over,
+                                                              const int32_t* __restrict__ err) {
+  const int64_t nf = min((int64_t)*f.count, max_rows);
+  if (nf <= 0) return;
+  const int32_t ns = collect_splits(grid, nf, nb);
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < nf;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t r = f.rows[i];
+    const int64_t j = inv ? (int64_t)inv[r] : row0 + r;
+    uint64_t v[1];  // M <= 32
+    const bool ok = *err == 0 && rerank_collected(
+                                     xw + (ids ? (int64_t)ids[j] : j) * dpad, xw, i, ns, cols, ncols, cap, dpad, metric,
+                                     [&](int64_t pos) { return ids ? (int64_t)ids[pos] : pos; },
+                                     [&](uint32_t c) { return inv ? (uint32_t)inv[c] : c; }, v);
+    if (ok)
+      write_fwd(v, j, M, fwd, fwd_d);
+    else if ((threadIdx.x & 31) == 0)
+      over[1 + atomicAdd(over, 1)] = (int32_t)(row0 + r);
+  }
+}
+
+void launch_rerank_collected_fwd(const float* xw, const int32_t* ids, const FlaggedRows& f, int64_t max_rows,
+                                 int64_t row0, int32_t dpad, int32_t metric, const int32_t* inv, int64_t nb,
+                                 unsigned grid, const uint32_t* cols, const int32_t* ncols, int32_t cap, int32_t M,
+                                 int32_t* fwd, float* fwd_d, int32_t* over, const int32_t* err, cudaStream_t st) {
+  int g = (int)((max_rows + 7) / 8);
+  if (g > 152 * 16) g = 152 * 16;
+  k_rerank_collected_fwd<<<g, 256, 0, st>>>(xw, ids, f, max_rows, row0, dpad, metric, inv, nb, grid, cols, ncols, cap,
+                                            M, fwd, fwd_d, over, err);
+}
+
+__global__ void __launch_bounds__(256) k_rerank_collected_knn(const float* __restrict__ Q, const float* __restrict__ X,
+                                                              FlaggedRows f, int64_t max_rows, int32_t dpad,
+                                                              int32_t metric, int64_t nb, unsigned grid,
+                                                              const uint32_t* __restrict__ cols,
+                                                              const int32_t* __restrict__ ncols, int32_t cap,
+                                                              int32_t k, int64_t* __restrict__ out_ids,
+                                                              float* __restrict__ out_d, int32_t* __restrict__ over,
+                                                              const int32_t* __restrict__ err) {
+  const int64_t nf = min((int64_t)*f.count, max_rows);
+  if (nf <= 0) return;
+  const int32_t ns = collect_splits(grid, nf, nb);
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < nf;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t q = f.rows[i];
+    uint64_t v[4];  // k <= 112
+    const bool ok = *err == 0 &&
+                    rerank_collected(
+                        Q + q * dpad, X, i, ns, cols, ncols, cap, dpad, metric, [](int64_t c) { return c; },
+                        [](uint32_t c) { return c; }, v) &&
+                    list_key(v, k - 1) != kEmpty;
+    if (ok)
+      write_knn(v, q, k, metric, out_ids, out_d);
+    else if ((threadIdx.x & 31) == 0)
+      over[1 + atomicAdd(over, 1)] = (int32_t)q;
+  }
+}
+
+void launch_rerank_collected_knn(const float* Q, const float* X, const FlaggedRows& f, int64_t max_rows, int32_t dpad,
+                                 int32_t metric, int64_t nb, unsigned grid, const uint32_t* cols,
+                                 const int32_t* ncols, int32_t cap, int32_t k, int64_t* out_ids, float* out_d,
+                                 int32_t* over, const int32_t* err, cudaStream_t st) {
+  int g = (int)((max_rows + 7) / 8);
+  if (g > 152 * 16) g = 152 * 16;
+  k_rerank_collected_knn<<<g, 256, 0, st>>>(Q, X, f, max_rows, dpad, metric, nb, grid, cols, ncols, cap, k, out_ids,
+                                            out_d, over, err);
 }
 
 // Exact forward lists of flagged rows, batched: a block takes RT flagged
@@ -500,14 +872,17 @@ void launch_exact_rows(const float* xw, const int32_t* ids, int64_t s, int32_t d
 template <int KP>
 __global__ void k_rerank_queries(const float* __restrict__ Q, int64_t nq, const float* __restrict__ X, int32_t dpad,
                                  int32_t metric, const uint64_t* __restrict__ cand, int32_t k,
-                                 int64_t* __restrict__ out_ids, float* __restrict__ out_d) {
+                                 int64_t* __restrict__ out_ids, float* __restrict__ out_d,
+                                 const int32_t* __restrict__ rowsel, const int32_t* __restrict__ count) {
   const int lane = threadIdx.x & 31;
-  for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; q < nq;
-       q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+  const int64_t nl = count ? min(nq, (int64_t)*count) : nq;
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < nl;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t q = rowsel ? (int64_t)rowsel[i] : i;
     WarpList<KP> list;
     list.clear();
     for (int c = 0; c < KP; ++c) {
-      uint64_t key = cand[q * KP + c];
+      uint64_t key = cand[i * KP + c];
       if (key == kEmpty) break;
       uint32_t col = key_index(key);
       float dv = warp_exact_dist(Q + q * dpad, X + (int64_t)col * dpad, dpad, metric);
@@ -528,15 +903,16 @@ __global__ void k_rerank_queries(const float* __restrict__ Q, int64_t nq, const 
 }
 
 void launch_rerank_queries(const float* Q, int64_t nq, const float* X, int32_t dpad, int32_t metric, const uint64_t* cand,
-                           int32_t KP, int32_t k, int64_t* out_ids, float* out_d, cudaStream_t st) {
+                           int32_t KP, int32_t k, int64_t* out_ids, float* out_d, const int32_t* rowsel,
+                           const int32_t* count, cudaStream_t st) {
   int grid = (int)((nq + 7) / 8);
   if (grid > 152 * 32) grid = 152 * 32;
   if (grid < 1) grid = 1;
   switch (KP) {
-    case 32: k_rerank_queries<32><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d); break;
-    case 64: k_rerank_queries<64><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d); break;
-    case 128: k_rerank_queries<128><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d); break;
-    default: k_rerank_queries<256><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d); break;
+    case 32: k_rerank_queries<32><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
+    case 64: k_rerank_queries<64><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
+    case 128: k_rerank_queries<128><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
+    default: k_rerank_queries<256><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
   }
 }
 

@@ -7,7 +7,9 @@
 // (causal, NSW) or c != r (kNN graph); mode 2 takes the rows from one set
 // (queries) and every column from another (a layer's points); mode 3 is
 // mode 2 writing every tile value (the distance matrix, as 16-bit keys that
-// keep the order of the distances) instead of lists.
+// keep the order of the distances) instead of lists; mode 4 keeps no lists
+// either: every row has a fixed threshold, and each valid column whose tile
+// value is at or under it is appended to the row's buffer in global memory.
 //
 // Precision: each FP32 operand is split into x = hi + lo with hi =
 // bf16(x), lo = bf16(x - hi); the tile accumulates hi.hi + lo.hi + hi.lo in
@@ -34,6 +36,7 @@
 #include <cudaTypedefs.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstddef>
 #include <cstdlib>
@@ -299,9 +302,20 @@ __device__ __forceinline__ void heap_replace(uint64_t* heap, uint64_t key) {
 
 using namespace tc;
 
+// Per-row arguments of a tile launch (each nullable) and mode 4's output.
+struct TileRows {
+  const int32_t* lim;    // row r takes columns 0 .. lim[r] - 1
+  const int32_t* self;   // ... except column self[r] (-1: none)
+  const float* thr;      // mode 4: the rows' thresholds
+  const int32_t* count;  // mode 4: the number of rows, on the device
+  uint32_t* cols;        // mode 4: CTA b, row r of its block: cap columns at (b * 128 + r) * cap
+  int32_t* ncols;        // ... and their number (over cap: dropped)
+  int32_t cap;
+};
+
 // EPI: epilogue warps, 4 (one per TMEM sub-partition; the per-row lists of
-// modes 0-2 need it) or 8 (mode 3: two per sub-partition, each taking half of
-// every tile's chunks); the launch has 64 + 32 * EPI threads
+// modes 0-2 need it) or 8 (modes 3 and 4: two per sub-partition, each taking
+// half of every tile's chunks); the launch has 64 + 32 * EPI threads
 template <bool kStream, int BN, int EPI>
 __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     k_tile_topk_tc(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
@@ -310,26 +324,39 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
                    const float* __restrict__ norms, const float* __restrict__ norms_c, int64_t s, int64_t sc,
                    int32_t kc, int32_t mode, uint64_t* __restrict__ out, uint16_t* __restrict__ out_d, int64_t ldo,
                    float* __restrict__ out_cmin, int64_t ldc,
-                   int32_t nsplit, int32_t* __restrict__ err, long long spin_limit, int32_t hold) {
+                   int32_t nsplit, const __grid_constant__ TileRows rows, int32_t* __restrict__ err,
+                   long long spin_limit, int32_t hold) {
   using Smem = typename std::conditional<kStream, SmemStr<BN>, SmemRes<BN>>::type;
   constexpr int NST = kStream ? NS_STR : NS;
   constexpr int B_CHUNK = BN * BK * 2;  // one plane of a B slice
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (EPI == 8 && rows.count) {
+    // mode 4: the number of rows is read on the device, and the grid's CTAs
+    // are shared out over the row blocks there are
+    s = min((int64_t)*rows.count, s);
+    if (s <= 0) return;
+    nsplit = collect_splits(gridDim.x, s, sc);
+    if (blockIdx.x >= (unsigned)(((s + BM - 1) / BM) * nsplit)) return;
+  }
   const int64_t nrb = (s + BM - 1) / BM;
-  // nsplit CTAs per row block (mode 3, which keeps no per-row lists), each
-  // taking a contiguous run of the block's tiles
+  // nsplit CTAs per row block: in mode 3 each takes a contiguous run of the
+  // block's tiles, else every nsplit-th one (so that points that lie together
+  // in the order are spread over the CTAs' lists)
   const int64_t bid = blockIdx.x / nsplit;
   const int sp = (int)(blockIdx.x % nsplit);
   const int64_t rb = (mode == 0) ? (nrb - 1 - bid) : bid;
   const int64_t r0 = rb * BM;
-  // s rows; sc columns (== s unless mode 2 or 3)
+  // s rows; sc columns (== s in modes 0 and 1)
   const int64_t cend = (mode == 0) ? min(s, r0 + BM) : sc;
   const int nt_all = (int)((cend + BN - 1) / BN);
+  const bool runs = EPI == 8 && mode == 3;
   const int tps = (nt_all + nsplit - 1) / nsplit;
-  const int t0 = min(nt_all, sp * tps);
-  const int nt = min(nt_all, t0 + tps) - t0;  // this CTA's tiles: t0 .. t0 + nt - 1
+  const int tstep = runs ? 1 : nsplit;
+  const int t0 = runs ? min(nt_all, sp * tps) : sp;
+  // this CTA's tiles: t0, t0 + tstep, ... (nt of them)
+  const int nt = runs ? min(nt_all, t0 + tps) - t0 : (sp < nt_all ? (nt_all - sp + nsplit - 1) / nsplit : 0);
   const int chunks_per_tile = 2 * kc;  // (B_hi, B_lo) per 64-wide slice
 
   if (threadIdx.x == 0) {
@@ -346,8 +373,13 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
-  for (int i = threadIdx.x; i < BM * (KP + 2); i += blockDim.x)
-    (&sm.heap[0][0])[i] = (i % (KP + 2) == KP + 1) ? 0ull : kEmpty;
+  // the rows' heaps; in mode 4 the rows' column counts instead
+  if (EPI == 4) {
+    for (int i = threadIdx.x; i < BM * (KP + 2); i += blockDim.x)
+      (&sm.heap[0][0])[i] = (i % (KP + 2) == KP + 1) ? 0ull : kEmpty;
+  } else if (threadIdx.x < BM) {
+    reinterpret_cast<int*>(&sm.heap[0][0])[threadIdx.x] = 0;
+  }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(tc::smem_u32(&sm.tmem_base)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -372,7 +404,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
           tc::tma_load_2d(sm.a[MAX_KC_RES + c], &ta_lo, &sm.afull, c * BK, (int)r0);
         }
         for (int lt = 0; lt < nt && ok; ++lt) {
-          const int t = t0 + lt;
+          const int t = t0 + lt * tstep;
           for (int j = 0; j < chunks_per_tile && ok; ++j, ++it) {
             const int st = (int)(it % NST);
             const uint32_t ph = (uint32_t)((it / NST) & 1);
@@ -388,7 +420,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       } else {
         // per slice: the A slice (hi | lo), B hi, B lo, in this order
         for (int lt = 0; lt < nt && ok; ++lt) {
-          const int t = t0 + lt;
+          const int t = t0 + lt * tstep;
           for (int j = 0; j < kc && ok; ++j) {
             for (int part = 0; part < 3; ++part, ++it) {
               const int st = (int)(it % NST);
@@ -503,12 +535,17 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     const int64_t grow = r0 + row_l;
     const float nrow = grow < s ? norms[grow] : 0.f;
     // valid columns of this row: [0, lim), minus the row itself for kNN
-    const int32_t lim = grow >= s ? 0 : (int32_t)(mode == 0 ? grow : sc);
-    const int32_t self = mode == 1 ? (int32_t)grow : -1;
+    // (rows.lim: a limit per row, rows.self: an excluded column per row)
+    const int32_t lim = grow >= s ? 0 : (rows.lim ? rows.lim[grow] : (int32_t)(mode == 0 ? grow : sc));
+    const int32_t self = rows.self && grow < s ? rows.self[grow] : (mode == 1 ? (int32_t)grow : -1);
     const float kInf = __int_as_float(0x7f800000);
     // the row's threshold with its own norm folded in:
     // n_row + n_col - 2v <= thr  <=>  n_col - 2v <= thr - n_row
     float thr_adj = kInf;
+    if (EPI == 8 && mode == 4) {
+      const float thr = grow < s ? rows.thr[grow] : 0.f;
+      thr_adj = thr - nrow + 1e-6f * (fabsf(thr) + fabsf(nrow));
+    }
     uint64_t* heap = sm.heap[row_l];
     uint64_t root = kEmpty;
     // mode 3 keeps no lists: the heap space holds each warp's 4 KB store
@@ -522,7 +559,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       pn[q] = c < sc && q >= qlo && q < qhi ? __ldg(norms_c + c) : 0.f;
     }
     for (int lt = 0; lt < nt; ++lt) {
-      const int t = t0 + lt;
+      const int t = t0 + lt * tstep;
       const int as = lt & 1;
       const uint32_t aph = (uint32_t)((lt >> 1) & 1);
       if (!tc::mbar_wait(&sm.tfull[as], aph, abort_flag, spin_limit)) {
@@ -538,7 +575,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
         if (q >= qlo && q < qhi) ncs[q * 32 + lane] = pn[q];
 #pragma unroll
       for (int q = 0; q < BN / 32; ++q) {
-        const int64_t c = (int64_t)(t + 1) * BN + q * 32 + lane;
+        const int64_t c = (int64_t)(t + tstep) * BN + q * 32 + lane;
         pn[q] = c < sc && q >= qlo && q < qhi ? __ldg(norms_c + c) : 0.f;
       }
       if (mode == 3 && out_cmin)
@@ -598,7 +635,48 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
         }
         __syncwarp();
       };
-      if (mode != 3) {
+      if (EPI == 8 && mode == 4) {
+        // the columns at or under the row's threshold, appended to its
+        // buffer: few once the threshold is a row's known M-th distance
+        int* cnt = reinterpret_cast<int*>(&sm.heap[0][0]);
+        uint32_t* buf = rows.cols + ((int64_t)blockIdx.x * BM + row_l) * rows.cap;
+#pragma unroll 1
+        for (int q = qlo; q < qhi; q += 2) {
+          const int64_t ca = (int64_t)t * BN + q * 32;
+          uint32_t ra[32], rb[32];
+          tc::tmem_ld32_issue(tacc + (uint32_t)q * 32, ra);
+          tc::tmem_ld32_issue(tacc + (uint32_t)(q + 1) * 32, rb);
+          tc::tmem_ld_wait(ra);
+          tc::tmem_regs_after(rb);
+          if (ca >= cend) continue;  // warp-uniform
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float v[32];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(h == 0 ? ra[i] : rb[i]);
+            const float vmin = prep(q + h, v);
+            if (!(vmin <= thr_adj)) continue;
+            const int32_t c0 = (int32_t)ca + 32 * h;
+            const int32_t rem = lim - c0;
+            unsigned keep = 0;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) keep |= (v[j] <= thr_adj) ? (1u << j) : 0u;
+            keep &= rem >= 32 ? 0xffffffffu : (rem <= 0 ? 0u : ((1u << rem) - 1u));
+            const int32_t so = self - c0;
+            if (so >= 0 && so < 32) keep &= ~(1u << so);
+            if (!keep) continue;
+            int at = atomicAdd(&cnt[row_l], __popc(keep));
+            do {
+              const int j = __ffs(keep) - 1;
+              keep &= keep - 1;
+              if (at < rows.cap) buf[at] = (uint32_t)(c0 + j);
+              ++at;
+            } while (keep);
+          }
+          __syncwarp();
+        }
+      }
+      if (EPI == 4) {
         // two chunks at a time: both TMEM loads behind one wait, the two
         // chunks' distance terms interleaved, then their inserts in chunk
         // order (the same lists as one chunk at a time)
@@ -626,7 +704,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       // mode 3: the distances as 16-bit keys, two 32-column chunks (64
       // columns, one 128-byte row of the box) at a time behind one TMEM wait
 #pragma unroll 1
-      for (int q = qlo; q < qhi && mode == 3; q += 2) {
+      for (int q = qlo; q < qhi && runs; q += 2) {
         const int64_t c0 = (int64_t)t * BN + q * 32;
         uint32_t ra[32], rb[32];
         tc::tmem_ld32_issue(tacc + (uint32_t)q * 32, ra);
@@ -716,14 +794,17 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     if (mode == 3 && lane == 0) tc::bulk_wait_all();
     // this warp's 32 rows, each heap sorted ascending across the warp
     __syncwarp();
-    for (int i = 0; i < 32 && mode != 3; ++i) {
+    for (int i = 0; i < 32 && EPI == 4; ++i) {
       const int64_t gr = r0 + 32 * sub + i;
       const uint64_t x = warp_sort_asc(sm.heap[32 * sub + i][1 + lane]);
-      if (gr < s) out[gr * KP + lane] = x;
+      if (gr < s) out[((int64_t)sp * s + gr) * KP + lane] = x;
     }
   }
   tc::fence_before();
   __syncthreads();
+  // mode 4: how many columns each row has (over rows.cap: the rest were dropped)
+  if (EPI == 8 && mode == 4 && threadIdx.x < BM)
+    rows.ncols[(int64_t)blockIdx.x * BM + threadIdx.x] = reinterpret_cast<const int*>(&sm.heap[0][0])[threadIdx.x];
   if (sm.abort) {
     // let any bulk copy still in flight land before the CTA leaves
     __nanosleep(100000);
@@ -824,16 +905,16 @@ static_assert((2 * A_CHUNK) <= STAGE && BN_MAX * BK * 2 <= STAGE && A_CHUNK % 10
 // variant.
 struct TileVariant {
   void (*fn)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, const float*, const float*, int64_t,
-             int64_t, int32_t, int32_t, uint64_t*, uint16_t*, int64_t, float*, int64_t, int32_t, int32_t*, long long,
-             int32_t);
+             int64_t, int32_t, int32_t, uint64_t*, uint16_t*, int64_t, float*, int64_t, int32_t, TileRows, int32_t*,
+             long long, int32_t);
   size_t smem;
 };
 
-static cudaError_t tile_variant(int32_t kc, int32_t bn, bool matrix, TileVariant* v) {
+static cudaError_t tile_variant(int32_t kc, int32_t bn, bool eight, TileVariant* v) {
   static std::atomic<bool> attr_set[8][64];
   const int stream = kc > MAX_KC_RES ? 1 : 0;
   const int narrow = bn == 128 ? 1 : 0;
-  const int which = 4 * (matrix ? 1 : 0) + 2 * stream + narrow;
+  const int which = 4 * (eight ? 1 : 0) + 2 * stream + narrow;
   switch (which) {
     case 0: v->fn = k_tile_topk_tc<false, 256, 4>; v->smem = sizeof(SmemRes<256>); break;
     case 1: v->fn = k_tile_topk_tc<false, 128, 4>; v->smem = sizeof(SmemRes<128>); break;
@@ -856,27 +937,104 @@ static cudaError_t tile_variant(int32_t kc, int32_t bn, bool matrix, TileVariant
   return cudaSuccess;
 }
 
-cudaError_t launch_tile_topk_tc(const float* xo, const float* norms, int64_t s, int32_t dpad, int32_t mode,
-                                uint64_t* out, void* scratch_hi, void* scratch_lo, int32_t* err, cudaStream_t st) {
-  const int32_t dk = ((dpad + BK - 1) / BK) * BK;
-  __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(scratch_hi);
-  __nv_bfloat16* lo = static_cast<__nv_bfloat16*>(scratch_lo);
-  k_split_bf16<<<152 * 8, 256, 0, st>>>(xo, s, dpad, dk, hi, lo);
+static int sm_count(int dev) {
+  int sms = 1;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
+  return sms;
+}
+
+// CTAs per row block for the list modes: the split with the fewest
+// tile-times over all waves of one CTA per SM, or for the causal mode (whose
+// row blocks are unequal, the longest first) the longer of the even share and
+// the longest CTA.  A CTA's fixed work -- set-up, the first fill of its lists
+// -- counts as kListFill tiles.
+constexpr int kListFill = 6;
+
+int32_t tile_list_splits(int64_t na, int64_t nb, bool causal) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  const int64_t sms = sm_count(dev);
+  const int64_t nrb = (na + BM - 1) / BM;
+  const int64_t nt = (nb + BN_MAX - 1) / BN_MAX;
+  double best = 1e300;
+  int32_t pick = 1;
+  for (int64_t k = 1; k <= nt && k <= (causal ? 16 : sms); ++k) {
+    const double longest = (double)((nt + k - 1) / k + kListFill);
+    double cost;
+    if (causal)
+      cost = std::max((double)nrb * (0.5 * (double)nt + (double)(k * kListFill)) / (double)sms, longest);
+    else
+      cost = (double)((nrb * k + sms - 1) / sms) * longest;
+    if (cost < best * 0.99) {  // more lists only for a gain
+      best = cost;
+      pick = (int32_t)k;
+    }
+  }
+  return pick;
+}
+
+cudaError_t launch_tile_lists_tc(const void* a_hi, const void* a_lo, const float* a_norms, int64_t na,
+                                 const void* b_hi, const void* b_lo, const float* b_norms, int64_t nb, int32_t dk,
+                                 int32_t mode, const int32_t* lim, int32_t splits, uint64_t* out, int32_t* err,
+                                 cudaStream_t st) {
+  if (dk % BK != 0 || dk / BK > MAX_KC || na < 1 || nb < 1 || splits < 1 || mode < 0 || mode > 2)
+    return cudaErrorInvalidValue;
   CUtensorMap mah, mal, mbh, mbl;
-  if (!make_map(&mah, hi, s, dk, BM) || !make_map(&mal, lo, s, dk, BM) || !make_map(&mbh, hi, s, dk, BN_MAX) ||
-      !make_map(&mbl, lo, s, dk, BN_MAX))
+  if (!make_map(&mah, a_hi, na, dk, BM) || !make_map(&mal, a_lo, na, dk, BM) || !make_map(&mbh, b_hi, nb, dk, BN_MAX) ||
+      !make_map(&mbl, b_lo, nb, dk, BN_MAX))
     return cudaErrorInvalidValue;
   TileVariant v;
   cudaError_t e = tile_variant(dk / BK, BN_MAX, false, &v);
   if (e != cudaSuccess) return e;
-  const int64_t nrb = (s + BM - 1) / BM;
-  CUtensorMap none;  // no matrix output in modes 0 and 1
+  const int64_t nrb = (na + BM - 1) / BM;
+  CUtensorMap none;  // no matrix output
   std::memset(&none, 0, sizeof(none));
+  TileRows rows;
+  std::memset(&rows, 0, sizeof(rows));
+  rows.lim = lim;
   long long spin_limit;
   int32_t hold;
   wait_policy(&spin_limit, &hold);
-  v.fn<<<(unsigned)nrb, 192, v.smem, st>>>(mah, mal, mbh, mbl, none, norms, norms, s, s, dk / BK, mode, out, nullptr,
-                                           0, nullptr, 0, 1, err, spin_limit, hold);
+  v.fn<<<(unsigned)(nrb * splits), 192, v.smem, st>>>(mah, mal, mbh, mbl, none, a_norms, b_norms, na, nb, dk / BK, mode,
+                                                      out, nullptr, 0, nullptr, 0, splits, rows, err, spin_limit,
+                                                      hold);
+  return cudaGetLastError();
+}
+
+unsigned tile_collect_grid(int64_t max_rows) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  return (unsigned)std::max<int64_t>(sm_count(dev), (max_rows + BM - 1) / BM);
+}
+
+cudaError_t launch_tile_collect_tc(const void* a_hi, const void* a_lo, const float* a_norms, int64_t max_rows,
+                                   const void* b_hi, const void* b_lo, const float* b_norms, int64_t nb, int32_t dk,
+                                   const int32_t* lim, const int32_t* self, const float* thr, const int32_t* count,
+                                   unsigned grid, uint32_t* cols, int32_t* ncols, int32_t cap, int32_t* err,
+                                   cudaStream_t st) {
+  if (dk % BK != 0 || dk / BK > MAX_KC || max_rows < 1 || nb < 1 || !thr || !count) return cudaErrorInvalidValue;
+  CUtensorMap mah, mal, mbh, mbl;
+  if (!make_map(&mah, a_hi, max_rows, dk, BM) || !make_map(&mal, a_lo, max_rows, dk, BM) ||
+      !make_map(&mbh, b_hi, nb, dk, BN_MAX) || !make_map(&mbl, b_lo, nb, dk, BN_MAX))
+    return cudaErrorInvalidValue;
+  TileVariant v;
+  cudaError_t e = tile_variant(dk / BK, BN_MAX, true, &v);
+  if (e != cudaSuccess) return e;
+  CUtensorMap none;
+  std::memset(&none, 0, sizeof(none));
+  TileRows rows;
+  rows.lim = lim;
+  rows.self = self;
+  rows.thr = thr;
+  rows.count = count;
+  rows.cols = cols;
+  rows.ncols = ncols;
+  rows.cap = cap;
+  long long spin_limit;
+  int32_t hold;
+  wait_policy(&spin_limit, &hold);
+  v.fn<<<grid, 64 + 32 * 8, v.smem, st>>>(mah, mal, mbh, mbl, none, a_norms, b_norms, max_rows, nb, dk / BK, 4, nullptr,
+                                          nullptr, 0, nullptr, 0, 1, rows, err, spin_limit, hold);
   return cudaGetLastError();
 }
 
@@ -919,8 +1077,7 @@ cudaError_t launch_tile_cross_tc(const void* a_hi, const void* a_lo, const float
   // fits), choosing the split with the fewest tile-times over all waves
   int32_t nsplit = 1;
   if (out_d) {
-    int sms = 1;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
+    const int sms = sm_count(dev);
     const int64_t nt_all = (nb + BN - 1) / BN;
     double best = 1e300;
     for (int64_t k = 1; k <= nt_all && k <= 16; ++k) {
@@ -939,9 +1096,11 @@ cudaError_t launch_tile_cross_tc(const void* a_hi, const void* a_lo, const float
   int32_t hold;
   wait_policy(&spin_limit, &hold);
   // mode 3: eight epilogue warps (two per TMEM sub-partition); mode 2: four
-  v.fn<<<(unsigned)(nrb * nsplit), out_d ? 64 + 32 * 8 : 64 + 32 * 4, v.smem, st>>>(mah, mal, mbh, mbl, mo, a_norms, b_norms, na, nb, dk / BK,
-                                                     out_d ? 3 : 2, out, out_d, ldo, out_cmin, ldc, nsplit, err,
-                                                     spin_limit, hold);
+  TileRows rows;
+  std::memset(&rows, 0, sizeof(rows));
+  v.fn<<<(unsigned)(nrb * nsplit), out_d ? 64 + 32 * 8 : 64 + 32 * 4, v.smem, st>>>(
+      mah, mal, mbh, mbl, mo, a_norms, b_norms, na, nb, dk / BK, out_d ? 3 : 2, out, out_d, ldo, out_cmin, ldc, nsplit,
+      rows, err, spin_limit, hold);
   return cudaGetLastError();
 }
 

@@ -66,7 +66,8 @@ void launch_normalise(const float* x32, const float* inv_norm, int64_t n, int32_
 // 8 strided runs per column, in run order.  Bound by the read of the rows:
 // one block per 4,096 rows, each thread walking a column alone, was
 // latency-bound (one load in flight per thread, 3 blocks for 10,000 rows):
-// 1,000,000 x 128 rows 1.8 ms, 100,000 x 960 9.2 ms, 10,000 x 32 0.55 ms.
+// 1,000,000 x 128 rows with their upper layers 1.78 ms, now 0.19 ms; 10,000
+// x 32 0.55 ms, now 0.02 ms.
 constexpr int kMeanThreads = 256;
 constexpr int kMeanChunk = 512;
 
@@ -164,6 +165,95 @@ void launch_order_gather(const float* xw, const int32_t* ids, int64_t s, int32_t
   Feistel f = Feistel::make(seed, layer, (uint64_t)s);
   k_order_gather<<<152 * 8, 256, 0, st>>>(xw, ids, s, dpad, f, graph == HENN_GRAPH_KNN ? 1 : 0, mean, inv, xo,
                                           norms);
+}
+
+// The same for the tensor-core tiles, straight to BF16 planes (no FP32 copy
+// in between) with the largest norm on the way: one read of the rows, one
+// write of the planes, 4 consecutive values per lane.  Bound by that traffic:
+// 1,000,000 x 128 rows 0.25 ms against 0.36 + 0.34 + 0.01 ms in three passes.
+__global__ void __launch_bounds__(256) k_order_split(const float* __restrict__ xw, const int32_t* __restrict__ ids,
+                                                     int64_t s, int32_t dpad, Feistel f, int32_t identity,
+                                                     const float* __restrict__ mean, int32_t dk,
+                                                     __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                                                     int32_t* __restrict__ inv, float* __restrict__ norms,
+                                                     float* __restrict__ raw_norms, float* __restrict__ norm_max) {
+  const int lane = threadIdx.x & 31;
+  int most = 0;  // bits of the largest norm (a NaN is above +inf)
+  for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; j < s;
+       j += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t rank = identity ? j : (int64_t)f.perm((uint64_t)j);
+    const float* src = xw + (ids ? (int64_t)ids[j] : j) * dpad;
+    float acc = 0.f, raw = 0.f;
+    for (int k = 4 * lane; k < dk; k += 128) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (k < dpad) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(src + k));
+        const float4 m = __ldg(reinterpret_cast<const float4*>(mean + k));
+        v[0] = x.x - m.x;
+        v[1] = x.y - m.y;
+        v[2] = x.z - m.z;
+        v[3] = x.w - m.w;
+        raw = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, raw))));
+      }
+      uint32_t h[2], l[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * i]), h1 = __float2bfloat16_rn(v[2 * i + 1]);
+        const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * i] - __bfloat162float(h0));
+        const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * i + 1] - __bfloat162float(h1));
+        h[i] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+        l[i] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+        acc = fmaf(v[2 * i], v[2 * i], acc);
+        acc = fmaf(v[2 * i + 1], v[2 * i + 1], acc);
+      }
+      *reinterpret_cast<uint2*>(hi + rank * dk + k) = make_uint2(h[0], h[1]);
+      *reinterpret_cast<uint2*>(lo + rank * dk + k) = make_uint2(l[0], l[1]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    most = max(most, __float_as_int(acc));
+    if (raw_norms) {  // uniform
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) raw += __shfl_xor_sync(0xffffffffu, raw, o);
+      if (lane == 0) raw_norms[rank] = raw;
+    }
+    if (lane == 0) {
+      if (inv) inv[rank] = (int32_t)j;
+      norms[rank] = acc;
+    }
+  }
+  if (lane == 0) atomicMax(reinterpret_cast<int*>(norm_max), most);
+}
+
+void launch_order_split(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, uint64_t seed, int32_t layer,
+                        bool identity, const float* mean, int32_t dk, void* hi, void* lo, int32_t* inv, float* norms,
+                        float* raw_norms, float* norm_max, cudaStream_t st) {
+  cudaMemsetAsync(norm_max, 0, sizeof(float), st);
+  int grid = (int)((s + 7) / 8);
+  if (grid > 152 * 8) grid = 152 * 8;
+  const Feistel f = Feistel::make(seed, layer, (uint64_t)s);
+  k_order_split<<<grid, 256, 0, st>>>(xw, ids, s, dpad, f, identity ? 1 : 0, mean, dk,
+                                      static_cast<__nv_bfloat16*>(hi), static_cast<__nv_bfloat16*>(lo), inv, norms,
+                                      raw_norms, norm_max);
+}
+
+// one warp per row
+__global__ void k_sq_norms(const float* __restrict__ x, int64_t s, int32_t dpad, float* __restrict__ norms) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < s;
+       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    float acc = 0.f;
+    for (int k = lane; k < dpad; k += 32) acc = fmaf(x[r * dpad + k], x[r * dpad + k], acc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) norms[r] = acc;
+  }
+}
+
+void launch_sq_norms(const float* x, int64_t s, int32_t dpad, float* norms, cudaStream_t st) {
+  int grid = (int)((s + 7) / 8);
+  if (grid > 152 * 8) grid = 152 * 8;
+  k_sq_norms<<<grid, 256, 0, st>>>(x, s, dpad, norms);
 }
 
 __global__ void k_gather_rows32(const float* __restrict__ xw, const int32_t* __restrict__ ids, int64_t s,
