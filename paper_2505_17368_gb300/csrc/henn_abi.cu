@@ -571,6 +571,7 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
   tr.mark("mean/order/norms", li);
   // tiles + top-KP
   uint64_t* cand = sc.get<uint64_t>((size_t)s * KP);
+  float* thr = nullptr;  // the candidate pools' bounds (tensor-core lists)
   double tile_u;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   CK(cudaEventCreate(&ev0));
@@ -580,9 +581,11 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
     int32_t* err = sc.get<int32_t>(1);
     CK(cudaMemsetAsync(err, 0, sizeof(int32_t), st));
     const int32_t splits = tile_list_splits(s, s, mode == 0);
+    thr = sc.get<float>(s);
     uint64_t* lists = splits > 1 ? sc.get<uint64_t>((size_t)splits * s * KP) : cand;
-    CK(launch_tile_lists_tc(hi, lo, norms, s, hi, lo, norms, s, dk, mode, nullptr, splits, lists, err, st));
-    if (splits > 1) launch_merge_lists(lists, s, splits, KP, cand, sc.get<float>(s), st);
+    float* lthr = splits > 1 ? sc.get<float>((size_t)splits * s) : thr;
+    CK(launch_tile_lists_tc(hi, lo, norms, s, hi, lo, norms, s, dk, mode, nullptr, splits, lists, lthr, err, st));
+    if (splits > 1) launch_merge_lists(lists, lthr, s, splits, KP, cand, thr, st);
     int32_t herr = 0;
     CK(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -609,8 +612,8 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
   flagged.rows = sc.get<int32_t>(s);
   flagged.thr = sc.get<float>(s);
   CK(cudaMemsetAsync(flagged.count, 0, sizeof(int32_t), st));
-  launch_rerank_fwd(ix->xw, Ly.ids, s, 0, dpad, ix->metric, inv, cand, KP, M, norms, nmax, tile_u, Ly.fwd, Ly.fwd_d,
-                    flagged, st);
+  launch_rerank_fwd(ix->xw, Ly.ids, s, 0, dpad, ix->metric, inv, cand, thr, s, mode == 0, KP, M, norms, nmax, tile_u,
+                    Ly.fwd, Ly.fwd_d, flagged, st);
   CKL("rerank");
   int32_t nunc = 0;
   CK(cudaMemcpyAsync(&nunc, flagged.count, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -1104,15 +1107,17 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
         uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)c * KP) : lists;
         int32_t* err = sc.get<int32_t>(2);  // the tile launch's error flag, the flagged rows' number
         CK(cudaMemsetAsync(err, 0, 2 * sizeof(int32_t), st));
+        float* thr = sc.get<float>(c);
+        float* lthr = splits > 1 ? sc.get<float>((size_t)splits * c) : thr;
         CK(launch_tile_lists_tc(hi + (size_t)s0 * dk, lo + (size_t)s0 * dk, norms + s0, c, hi, lo, norms, s1, dk, 2,
-                                drows, splits, lists, err, st));
-        if (splits > 1) launch_merge_lists(lists, c, splits, KP, cand, sc.get<float>(c), st);
+                                drows, splits, lists, lthr, err, st));
+        if (splits > 1) launch_merge_lists(lists, lthr, c, splits, KP, cand, thr, st);
         FlaggedRows flagged;
         flagged.count = err + 1;
         flagged.rows = sc.get<int32_t>(c);
         flagged.thr = sc.get<float>(c);
-        launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, KP, M, norms + s0, nmax,
-                          tc_tile_unit_error(dk), Ly.fwd, Ly.fwd_d, flagged, st);
+        launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, thr, s1, true, KP, M, norms + s0,
+                          nmax, tc_tile_unit_error(dk), Ly.fwd, Ly.fwd_d, flagged, st);
         CKL("rerank");
         int32_t host[2] = {0, 0};
         CK(cudaMemcpyAsync(host, err, sizeof(host), cudaMemcpyDeviceToHost, st));
@@ -1777,14 +1782,16 @@ void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t 
   uint16_t* qlo = sc.get<uint16_t>((size_t)nb * dk);
   float* qn = sc.get<float>(nb);
   float* qraw = sc.get<float>(nb);
-  // the pool: 32, 64 or 128 candidates, at least 16 more than k; wider than a
-  // list, it takes lists enough that one seldom holds more than 8 of the k
+  // the pool: 32, 64 or 128 candidates, at least 16 more than k; for more
+  // than 16, lists enough that one (16 of half a split's columns) seldom
+  // holds as many of the k as it is long: 6 on average
   const int32_t KP = k <= 16 ? 32 : (k <= 48 ? 64 : 128);
   const int64_t tiles = (n + kTileCols - 1) / kTileCols;
   int32_t splits = tile_list_splits(nb, n, false);
-  if (k > 16) splits = (int32_t)std::min<int64_t>(tiles, std::max(splits, (k + 7) / 8));
+  if (k > 16) splits = (int32_t)std::min<int64_t>(tiles, std::max(splits, (k + 11) / 12));
   uint64_t* lists = sc.get<uint64_t>((size_t)splits * nb * 32);
   uint64_t* cand = sc.get<uint64_t>((size_t)nb * KP);
+  float* lthr = sc.get<float>((size_t)splits * nb);
   float* thr = sc.get<float>(nb);
   void* fhi = sc.get<uint16_t>((size_t)nb * dk);
   void* flo = sc.get<uint16_t>((size_t)nb * dk);
@@ -1815,8 +1822,8 @@ void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t 
     CK(cudaMemsetAsync(over, 0, sizeof(int32_t), st));
     CK(cudaMemsetAsync(flagged.count, 0, 2 * sizeof(int32_t), st));
     launch_order_split(q, nullptr, c, dpad, 0, 0, true, mean, dk, qhi, qlo, nullptr, qn, qraw, nmax + 1, st);
-    CK(launch_tile_lists_tc(qhi, qlo, qn, c, hi, lo, xn, n, dk, 2, nullptr, splits, lists, err, st));
-    launch_merge_lists(lists, c, splits, KP, cand, thr, st);
+    CK(launch_tile_lists_tc(qhi, qlo, qn, c, hi, lo, xn, n, dk, 2, nullptr, splits, lists, lthr, err, st));
+    launch_merge_lists(lists, lthr, c, splits, KP, cand, thr, st);
     launch_rerank_knn(q, c, xp, n, dpad, metric, cand, thr, KP, k, qn, nmax, tile_u, err, oi, od, flagged, st);
     launch_gather_flagged(flagged, c, 0, false, false, n, qhi, qlo, qn, dk, fhi, flo, fnorms, lim, self, st);
     CK(launch_tile_collect_tc(fhi, flo, fnorms, c, hi, lo, xn, n, dk, lim, self, flagged.thr, flagged.count, grid, cols,

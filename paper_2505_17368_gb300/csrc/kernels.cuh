@@ -86,24 +86,28 @@ void launch_tile_topk_simt(const float* A, const float* An, int64_t na, const fl
                            uint64_t* out, const int32_t* rowsel, const int32_t* count, cudaStream_t st);
 void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t KP, int32_t splits, uint64_t* out,
                          const int32_t* count, cudaStream_t st);
-// Sorted lists of 32 keys per row and split (splits x rows x 32) -> the KP
-// (32, 64 or 128) smallest of each row, and a bound on what they leave out:
-// every column of the row that is not among them has a tile distance of at
-// least thr[row] (+inf: every column that the lists were offered is there).
-void launch_merge_lists(const uint64_t* in, int64_t rows, int32_t splits, int32_t KP, uint64_t* out, float* thr,
-                        cudaStream_t st);
+// Sorted lists of 32 keys per row and split (splits x rows x 32, with their
+// bounds thr_in) -> the KP (32, 64 or 128) smallest of each row, and a bound
+// on what they leave out: every column of the row that is not among them has
+// a tile distance of at least thr[row] (+inf: every column that the lists
+// were offered is there).
+void launch_merge_lists(const uint64_t* in, const float* thr_in, int64_t rows, int32_t splits, int32_t KP,
+                        uint64_t* out, float* thr, cudaStream_t st);
 // knn_tc.cu: the same tiles on tcgen05 tensor cores (split BF16, lists of
 // KP = 32, dpad <= 1024) from BF16 planes of rows and columns, dk =
 // roundup(dpad, 64) wide
 bool tc_tiles_supported(int32_t dpad, int32_t KP);
 // CTAs per row block, each with its own lists, for na rows against nb columns
 int32_t tile_list_splits(int64_t na, int64_t nb, bool causal);
-// modes 0 - 2; out: splits x na x 32 keys, each list sorted; lim (nullable):
-// row r takes columns 0 .. lim[r] - 1 only
+// modes 0 - 2; out: splits x na x 32 keys, each list sorted: the row's 16
+// nearest columns of two halves of the split's columns (dk > 128: its 32
+// nearest of the split); thr (splits x na):
+// every other column of the split has a tile distance of at least this (+inf:
+// there is none); lim (nullable): row r takes columns 0 .. lim[r] - 1 only
 cudaError_t launch_tile_lists_tc(const void* a_hi, const void* a_lo, const float* a_norms, int64_t na,
                                  const void* b_hi, const void* b_lo, const float* b_norms, int64_t nb, int32_t dk,
-                                 int32_t mode, const int32_t* lim, int32_t splits, uint64_t* out, int32_t* err,
-                                 cudaStream_t st);
+                                 int32_t mode, const int32_t* lim, int32_t splits, uint64_t* out, float* thr,
+                                 int32_t* err, cudaStream_t st);
 // Every column of a row whose tile distance is at or under the row's
 // threshold.  The number of rows is *count (device, at most max_rows); the
 // grid's CTAs are shared out over the 128-row blocks there are
@@ -153,11 +157,13 @@ struct FlaggedRows {
 };
 // exact FP32 rerank of layer candidates -> forward lists (layer-local ids).
 // Row r is layer position inv[r], or row0 + r with inv == nullptr (columns
-// are then positions too).
+// are then positions too).  thr: the pools' bounds (nullptr: a full pool's
+// last key).  nb: the columns; a row may take those before row0 + r (causal)
+// or all but itself.
 void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
-                       const int32_t* inv, const uint64_t* cand, int32_t KP, int32_t M, const float* norms,
-                       const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d, const FlaggedRows& flagged,
-                       cudaStream_t st);
+                       const int32_t* inv, const uint64_t* cand, const float* thr, int64_t nb, bool causal, int32_t KP,
+                       int32_t M, const float* norms, const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d,
+                       const FlaggedRows& flagged, cudaStream_t st);
 // The flagged rows' BF16 planes and norms, compact; lim[i]: causal the row's
 // own rank row0 + r, else nb; self[i]: r with skip_self, else -1.
 void launch_gather_flagged(const FlaggedRows& f, int64_t max_rows, int64_t row0, bool causal, bool skip_self,

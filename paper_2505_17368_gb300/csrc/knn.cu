@@ -304,39 +304,39 @@ __device__ __forceinline__ void merge_sorted32(uint64_t (&v)[R], uint64_t keys) 
 }
 
 template <int KP>
-__global__ void __launch_bounds__(256) k_merge_lists(const uint64_t* __restrict__ in, int64_t rows, int32_t splits,
-                                                     uint64_t* __restrict__ out, float* __restrict__ thr) {
+__global__ void __launch_bounds__(256) k_merge_lists(const uint64_t* __restrict__ in, const float* __restrict__ thr_in,
+                                                     int64_t rows, int32_t splits, uint64_t* __restrict__ out,
+                                                     float* __restrict__ thr) {
   const int lane = threadIdx.x & 31;
+  const float kInf = __int_as_float(0x7f800000);
   for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < rows;
        r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
     uint64_t v[KP / 32];
 #pragma unroll
     for (int i = 0; i < KP / 32; ++i) v[i] = kEmpty;
-    uint64_t bound = kEmpty;  // smallest last key of a full list
+    float bound = kInf;
     for (int s = 0; s < splits; ++s) {
-      const uint64_t b = __ldg(in + ((int64_t)s * rows + r) * 32 + lane);
-      const uint64_t last = shfl64(b, 31);
-      bound = last < bound ? last : bound;
-      merge_sorted32(v, b);
+      bound = fminf(bound, __ldg(thr_in + (int64_t)s * rows + r));
+      merge_sorted32(v, __ldg(in + ((int64_t)s * rows + r) * 32 + lane));
     }
     const uint64_t last = shfl64(v[KP / 32 - 1], 31);
-    bound = last < bound ? last : bound;
+    if (last != kEmpty) bound = fminf(bound, key_dist(last));
 #pragma unroll
     for (int i = 0; i < KP / 32; ++i) out[r * KP + 32 * i + lane] = v[i];
-    if (lane == 0) thr[r] = bound == kEmpty ? __int_as_float(0x7f800000) : key_dist(bound);
+    if (lane == 0) thr[r] = bound;
   }
 }
 
-void launch_merge_lists(const uint64_t* in, int64_t rows, int32_t splits, int32_t KP, uint64_t* out, float* thr,
-                        cudaStream_t st) {
+void launch_merge_lists(const uint64_t* in, const float* thr_in, int64_t rows, int32_t splits, int32_t KP,
+                        uint64_t* out, float* thr, cudaStream_t st) {
   int grid = (int)((rows + 7) / 8);
   if (grid > 152 * 16) grid = 152 * 16;
   if (KP == 32)
-    k_merge_lists<32><<<grid, 256, 0, st>>>(in, rows, splits, out, thr);
+    k_merge_lists<32><<<grid, 256, 0, st>>>(in, thr_in, rows, splits, out, thr);
   else if (KP == 64)
-    k_merge_lists<64><<<grid, 256, 0, st>>>(in, rows, splits, out, thr);
+    k_merge_lists<64><<<grid, 256, 0, st>>>(in, thr_in, rows, splits, out, thr);
   else
-    k_merge_lists<128><<<grid, 256, 0, st>>>(in, rows, splits, out, thr);
+    k_merge_lists<128><<<grid, 256, 0, st>>>(in, thr_in, rows, splits, out, thr);
 }
 
 // The certificate of a candidate pool.  The tile distance of any column
@@ -413,10 +413,12 @@ __device__ __forceinline__ void write_knn(const uint64_t (&v)[R], int64_t q, int
 
 // Forward lists from the KP tile candidates of each row (rank space), with
 // the certificate above; a row that fails it is flagged.
+constexpr int kTakeAll = 128;  // half a tile's columns
 template <int KP>
 __global__ void __launch_bounds__(256) k_rerank_fwd(const float* __restrict__ xw, const int32_t* __restrict__ ids,
                                                     int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
                                                     const int32_t* __restrict__ inv, const uint64_t* __restrict__ cand,
+                                                    const float* __restrict__ thr, int64_t nb, int32_t causal,
                                                     int32_t M, const float* __restrict__ norms,
                                                     const float* __restrict__ norm_max, double tile_u,
                                                     int32_t* __restrict__ fwd, float* __restrict__ fwd_d,
@@ -430,28 +432,37 @@ __global__ void __launch_bounds__(256) k_rerank_fwd(const float* __restrict__ xw
 #pragma unroll
     for (int i = 0; i < KP / 32; ++i) v[i] = kEmpty;
     uint64_t last = kEmpty;  // the pool's last key, if it is full
+    // a row with few columns takes them all: its two lists need not share
+    // them evenly, and a bound from half of them seldom proves anything
+    const int64_t ncols = causal ? row0 + r : nb;
+    const bool all = ncols <= kTakeAll;
+    const int pool = all ? (int)ncols : KP;
 #pragma unroll 1
-    for (int b = 0; b < KP; b += 32) {
-      const uint64_t key = __ldg(cand + r * KP + b + lane);
-      const int cnt = __popc(__ballot_sync(0xffffffffu, key != kEmpty));  // the pool is sorted: empty keys last
+    for (int b = 0; b < pool; b += 32) {
+      const int c = b + lane;
+      const uint64_t key = !all ? __ldg(cand + r * KP + c) : (c < pool && (causal || c != r) ? pack(0.f, c) : kEmpty);
       last = shfl64(key, 31);
-      if (cnt == 0) break;
+      const unsigned valid = __ballot_sync(0xffffffffu, key != kEmpty);
+      if (valid == 0) break;  // only at the pool's end: its keys are sorted, the empty ones last
       int64_t qj = 0, gq = 0;
-      if (lane < cnt) {
+      if (key != kEmpty) {
         qj = inv ? (int64_t)inv[key_index(key)] : (int64_t)key_index(key);
         gq = ids ? (int64_t)ids[qj] : qj;
       }
-      const float dv = warp_exact_dist32(xj, xw, gq, cnt, dpad, metric);
-      merge_sorted32(v, warp_sort_asc(lane < cnt ? pack(dv, (uint32_t)qj) : kEmpty));
+      const float dv = warp_exact_dist32(xj, xw, gq, 32 - __clz(valid), dpad, metric);
+      merge_sorted32(v, warp_sort_asc(key != kEmpty ? pack(dv, (uint32_t)qj) : kEmpty));
     }
-    if (last != kEmpty) {
+    // what bounds the columns left out (+inf: there are none)
+    const float bound = all ? __int_as_float(0x7f800000)
+                        : thr ? thr[r] : (last == kEmpty ? __int_as_float(0x7f800000) : key_dist(last));
+    if (!isinf(bound)) {
       const uint64_t mkey = list_key(v, M - 1);
       double dm = (mkey == kEmpty) ? 1e300 : (double)key_dist(mkey);
       // exact distances here are of raw vectors; tile distances of centred
       // ones: identical in exact arithmetic.  Angular: tile values are 2x.
       if (metric == HENN_ANGULAR) dm *= 2.0;
       float collect;
-      if (!pool_certified((double)key_dist(last), dm, norms[r], *norm_max, tile_u, dpad, &collect))
+      if (!pool_certified((double)bound, dm, norms[r], *norm_max, tile_u, dpad, &collect))
         flag_row(flagged, (int32_t)r, collect);
     }
     write_fwd(v, j, M, fwd, fwd_d);
@@ -459,23 +470,23 @@ __global__ void __launch_bounds__(256) k_rerank_fwd(const float* __restrict__ xw
 }
 
 void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
-                       const int32_t* inv, const uint64_t* cand, int32_t KP, int32_t M, const float* norms,
-                       const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d, const FlaggedRows& flagged,
-                       cudaStream_t st) {
+                       const int32_t* inv, const uint64_t* cand, const float* thr, int64_t nb, bool causal, int32_t KP,
+                       int32_t M, const float* norms, const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d,
+                       const FlaggedRows& flagged, cudaStream_t st) {
   int grid = (int)((nr + 7) / 8);
   if (grid > 152 * 32) grid = 152 * 32;
   if (grid < 1) grid = 1;
   switch (KP) {
     case 32:
-      k_rerank_fwd<32><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, M, norms, norm_max, tile_u, fwd,
+      k_rerank_fwd<32><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, M, norms, norm_max, tile_u, fwd,
                                              fwd_d, flagged);
       break;
     case 64:
-      k_rerank_fwd<64><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, M, norms, norm_max, tile_u, fwd,
+      k_rerank_fwd<64><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, M, norms, norm_max, tile_u, fwd,
                                              fwd_d, flagged);
       break;
     default:
-      k_rerank_fwd<128><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, M, norms, norm_max, tile_u,
+      k_rerank_fwd<128><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, M, norms, norm_max, tile_u,
                                               fwd, fwd_d, flagged);
       break;
   }

@@ -60,7 +60,11 @@ constexpr int STAGE = 32768;     // bytes of one stage of the streamed pipeline
 constexpr int MAX_KC_RES = 2;    // resident A: dpad <= 128, at most 2 chunks of 64 per plane
 constexpr int MAX_KC = 16;       // streamed A: dpad <= 1024
 constexpr int KP = 32;
-constexpr int S_LD = 33;
+constexpr int S_LD = 33;       // staging row, four warps: a chunk's 32 values
+constexpr int S_LD8 = 17;      // ... eight warps: half a chunk's
+constexpr int HEAP_WORDS = 2 * BM * (KP / 2 + 2);
+constexpr int STAGE_WORDS = 8 * 32 * S_LD8;
+static_assert(HEAP_WORDS >= BM * (KP + 2) && STAGE_WORDS >= 4 * 32 * S_LD, "the four-warp forms fit");
 constexpr long long kSpinLimit = 1ll << 18;  // x 20 us hint: seconds at most
 
 // Resident A (rows of at most 128 values); BN columns per tile.
@@ -69,12 +73,12 @@ struct SmemRes {
   // 1024-byte aligned operand buffers first
   uint8_t a[2 * MAX_KC_RES][A_CHUNK];  // hi chunks then lo chunks
   uint8_t b[NS][BN * BK * 2];
-  // running top-KP of each row: a max-heap of keys, 1-based (children of
-  // p at 2p and 2p + 1, so a sibling pair is one 16-byte load), root = the
-  // KP-th smallest so far; slot KP + 1 holds 0 (no child), slot 0 is unused
-  uint64_t heap[BM][KP + 2];
-  alignas(16) float ncol[4][BN];   // column norms of the current tile, one copy per epilogue warp
-  float s[4][32][S_LD];            // epilogue transposition, one slab per warp
+  // the running lists: max-heaps of LP keys, 1-based, root = the LP-th
+  // smallest so far, slot LP + 1 holds 0 (no child), slot 0 is unused; one of
+  // 32 keys per row (four epilogue warps) or two of 16 (eight)
+  uint64_t heap[HEAP_WORDS];
+  alignas(16) float ncol[4][BN];   // column norms of the current tile, one copy per sub-partition
+  float s[STAGE_WORDS];            // staging of passing values, a slab per warp
   uint64_t full[NS], empty[NS], tfull[2], tempty[2], afull;
   uint32_t tmem_base;
   int abort;
@@ -86,9 +90,9 @@ struct SmemRes {
 template <int BN>
 struct SmemStr {
   uint8_t ring[NS_STR][STAGE];
-  uint64_t heap[BM][KP + 2];
+  uint64_t heap[HEAP_WORDS];
   alignas(16) float ncol[4][BN];
-  float s[4][32][S_LD];
+  float s[STAGE_WORDS];
   uint64_t full[NS_STR], empty[NS_STR], tfull[2], tempty[2], afull;
   uint32_t tmem_base;
   int abort;
@@ -277,14 +281,16 @@ __device__ __forceinline__ void tmem_regs_after(uint32_t (&r)[32]) {
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Replaces the root of a row's max-heap (heap[1..KP], heap[KP + 1] = 0) by
-// a smaller key and sifts it down.  The heap is 4-ary: the children of node
-// p are 4p - 2 .. 4p + 1 (node 8's last child is the sentinel), read as two
-// 16-byte loads, three levels below the root where a binary heap has five.
-static_assert(KP == 32, "node 8's children end at the sentinel KP + 1");
+// Replaces the root of a row's max-heap (heap[1..LP], heap[LP + 1] = 0) by a
+// smaller key and sifts it down.  The heap is 4-ary: the children of node p
+// are 4p - 2 .. 4p + 1 (the last inner node's last child is the sentinel),
+// read as two 16-byte loads: three levels below the root for 32 keys, two for
+// 16.
+template <int LP>
 __device__ __forceinline__ void heap_replace(uint64_t* heap, uint64_t key) {
+  static_assert(LP == 32 || LP == 16, "the last inner node's children end at the sentinel LP + 1");
   int p = 1;
-  for (int c = 2; c <= KP; c = 4 * p - 2) {
+  for (int c = 2; c <= LP; c = 4 * p - 2) {
     const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(heap + c);
     const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(heap + c + 2);
     const bool ra = a.y > a.x, rb = b.y > b.x;
@@ -307,15 +313,29 @@ struct TileRows {
   const int32_t* lim;    // row r takes columns 0 .. lim[r] - 1
   const int32_t* self;   // ... except column self[r] (-1: none)
   const float* thr;      // mode 4: the rows' thresholds
+  float* thr_out;        // list modes: every column of the row (of this CTA's tiles) that is
+                         // not in its list has a tile distance of at least this (+inf: none is left out)
   const int32_t* count;  // mode 4: the number of rows, on the device
   uint32_t* cols;        // mode 4: CTA b, row r of its block: cap columns at (b * 128 + r) * cap
   int32_t* ncols;        // ... and their number (over cap: dropped)
   int32_t cap;
 };
 
-// EPI: epilogue warps, 4 (one per TMEM sub-partition; the per-row lists of
-// modes 0-2 need it) or 8 (modes 3 and 4: two per sub-partition, each taking
-// half of every tile's chunks); the launch has 64 + 32 * EPI threads
+// EPI: epilogue warps; the launch has 64 + 32 * EPI threads.  4, one per TMEM
+// sub-partition, keeping the 32 smallest keys of each row.  8, two per
+// sub-partition, each taking half of every tile's chunks: in modes 0 - 2 each
+// keeps the 16 smallest keys of the row in its half, so that a row has 32
+// candidates which hold its 16 nearest, and a bound (thr_out: the smaller of
+// the two 16th keys) below which no other column lies.  With rows of up to
+// 128 values the epilogue sets the pace of the list modes: a chunk that
+// offers any of the warp's 32 rows a column costs a few hundred cycles of one
+// warp's dependent shared-memory steps, and nearly every chunk does until a
+// list has seen some 1,000 times its length of columns.  Two warps per
+// scheduler overlap those steps, and lists half as long end the phase earlier
+// (10,000 queries x 1,000,000 x 128: 11.6 -> 6.9 ms; the 1,000,000 x 128
+// build 329 -> 300 ms).  Wider rows are bound by the MMAs, which hide four
+// warps' epilogue (100,000 x 960 tiles: 18.5 ms either way), and one list of
+// 32 leaves fewer rows open.
 template <bool kStream, int BN, int EPI>
 __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     k_tile_topk_tc(const __grid_constant__ CUtensorMap ta_hi, const __grid_constant__ CUtensorMap ta_lo,
@@ -374,11 +394,12 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   // the rows' heaps; in mode 4 the rows' column counts instead
-  if (EPI == 4) {
-    for (int i = threadIdx.x; i < BM * (KP + 2); i += blockDim.x)
-      (&sm.heap[0][0])[i] = (i % (KP + 2) == KP + 1) ? 0ull : kEmpty;
+  constexpr int LP = EPI == 8 ? KP / 2 : KP;  // keys per list
+  if (mode <= 2) {
+    for (int i = threadIdx.x; i < (EPI / 4) * BM * (LP + 2); i += blockDim.x)
+      sm.heap[i] = (i % (LP + 2) == LP + 1) ? 0ull : kEmpty;
   } else if (threadIdx.x < BM) {
-    reinterpret_cast<int*>(&sm.heap[0][0])[threadIdx.x] = 0;
+    reinterpret_cast<int*>(sm.heap)[threadIdx.x] = 0;
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(tc::smem_u32(&sm.tmem_base)));
@@ -529,7 +550,14 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     const int ew = warp - 2;
     const int sub = warp & 3;  // TMEM sub-partition of this warp
     constexpr int halves = EPI / 4;
-    const int qlo = (ew >> 2) * (BN / 32) / halves, qhi = qlo + (BN / 32) / halves;  // this warp's chunks
+    // this warp's chunks, two at a time: half of the tile, or in the list
+    // modes every other pair (so that a row with few columns has them in both
+    // of its lists)
+    const bool pairs = EPI == 8 && mode <= 2;
+    const int qlo = pairs ? 2 * (ew >> 2) : (ew >> 2) * (BN / 32) / halves;
+    const int qhi = pairs ? BN / 32 : qlo + (BN / 32) / halves;
+    const int qstep = pairs ? 4 : 2;
+    auto mine = [&](const int q) { return pairs ? ((q >> 1) & 1) == (ew >> 2) : q >= qlo && q < qhi; };
     const int ews = ew & 3;  // per-sub-partition staging, shared by its warps on disjoint chunks
     const int row_l = 32 * sub + lane;
     const int64_t grow = r0 + row_l;
@@ -546,17 +574,18 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       const float thr = grow < s ? rows.thr[grow] : 0.f;
       thr_adj = thr - nrow + 1e-6f * (fabsf(thr) + fabsf(nrow));
     }
-    uint64_t* heap = sm.heap[row_l];
+    uint64_t* heap = sm.heap + ((ew >> 2) * BM + row_l) * (LP + 2);
     uint64_t root = kEmpty;
     // mode 3 keeps no lists: the heap space holds each warp's 4 KB store
     // box (1024-byte aligned)
-    uint32_t* m3_stage = reinterpret_cast<uint32_t*>(&sm.heap[0][0]) + ew * 1024;
+    uint32_t* m3_stage = reinterpret_cast<uint32_t*>(sm.heap) + ew * 1024;
+    float* m3_min = sm.s + (ews * 32 + lane) * S_LD;  // mode 3: the row's chunk minima
     bool ok = true;
     float pn[BN / 32];  // column norms of the next tile, one per lane and chunk
 #pragma unroll
     for (int q = 0; q < BN / 32; ++q) {
       const int64_t c = (int64_t)t0 * BN + q * 32 + lane;
-      pn[q] = c < sc && q >= qlo && q < qhi ? __ldg(norms_c + c) : 0.f;
+      pn[q] = c < sc && mine(q) ? __ldg(norms_c + c) : 0.f;
     }
     for (int lt = 0; lt < nt; ++lt) {
       const int t = t0 + lt * tstep;
@@ -572,14 +601,14 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       float* ncs = sm.ncol[ews];
 #pragma unroll
       for (int q = 0; q < BN / 32; ++q)
-        if (q >= qlo && q < qhi) ncs[q * 32 + lane] = pn[q];
+        if (mine(q)) ncs[q * 32 + lane] = pn[q];
 #pragma unroll
       for (int q = 0; q < BN / 32; ++q) {
         const int64_t c = (int64_t)(t + tstep) * BN + q * 32 + lane;
-        pn[q] = c < sc && q >= qlo && q < qhi ? __ldg(norms_c + c) : 0.f;
+        pn[q] = c < sc && mine(q) ? __ldg(norms_c + c) : 0.f;
       }
       if (mode == 3 && out_cmin)
-        for (int q = qlo; q < qhi; ++q) sm.s[ews][lane][q] = kInf;
+        for (int q = qlo; q < qhi; ++q) m3_min[q] = kInf;
       __syncwarp();
       const uint32_t tacc = tmem + ((uint32_t)(32 * sub) << 16) + (uint32_t)(as * BN);
       // n_col - 2<a,b> for the 32 columns of chunk q, in place, and their
@@ -612,33 +641,53 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
           for (int j = 0; j < 32; ++j) keep |= (v[j] <= thr_adj) ? (1u << j) : 0u;
           keep &= vmask;
         }
-        if (keep) {
-          // this lane's row: stage the passing values, then offer them to
-          // the row's heap one by one
-          float* srow = sm.s[ews][lane];
+        auto offer = [&](const float x, const int j) {
+          const float dv = fmaxf(nrow + x, 0.f);
+          const uint64_t key = pack(dv, (uint32_t)(c0 + j));
+          if (!isinf(dv) && key < root) {
+            tc::heap_replace<LP>(heap, key);
+            root = heap[1];
+            const float nthr = root == kEmpty ? kInf : key_dist(root);
+            // slightly permissive: rounding of the folded threshold must
+            // not drop a column the certified pool counts on
+            thr_adj = nthr - nrow + 1e-6f * (fabsf(nthr) + fabsf(nrow));
+          }
+        };
+        // this lane's row: stage the passing values, then offer them to the
+        // row's heap one by one
+        if constexpr (EPI == 4) {
+          if (keep) {
+            float* srow = sm.s + (ews * 32 + lane) * S_LD;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) srow[j] = v[j];
-          do {
-            const int j = __ffs(keep) - 1;
-            keep &= keep - 1;
-            const float dv = fmaxf(nrow + srow[j], 0.f);
-            const uint64_t key = pack(dv, (uint32_t)(c0 + j));
-            if (!isinf(dv) && key < root) {
-              tc::heap_replace(heap, key);
-              root = heap[1];
-              const float nthr = root == kEmpty ? kInf : key_dist(root);
-              // slightly permissive: rounding of the folded threshold must
-              // not drop a column the certified pool counts on
-              thr_adj = nthr - nrow + 1e-6f * (fabsf(nthr) + fabsf(nrow));
+            for (int j = 0; j < 32; ++j) srow[j] = v[j];
+            do {
+              const int j = __ffs(keep) - 1;
+              keep &= keep - 1;
+              offer(srow[j], j);
+            } while (keep);
+          }
+        } else {
+          float* srow = sm.s + (ew * 32 + lane) * S_LD8;
+#pragma unroll
+          for (int hh = 0; hh < 2; ++hh) {
+            unsigned kk = (keep >> (16 * hh)) & 0xFFFFu;
+            if (kk) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) srow[j] = v[16 * hh + j];
+              do {
+                const int j = __ffs(kk) - 1;
+                kk &= kk - 1;
+                offer(srow[j], 16 * hh + j);
+              } while (kk);
             }
-          } while (keep);
+          }
         }
         __syncwarp();
       };
       if (EPI == 8 && mode == 4) {
         // the columns at or under the row's threshold, appended to its
         // buffer: few once the threshold is a row's known M-th distance
-        int* cnt = reinterpret_cast<int*>(&sm.heap[0][0]);
+        int* cnt = reinterpret_cast<int*>(sm.heap);
         uint32_t* buf = rows.cols + ((int64_t)blockIdx.x * BM + row_l) * rows.cap;
 #pragma unroll 1
         for (int q = qlo; q < qhi; q += 2) {
@@ -676,12 +725,12 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
           __syncwarp();
         }
       }
-      if (EPI == 4) {
+      if (mode <= 2) {
         // two chunks at a time: both TMEM loads behind one wait, the two
         // chunks' distance terms interleaved, then their inserts in chunk
         // order (the same lists as one chunk at a time)
 #pragma unroll 1
-        for (int q = 0; q < BN / 32; q += 2) {
+        for (int q = qlo; q < qhi; q += qstep) {
           const int64_t ca = (int64_t)t * BN + q * 32, cb = ca + 32;
           uint32_t ra[32], rb[32];
           tc::tmem_ld32_issue(tacc + (uint32_t)q * 32, ra);
@@ -769,8 +818,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
         if (out_cmin) {
           // the lower ends of the minima's key buckets: the minimum of a
           // chunk's key lower ends
-          sm.s[ews][lane][q] = key16_floor(cm[0]);
-          sm.s[ews][lane][q + 1] = key16_floor(cm[1]);
+          m3_min[q] = key16_floor(cm[0]);
+          m3_min[q + 1] = key16_floor(cm[1]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
@@ -780,7 +829,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       if (mode == 3 && out_cmin && grow < s) {
         // this row's chunk minima of this warp's chunks, as 8-byte stores
         float2* dst = reinterpret_cast<float2*>(out_cmin + grow * ldc + (int64_t)t * (BN / 32) + qlo);
-        const float* src = sm.s[ews][lane] + qlo;
+        const float* src = m3_min + qlo;
         for (int j = 0; j < (qhi - qlo) / 2; ++j) dst[j] = make_float2(src[2 * j], src[2 * j + 1]);
       }
       tc::fence_before();
@@ -792,19 +841,36 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       sm.abort = 1;
     }
     if (mode == 3 && lane == 0) tc::bulk_wait_all();
-    // this warp's 32 rows, each heap sorted ascending across the warp
-    __syncwarp();
-    for (int i = 0; i < 32 && EPI == 4; ++i) {
-      const int64_t gr = r0 + 32 * sub + i;
-      const uint64_t x = warp_sort_asc(sm.heap[32 * sub + i][1 + lane]);
-      if (gr < s) out[((int64_t)sp * s + gr) * KP + lane] = x;
+    if (mode <= 2) {
+      // the rows' lists, sorted ascending across the warp: 32 rows a warp,
+      // or 16 with the two halves of a row together
+      if constexpr (EPI == 8) {
+        asm volatile("bar.sync 1, 256;" ::: "memory");  // the other half's warp is done too
+      } else {
+        __syncwarp();
+      }
+      for (int i = 0; i < BM / EPI; ++i) {
+        const int rl = 32 * sub + (ew >> 2) * (BM / EPI) + i;
+        const int64_t gr = r0 + rl;
+        const uint64_t* h = EPI == 4 ? sm.heap + rl * (LP + 2) + 1 + lane
+                                     : sm.heap + ((lane >> 4) * BM + rl) * (LP + 2) + 1 + (lane & 15);
+        const uint64_t x = warp_sort_asc(*h);
+        if (gr < s) {
+          out[((int64_t)sp * s + gr) * KP + lane] = x;
+          if (rows.thr_out && lane == 0) {
+            uint64_t m = sm.heap[rl * (LP + 2) + 1];
+            if (EPI == 8) m = min(m, sm.heap[(BM + rl) * (LP + 2) + 1]);
+            rows.thr_out[(int64_t)sp * s + gr] = m == kEmpty ? kInf : key_dist(m);
+          }
+        }
+      }
     }
   }
   tc::fence_before();
   __syncthreads();
   // mode 4: how many columns each row has (over rows.cap: the rest were dropped)
   if (EPI == 8 && mode == 4 && threadIdx.x < BM)
-    rows.ncols[(int64_t)blockIdx.x * BM + threadIdx.x] = reinterpret_cast<const int*>(&sm.heap[0][0])[threadIdx.x];
+    rows.ncols[(int64_t)blockIdx.x * BM + threadIdx.x] = reinterpret_cast<const int*>(sm.heap)[threadIdx.x];
   if (sm.abort) {
     // let any bulk copy still in flight land before the CTA leaves
     __nanosleep(100000);
@@ -892,7 +958,7 @@ bool tc_tiles_supported(int32_t dpad, int32_t KPv) { return dpad <= BK * MAX_KC 
 
 static_assert(sizeof(SmemRes<256>) + 1024 <= 227 * 1024, "shared memory of one CTA");
 static_assert(sizeof(SmemStr<256>) + 1024 <= 227 * 1024, "shared memory of one CTA");
-static_assert(sizeof(((SmemRes<128>*)nullptr)->heap) >= 4 * 8192, "mode 3 store boxes fit in the heap space");
+static_assert(HEAP_WORDS * 8 >= 8 * 4096, "mode 3 store boxes fit in the heap space");
 static_assert(offsetof(SmemRes<128>, heap) % 1024 == 0 && offsetof(SmemRes<256>, heap) % 1024 == 0,
               "store boxes 1024-byte aligned");
 static_assert(offsetof(SmemStr<128>, heap) % 1024 == 0 && offsetof(SmemStr<256>, heap) % 1024 == 0,
@@ -946,9 +1012,9 @@ static int sm_count(int dev) {
 // CTAs per row block for the list modes: the split with the fewest
 // tile-times over all waves of one CTA per SM, or for the causal mode (whose
 // row blocks are unequal, the longest first) the longer of the even share and
-// the longest CTA.  A CTA's fixed work -- set-up, the first fill of its lists
-// -- counts as kListFill tiles.
-constexpr int kListFill = 6;
+// the longest CTA.  A CTA's first tiles, while its lists fill, take about
+// half as long again (kFillTiles of them).
+constexpr int kFillTiles = 250;
 
 int32_t tile_list_splits(int64_t na, int64_t nb, bool causal) {
   int dev = 0;
@@ -956,13 +1022,14 @@ int32_t tile_list_splits(int64_t na, int64_t nb, bool causal) {
   const int64_t sms = sm_count(dev);
   const int64_t nrb = (na + BM - 1) / BM;
   const int64_t nt = (nb + BN_MAX - 1) / BN_MAX;
+  auto cta = [](double tiles) { return tiles + 0.5 * std::min(tiles, (double)kFillTiles) + 4.0; };
   double best = 1e300;
   int32_t pick = 1;
   for (int64_t k = 1; k <= nt && k <= (causal ? 16 : sms); ++k) {
-    const double longest = (double)((nt + k - 1) / k + kListFill);
+    const double longest = cta((double)((nt + k - 1) / k));
     double cost;
     if (causal)
-      cost = std::max((double)nrb * (0.5 * (double)nt + (double)(k * kListFill)) / (double)sms, longest);
+      cost = std::max((double)(nrb * k) * cta(0.5 * (double)nt / (double)k) / (double)sms, longest);
     else
       cost = (double)((nrb * k + sms - 1) / sms) * longest;
     if (cost < best * 0.99) {  // more lists only for a gain
@@ -975,8 +1042,8 @@ int32_t tile_list_splits(int64_t na, int64_t nb, bool causal) {
 
 cudaError_t launch_tile_lists_tc(const void* a_hi, const void* a_lo, const float* a_norms, int64_t na,
                                  const void* b_hi, const void* b_lo, const float* b_norms, int64_t nb, int32_t dk,
-                                 int32_t mode, const int32_t* lim, int32_t splits, uint64_t* out, int32_t* err,
-                                 cudaStream_t st) {
+                                 int32_t mode, const int32_t* lim, int32_t splits, uint64_t* out, float* thr,
+                                 int32_t* err, cudaStream_t st) {
   if (dk % BK != 0 || dk / BK > MAX_KC || na < 1 || nb < 1 || splits < 1 || mode < 0 || mode > 2)
     return cudaErrorInvalidValue;
   CUtensorMap mah, mal, mbh, mbl;
@@ -984,7 +1051,8 @@ cudaError_t launch_tile_lists_tc(const void* a_hi, const void* a_lo, const float
       !make_map(&mbl, b_lo, nb, dk, BN_MAX))
     return cudaErrorInvalidValue;
   TileVariant v;
-  cudaError_t e = tile_variant(dk / BK, BN_MAX, false, &v);
+  const bool eight = dk / BK <= MAX_KC_RES;
+  cudaError_t e = tile_variant(dk / BK, BN_MAX, eight, &v);
   if (e != cudaSuccess) return e;
   const int64_t nrb = (na + BM - 1) / BM;
   CUtensorMap none;  // no matrix output
@@ -992,10 +1060,11 @@ cudaError_t launch_tile_lists_tc(const void* a_hi, const void* a_lo, const float
   TileRows rows;
   std::memset(&rows, 0, sizeof(rows));
   rows.lim = lim;
+  rows.thr_out = thr;
   long long spin_limit;
   int32_t hold;
   wait_policy(&spin_limit, &hold);
-  v.fn<<<(unsigned)(nrb * splits), 192, v.smem, st>>>(mah, mal, mbh, mbl, none, a_norms, b_norms, na, nb, dk / BK, mode,
+  v.fn<<<(unsigned)(nrb * splits), 64 + 32 * (eight ? 8 : 4), v.smem, st>>>(mah, mal, mbh, mbl, none, a_norms, b_norms, na, nb, dk / BK, mode,
                                                       out, nullptr, 0, nullptr, 0, splits, rows, err, spin_limit,
                                                       hold);
   return cudaGetLastError();
