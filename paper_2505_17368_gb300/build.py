@@ -32,6 +32,7 @@ def _headers() -> list[str]:
     inc = os.path.join(os.path.dirname(HERE), "include")
     hs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     hs += [os.path.join(inc, f) for f in os.listdir(inc) if f.endswith(".h")]
+    hs.append(os.path.join(CSRC, "search.cu"))  # included by search_bf16.cu and search_fp8.cu
     return hs
 
 

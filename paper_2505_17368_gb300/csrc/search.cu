@@ -1,5 +1,8 @@
 // search.cu -- batched HENN query (Alg. 4 + layer-0 beam), one persistent
-// launch per batch, one warp per query.
+// launch per batch, one warp per query.  The kernels are templates over the
+// storage type: this file instantiates them for FP32 and is included by
+// search_bf16.cu and search_fp8.cu (HENN_SEARCH_ROWS defined) for the others,
+// so that the three compile side by side.
 //
 // Per query:
 //   S1  entry = node bounded(derive(derive(seed, ENTR), key), |L_L|) of the
@@ -30,6 +33,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "common.cuh"
@@ -38,15 +42,23 @@
 
 namespace henn {
 
-// Occupancy / memory-parallelism trade-off of the search kernels: blocks
-// of 4 warps guaranteed per SM (caps registers per thread at
-// 65536 / (128 * min_blocks)) and 16-byte chunks in flight per lane.
-#ifndef HENN_SEARCH_MIN_BLOCKS
-#define HENN_SEARCH_MIN_BLOCKS 6
-#endif
-#ifndef HENN_SEARCH_CHUNKS_IN_FLIGHT
-#define HENN_SEARCH_CHUNKS_IN_FLIGHT 4
-#endif
+// Occupancy / memory-parallelism trade-off of the search kernels: IF = the
+// 16-byte chunks of neighbour rows in flight per lane.  kFull (24 warps per
+// SM by its 80 registers) is for launches that fill the SMs; a launch that
+// cannot -- few queries, or wide beams whose shared memory leaves room for
+// few warps -- has registers to spare and waits for its rows in fewer round
+// trips: kHalf at up to 16 warps per SM (128 registers), kFew at up to 8
+// (255).  The arithmetic and its order are the same (rows_dist), so results
+// do not depend on the choice; search_in_flight has the rule.  Against kFull:
+// 2,000 queries over 100,000 x 960 BF16 rows 1.77 -> 1.35 ms (kHalf), 1,000
+// over 50,000 x 100 FP8 at ef 200 912 -> 735 us, one over 50,000 x 32 FP32
+// 172 -> 149 us (kFew), 64 over 1,000,000 x 128 BF16 (8 new rows an
+// expansion, one round trip either way) 421 -> 423 us.
+constexpr int kFull = 4, kHalf = 16, kFew = 32;
+template <int IF>
+struct SearchOcc {
+  static constexpr int kMinBlocks = IF == kFull ? 6 : (IF == kHalf ? 4 : 2);
+};
 // The beam's shared-memory pointers re-derived from the dynamic shared
 // memory base (1) or used as passed (0).
 #ifndef HENN_SEARCH_SMEM32
@@ -211,12 +223,12 @@ __device__ __forceinline__ uint4 load_row_chunk(const uint4* p) {
 // passes are all issued before any arithmetic, so one neighbour list costs
 // one or two memory round trips instead of one per pass.  Returns, in lane
 // j < count, the squared distance of row j.
-template <typename VT, int G, int CPL>
+template <typename VT, int G, int CPL, int IF>
 __device__ __forceinline__ float rows_dist(const VT* __restrict__ vec, const float* __restrict__ scale, int64_t stride_bytes,
                                            int32_t my_id, int count, const float* __restrict__ qs, int nchunk) {
   const int lane = lane_id();
   constexpr int RP = 32 / G;
-  constexpr int PB0 = HENN_SEARCH_CHUNKS_IN_FLIGHT / CPL;  // passes per batch
+  constexpr int PB0 = IF / CPL;  // passes per batch
   constexpr int PB = PB0 < 1 ? 1 : (PB0 > 32 / RP ? 32 / RP : PB0);
   const int g = lane % G, slot_in_pass = lane / G;
   float mine = 0.f;
@@ -281,7 +293,7 @@ __device__ __forceinline__ float team_rows(const Team& tm, const VT* __restrict_
   team_sync(tm);
   const int mine = (count + tm.size - 1) / tm.size;
   const int32_t id = lane < mine ? job->ids[lane * tm.size] : 0;
-  const float d = rows_dist<VT, G, CPL>(vec, scale, stride_bytes, id, mine, qs, nchunk);
+  const float d = rows_dist<VT, G, CPL, kFull>(vec, scale, stride_bytes, id, mine, qs, nchunk);
   if (lane < mine) job->dist[lane * tm.size] = d;
   team_sync(tm);
   return lane < count ? job->dist[lane] : 0.f;
@@ -299,8 +311,8 @@ __device__ __noinline__ void team_helper(const Team& tm, int rank, int64_t strid
     const int count = job->count;
     const int mine = (count - rank + tm.size - 1) / tm.size;  // rows rank, rank + T, ...
     const int32_t id = lane < mine ? job->ids[rank + lane * tm.size] : 0;
-    const float d = rows_dist<VT, G, CPL>(static_cast<const VT*>(job->vec), job->scale, stride_bytes, id, mine, qs,
-                                          nchunk);
+    const float d = rows_dist<VT, G, CPL, kFull>(static_cast<const VT*>(job->vec), job->scale, stride_bytes, id, mine,
+                                                 qs, nchunk);
     if (lane < mine) job->dist[rank + lane * tm.size] = d;
     team_sync(tm);
   }
@@ -349,7 +361,7 @@ __device__ __forceinline__ int lower_bound_w(const uint64_t* W, int nw, uint64_t
 // copies of the layer above's candidates) and `entry` is ignored.
 // The layer comes as its arrays and size (not a reference to a descriptor,
 // which would put a memory load before every adjacency-row address).
-template <typename VT, int G, int CPL, typename TM>
+template <typename VT, int G, int CPL, int IF, typename TM>
 __device__ __noinline__ int beam(const int32_t* __restrict__ adj, const void* vec_, const float* __restrict__ scale,
                                  int64_t size, int64_t stride, int nchunk, int32_t entry, int ef, uint64_t* W,
                                  int32_t* table, int HB, uint64_t* stage, const float* qs, int& evals_out,
@@ -377,7 +389,7 @@ __device__ __noinline__ int beam(const int32_t* __restrict__ adj, const void* ve
     for (int j = lane; j < nw; j += 32) mark((int32_t)key_index(W[j] & kKeyMask));
   } else {
     if (lane == 0) mark(entry);
-    float d0 = rows_dist<VT, G, CPL>(vec, scale, stride, entry, 1, qs, nchunk);
+    float d0 = rows_dist<VT, G, CPL, IF>(vec, scale, stride, entry, 1, qs, nchunk);
     d0 = __shfl_sync(0xffffffffu, d0, 0);
     ++evals;
     if (lane == 0) W[0] = pack(d0, (uint32_t)entry);
@@ -428,7 +440,7 @@ __device__ __noinline__ int beam(const int32_t* __restrict__ adj, const void* ve
     if constexpr (TEAM)
       dn = team_rows<VT, G, CPL>(tm, vec, scale, stride, packed_id, cnt, qs, nchunk);
     else
-      dn = rows_dist<VT, G, CPL>(vec, scale, stride, packed_id, cnt, qs, nchunk);
+      dn = rows_dist<VT, G, CPL, IF>(vec, scale, stride, packed_id, cnt, qs, nchunk);
     evals += cnt;
     const uint64_t worst = nw < ef ? kEmpty : (W[nw - 1] & kKeyMask);
     uint64_t kk = lane < cnt ? pack(dn, (uint32_t)packed_id) : kEmpty;
@@ -523,7 +535,7 @@ __device__ __noinline__ int beam(const int32_t* __restrict__ adj, const void* ve
 // point belongs to the first `need` keys.  Otherwise, and for method 2,
 // every point of the layer is evaluated into a running top 32 (warp
 // bitonic merge of each sorted batch of 32).
-template <typename VT, int G, int CPL>
+template <typename VT, int G, int CPL, int IF>
 __device__ __noinline__ uint64_t exact_top32(const SearchArgs& a, const void* vec_, const float* __restrict__ scale,
                                              int64_t size, int64_t stride, int nchunk, const float* qs,
                                              const uint64_t* pre_row, float pre_qn, int need, int& evals) {
@@ -535,7 +547,7 @@ __device__ __noinline__ uint64_t exact_top32(const SearchArgs& a, const void* ve
     const uint64_t tk = pre_row[lane];
     const int cnt = __popc(__ballot_sync(0xffffffffu, tk != kEmpty));
     const int32_t id = tk != kEmpty ? (int32_t)key_index(tk) : 0;
-    const float dn = rows_dist<VT, G, CPL>(vec, scale, stride, id, cnt, qs, nchunk);
+    const float dn = rows_dist<VT, G, CPL, IF>(vec, scale, stride, id, cnt, qs, nchunk);
     evals += cnt;
     const uint64_t mine = warp_sort_asc(lane < cnt ? pack(dn, (uint32_t)id) : kEmpty);
     bool ok = cnt == s;  // the candidates are the whole layer
@@ -559,7 +571,7 @@ __device__ __noinline__ uint64_t exact_top32(const SearchArgs& a, const void* ve
   uint64_t mine = kEmpty;
   for (int c0 = 0; c0 < s; c0 += 32) {
     const int cnt = min(32, s - c0);
-    const float dn = rows_dist<VT, G, CPL>(vec, scale, stride, c0 + lane, cnt, qs, nchunk);
+    const float dn = rows_dist<VT, G, CPL, IF>(vec, scale, stride, c0 + lane, cnt, qs, nchunk);
     uint64_t kk = lane < cnt ? pack(dn, (uint32_t)(c0 + lane)) : kEmpty;
     if (!__any_sync(0xffffffffu, kk < shfl64(mine, 31))) continue;
     // the running list and the reversed sorted batch: their element-wise
@@ -590,7 +602,7 @@ struct RowShape {
 
 // S4 + output: exact FP32 rerank of the best rerank_mult * k entries
 // (BF16 / FP8 storage), then the first k of W in (distance, index) order.
-template <int G32, int CPL32>
+template <int G32, int CPL32, int IF>
 __device__ __noinline__ void finish_query(const SearchArgs& a, uint64_t* W, int nw, int k, const float* qs,
                                           int64_t* out_ids, float* out_d) {
   W = as_shared(W);
@@ -620,7 +632,7 @@ __device__ __noinline__ void finish_query(const SearchArgs& a, uint64_t* W, int 
       int i = b + lane;
       int32_t id = i < R ? (int32_t)key_index(W[i] & kKeyMask) : 0;
       int cntb = min(32, R - b);
-      float dx = rows_dist<float, G32, CPL32>(a.x32, nullptr, (int64_t)dpad * 4, id, cntb, qs, dpad / 4);
+      float dx = rows_dist<float, G32, CPL32, IF>(a.x32, nullptr, (int64_t)dpad * 4, id, cntb, qs, dpad / 4);
       __syncwarp();
       if (i < R) W[i] = pack(dx, (uint32_t)id);
       __syncwarp();
@@ -660,7 +672,7 @@ __device__ __noinline__ void finish_query(const SearchArgs& a, uint64_t* W, int 
 // One query, one warp: S1-S4 for the query row `qg` (d floats), writing
 // out_stride results to out_ids / out_d and 4 counters to stats (optional).
 // `my` is this warp's shared-memory slice.
-template <typename VT, int DMAX, typename TM>
+template <typename VT, int DMAX, int IF, typename TM>
 __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my, const float* __restrict__ qg, int k,
                                           int ef, uint64_t key, int64_t* out_ids, float* out_d, int32_t* stats,
                                           const uint64_t* pre_row, float pre_qn, const TM tm) {
@@ -712,7 +724,7 @@ __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my
     // the host keeps width <= 32 when the candidates seed the next layer
     const bool seeds = a.descend_all && width > 1;
     const int nw = seeds ? min(min(width, 32), (int)Ly.size) : 1;
-    const uint64_t mine = exact_top32<VT, G, CPL>(a, Ly.vec, Ly.scale, Ly.size, stride, nchunk, qs,
+    const uint64_t mine = exact_top32<VT, G, CPL, IF>(a, Ly.vec, Ly.scale, Ly.size, stride, nchunk, qs,
                                                   a.exact_method == 1 ? pre_row : nullptr, pre_qn, nw, evals);
     if (lane < nw) W[lane] = seeds ? ((mine & 0xFFFFFFFF00000000ull) | (uint32_t)Ly.down[key_index(mine)]) : mine;
     cur = Ly.down[key_index(shfl64(mine, 0))];
@@ -732,7 +744,7 @@ __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my
       const VT* vec = reinterpret_cast<const VT*>(Ly.vec);
       for (int c0 = 0; c0 < s; c0 += 32) {
         const int cnt = min(32, s - c0);
-        const float dn = rows_dist<VT, G, CPL>(vec, Ly.scale, stride, c0 + lane, cnt, qs, nchunk);
+        const float dn = rows_dist<VT, G, CPL, IF>(vec, Ly.scale, stride, c0 + lane, cnt, qs, nchunk);
         if (lane < cnt) keys[c0 + lane] = pack(dn, (uint32_t)(c0 + lane));
       }
       evals += s;
@@ -768,7 +780,7 @@ __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my
       __syncwarp();
     } else if (width > 1) {
       int ex = 0;
-      int nw = beam<VT, G, CPL, TM>(Ly.adj, Ly.vec, Ly.scale, Ly.size, stride, nchunk, cur, min(width, EFCAP), W,
+      int nw = beam<VT, G, CPL, IF, TM>(Ly.adj, Ly.vec, Ly.scale, Ly.size, stride, nchunk, cur, min(width, EFCAP), W,
                                     table, HB, stage, qs, evals, ex, evictions, nseed, tm);
       moves += ex;
       cur = (int32_t)key_index(W[0] & kKeyMask);
@@ -784,7 +796,7 @@ __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my
       __syncwarp();
     } else {
       const VT* vec = reinterpret_cast<const VT*>(Ly.vec);
-      float dc = rows_dist<VT, G, CPL>(vec, Ly.scale, stride, cur, 1, qs, nchunk);
+      float dc = rows_dist<VT, G, CPL, IF>(vec, Ly.scale, stride, cur, 1, qs, nchunk);
       dc = __shfl_sync(0xffffffffu, dc, 0);
       ++evals;
       for (;;) {
@@ -792,7 +804,7 @@ __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my
         unsigned valid = __ballot_sync(0xffffffffu, nb >= 0);
         int cnt = __popc(valid);
         // neighbours are packed at the front of each row (-1 padding after)
-        float dn = rows_dist<VT, G, CPL>(vec, Ly.scale, stride, nb, cnt, qs, nchunk);
+        float dn = rows_dist<VT, G, CPL, IF>(vec, Ly.scale, stride, nb, cnt, qs, nchunk);
         evals += cnt;
         uint64_t kk = lane < cnt ? pack(dn, (uint32_t)nb) : kEmpty;
         uint64_t best = warp_min64(kk);
@@ -807,11 +819,11 @@ __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my
 
   // S3: layer-0 beam
   const SearchLayer B = a.layers[0];
-  int nw = beam<VT, G, CPL, TM>(B.adj, B.vec, B.scale, B.size, stride, nchunk, cur, ef, W, table, HB, stage, qs,
+  int nw = beam<VT, G, CPL, IF, TM>(B.adj, B.vec, B.scale, B.size, stride, nchunk, cur, ef, W, table, HB, stage, qs,
                                 evals, expansions, evictions, nseed, tm);
 
   // S4 + output
-  finish_query<G32, CPL32>(a, W, nw, k, qs, out_ids, out_d);
+  finish_query<G32, CPL32, IF>(a, W, nw, k, qs, out_ids, out_d);
   if (stats && lane == 0) {
     stats[0] = evals;
     stats[1] = expansions;
@@ -828,8 +840,8 @@ __device__ __forceinline__ void run_query(const SearchArgs& a, unsigned char* my
 }
 
 // TM = Solo: one warp per query.  TM = Team: teams of a.team warps.
-template <typename VT, int DMAX, typename TM>
-__global__ void __launch_bounds__(128, HENN_SEARCH_MIN_BLOCKS) k_search(const __grid_constant__ SearchArgs a) {
+template <typename VT, int DMAX, int IF, typename TM>
+__global__ void __launch_bounds__(128, SearchOcc<IF>::kMinBlocks) k_search(const __grid_constant__ SearchArgs a) {
   constexpr int G = RowShape<VT, DMAX>::G, CPL = RowShape<VT, DMAX>::CPL;
   constexpr bool TEAM = std::is_same<TM, Team>::value;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -871,7 +883,7 @@ __global__ void __launch_bounds__(128, HENN_SEARCH_MIN_BLOCKS) k_search(const __
     const int k = a.kq ? a.kq[qi] : a.k_uniform;
     const int ef = a.efq ? a.efq[qi] : a.ef_uniform;
     const uint64_t key = a.keys ? a.keys[qi] : (uint64_t)qi;
-    run_query<VT, DMAX>(a, my, a.Q + qi * a.d, k, ef, key, a.out_ids + qi * a.out_stride,
+    run_query<VT, DMAX, IF>(a, my, a.Q + qi * a.d, k, ef, key, a.out_ids + qi * a.out_stride,
                         a.out_d + qi * a.out_stride, a.stats ? a.stats + qi * 4 : nullptr,
                         a.pre_keys ? a.pre_keys + qi * 32 : nullptr, a.pre_qnorm ? a.pre_qnorm[qi] : 0.f, tm);
   }
@@ -901,7 +913,7 @@ __device__ __forceinline__ long long ld_acquire_gpu(const long long* p) {
 // items are published and it has ended.  A finished query bumps its
 // request's counter in mapped host memory after a system-scope fence.
 template <typename VT, int DMAX>
-__global__ void __launch_bounds__(128, HENN_SEARCH_MIN_BLOCKS) k_serve(const __grid_constant__ ServeArgs s) {
+__global__ void __launch_bounds__(128, SearchOcc<kFull>::kMinBlocks) k_serve(const __grid_constant__ ServeArgs s) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = lane_id();
   unsigned char* my = smem + (size_t)(threadIdx.x >> 5) * s.base.warp_smem;
@@ -941,7 +953,7 @@ __global__ void __launch_bounds__(128, HENN_SEARCH_MIN_BLOCKS) k_serve(const __g
     const int32_t k = __ldcg(&s.desc[slot].k);
     const int32_t ef = __ldcg(&s.desc[slot].ef);
     const uint64_t key = __ldcg(&s.desc[slot].key);
-    run_query<VT, DMAX>(s.base, my, s.qring + slot * s.base.d, k, ef, key, s.out_ids + slot * s.base.out_stride,
+    run_query<VT, DMAX, kFull>(s.base, my, s.qring + slot * s.base.d, k, ef, key, s.out_ids + slot * s.base.out_stride,
                         s.out_d + slot * s.base.out_stride, nullptr, nullptr, 0.f, Solo());
     __syncwarp();
     if (lane == 0) {
@@ -995,14 +1007,14 @@ __global__ void __launch_bounds__(128) k_greedy_probe(const __grid_constant__ Gr
       }
       continue;
     }
-    float dc = rows_dist<VT, G, CPL>(vec, a.layer.scale, stride, cur, 1, qs, nchunk);
+    float dc = rows_dist<VT, G, CPL, kFull>(vec, a.layer.scale, stride, cur, 1, qs, nchunk);
     dc = __shfl_sync(0xffffffffu, dc, 0);
     int32_t moves = 0;
     for (;;) {
       const int32_t nb = a.layer.adj[(int64_t)cur * kMmax + lane];
       const int cnt = __popc(__ballot_sync(0xffffffffu, nb >= 0));
       // neighbours are packed at the front of each row (-1 padding after)
-      const float dn = rows_dist<VT, G, CPL>(vec, a.layer.scale, stride, nb, cnt, qs, nchunk);
+      const float dn = rows_dist<VT, G, CPL, kFull>(vec, a.layer.scale, stride, nb, cnt, qs, nchunk);
       const uint64_t kk = lane < cnt ? pack(dn, (uint32_t)nb) : kEmpty;
       const uint64_t best = warp_min64(kk);
       if (best == kEmpty || !(key_dist(best) < dc)) break;
@@ -1037,9 +1049,76 @@ static cudaError_t launch_probe_vt(const GreedyProbeArgs& a, cudaStream_t st) {
   return launch_probe_t<VT, 1024>(a, st);
 }
 
+// ------------------------------------------------------------ launches
+
+// Chunks in flight for a launch of grid blocks: by the warps that can be
+// resident together on an SM -- the launch's share of them, or what the
+// shared memory leaves room for.  The lines are the warps that the variants'
+// registers allow.
+static int search_in_flight(int warps, int grid, size_t smem) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return kFull;
+  const int by_smem = (int)((size_t)(227 * 1024) / (smem + 1024));
+  const int blocks = std::min((grid + sms - 1) / sms, by_smem);
+  if (blocks * warps <= 8) return kFew;
+  return blocks * warps <= 16 ? kHalf : kFull;
+}
+
+template <typename VT, int DMAX>
+static cudaError_t launch_t(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
+  auto kern = k_search<VT, DMAX, kFull, Solo>;
+  if (a.team > 1)
+    kern = k_search<VT, DMAX, kFull, Team>;
+  else if (const int f = search_in_flight(warps, grid, smem); f != kFull)
+    kern = f == kHalf ? k_search<VT, DMAX, kHalf, Solo> : k_search<VT, DMAX, kFew, Solo>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, warps * 32, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <typename VT>
+static cudaError_t launch_vt(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
+  if (a.dpad <= 32) return launch_t<VT, 32>(a, warps, grid, smem, st);
+  if (a.dpad <= 64) return launch_t<VT, 64>(a, warps, grid, smem, st);
+  if (a.dpad <= 128) return launch_t<VT, 128>(a, warps, grid, smem, st);
+  if (a.dpad <= 512) return launch_t<VT, 512>(a, warps, grid, smem, st);
+  return launch_t<VT, 1024>(a, warps, grid, smem, st);
+}
+
+template <typename VT, int DMAX>
+static cudaError_t launch_serve_t(const ServeArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
+  auto kern = k_serve<VT, DMAX>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kern<<<grid, warps * 32, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <typename VT>
+static cudaError_t launch_serve_vt(const ServeArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
+  if (a.base.dpad <= 32) return launch_serve_t<VT, 32>(a, warps, grid, smem, st);
+  if (a.base.dpad <= 64) return launch_serve_t<VT, 64>(a, warps, grid, smem, st);
+  if (a.base.dpad <= 128) return launch_serve_t<VT, 128>(a, warps, grid, smem, st);
+  if (a.base.dpad <= 512) return launch_serve_t<VT, 512>(a, warps, grid, smem, st);
+  return launch_serve_t<VT, 1024>(a, warps, grid, smem, st);
+}
+
+#ifndef HENN_SEARCH_ROWS  // the rest once, not per storage type
+
+#define HENN_DECLARE(T)                                                                                       \
+  cudaError_t launch_search_##T(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st);      \
+  cudaError_t launch_serve_##T(const ServeArgs& a, int warps, int grid, size_t smem, cudaStream_t st);        \
+  cudaError_t launch_probe_##T(const GreedyProbeArgs& a, cudaStream_t st);
+HENN_DECLARE(bf16)
+HENN_DECLARE(fp8)
+#undef HENN_DECLARE
+
 cudaError_t launch_greedy_probe(const GreedyProbeArgs& a, int storage, cudaStream_t st) {
-  if (storage == HENN_BF16) return launch_probe_vt<__nv_bfloat16>(a, st);
-  if (storage == HENN_FP8E4M3) return launch_probe_vt<__nv_fp8_e4m3>(a, st);
+  if (storage == HENN_BF16) return launch_probe_bf16(a, st);
+  if (storage == HENN_FP8E4M3) return launch_probe_fp8(a, st);
   return launch_probe_vt<float>(a, st);
 }
 
@@ -1470,48 +1549,12 @@ cudaError_t search_persistent_grid(int device, int warps, size_t smem, int* grid
   return cudaSuccess;
 }
 
-template <typename VT, int DMAX>
-static cudaError_t launch_t(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
-  auto kern = a.team > 1 ? k_search<VT, DMAX, Team> : k_search<VT, DMAX, Solo>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid, warps * 32, smem, st>>>(a);
-  return cudaGetLastError();
-}
-
-template <typename VT>
-static cudaError_t launch_vt(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
-  if (a.dpad <= 32) return launch_t<VT, 32>(a, warps, grid, smem, st);
-  if (a.dpad <= 64) return launch_t<VT, 64>(a, warps, grid, smem, st);
-  if (a.dpad <= 128) return launch_t<VT, 128>(a, warps, grid, smem, st);
-  if (a.dpad <= 512) return launch_t<VT, 512>(a, warps, grid, smem, st);
-  return launch_t<VT, 1024>(a, warps, grid, smem, st);
-}
-
-template <typename VT, int DMAX>
-static cudaError_t launch_serve_t(const ServeArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
-  auto kern = k_serve<VT, DMAX>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid, warps * 32, smem, st>>>(a);
-  return cudaGetLastError();
-}
-
-template <typename VT>
-static cudaError_t launch_serve_vt(const ServeArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
-  if (a.base.dpad <= 32) return launch_serve_t<VT, 32>(a, warps, grid, smem, st);
-  if (a.base.dpad <= 64) return launch_serve_t<VT, 64>(a, warps, grid, smem, st);
-  if (a.base.dpad <= 128) return launch_serve_t<VT, 128>(a, warps, grid, smem, st);
-  if (a.base.dpad <= 512) return launch_serve_t<VT, 512>(a, warps, grid, smem, st);
-  return launch_serve_t<VT, 1024>(a, warps, grid, smem, st);
-}
-
 cudaError_t launch_serve(const ServeArgs& a, int warps_per_block, int grid, cudaStream_t st) {
   ServeArgs b = a;
   b.base.warp_smem = (int32_t)search_warp_smem(a.base.ef_cap, a.base.hash_bits, a.base.dpad);
   size_t smem = (size_t)b.base.warp_smem * warps_per_block;
-  if (a.base.storage == HENN_BF16) return launch_serve_vt<__nv_bfloat16>(b, warps_per_block, grid, smem, st);
-  if (a.base.storage == HENN_FP8E4M3) return launch_serve_vt<__nv_fp8_e4m3>(b, warps_per_block, grid, smem, st);
+  if (a.base.storage == HENN_BF16) return launch_serve_bf16(b, warps_per_block, grid, smem, st);
+  if (a.base.storage == HENN_FP8E4M3) return launch_serve_fp8(b, warps_per_block, grid, smem, st);
   return launch_serve_vt<float>(b, warps_per_block, grid, smem, st);
 }
 
@@ -1522,9 +1565,11 @@ cudaError_t launch_search(const SearchArgs& a, int warps_per_block, int grid, cu
   b.team = team;
   b.warp_smem = (int32_t)search_team_smem(a.ef_cap, a.hash_bits, a.dpad, team);
   size_t smem = (size_t)b.warp_smem * (warps_per_block / team);
-  if (a.storage == HENN_BF16) return launch_vt<__nv_bfloat16>(b, warps_per_block, grid, smem, st);
-  if (a.storage == HENN_FP8E4M3) return launch_vt<__nv_fp8_e4m3>(b, warps_per_block, grid, smem, st);
+  if (a.storage == HENN_BF16) return launch_search_bf16(b, warps_per_block, grid, smem, st);
+  if (a.storage == HENN_FP8E4M3) return launch_search_fp8(b, warps_per_block, grid, smem, st);
   return launch_vt<float>(b, warps_per_block, grid, smem, st);
 }
+
+#endif  // HENN_SEARCH_ROWS
 
 }  // namespace henn
