@@ -502,15 +502,31 @@ __device__ __noinline__ int beam(const int32_t* __restrict__ adj, const void* ve
     cand = lane < ccnt ? stage[lane] : kEmpty;
     const int cpos = lane < ccnt ? lower_bound_w(W, nw, cand) + lane : 0x7fffffff;
     const int p0 = __shfl_sync(0xffffffffu, cpos, 0);
-    // entries at or after p0 shift right by the number of smaller candidates
-    for (int base = ((nw - 1) >> 5) << 5; base >= (p0 & ~31); base -= 32) {
-      const int i = base + lane;
-      const bool mv = i < nw && i >= p0;
-      const uint64_t w = mv ? W[i] : kEmpty;
-      int cl = 0;
-      for (int j = 0; j < ccnt; ++j) cl += stage[j] < (w & kKeyMask);
+    // entries at or after p0 shift right by the number of smaller candidates:
+    // entry i by those whose lower bound is <= i.  The bounds ascend over the
+    // lanes, so a search over the lanes by shuffles finds that number (6
+    // steps, whatever the candidates' number; comparing every entry with
+    // every candidate took most of an expansion at ef 512).  Two chunks at a
+    // time, from the end: both are read before either is written, and an
+    // entry moves by at most 32
+    const int lb = lane < ccnt ? cpos - lane : 0x7fffffff;
+    for (int base = ((nw - 1) >> 5) << 5; base >= (p0 & ~31); base -= 64) {
+      const int i1 = base + lane, i0 = i1 - 32;
+      const bool mv1 = i1 < nw && i1 >= p0, mv0 = i0 >= p0;  // i0 < nw
+      const uint64_t w1 = mv1 ? W[i1] : kEmpty, w0 = mv0 ? W[i0] : kEmpty;
+      int c1 = 0, c0 = 0;
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1) {
+        if (__shfl_sync(0xffffffffu, lb, c1 + step - 1) <= i1) c1 += step;
+        if (__shfl_sync(0xffffffffu, lb, c0 + step - 1) <= i0) c0 += step;
+      }
+      // 31 of them so far: the last lane's may be one more
+      const int top = __shfl_sync(0xffffffffu, lb, 31);
+      c1 += c1 == 31 && top <= i1;
+      c0 += c0 == 31 && top <= i0;
       __syncwarp();
-      if (mv && i + cl < ef) W[i + cl] = w;
+      if (mv1 && i1 + c1 < ef) W[i1 + c1] = w1;
+      if (mv0 && i0 + c0 < ef) W[i0 + c0] = w0;
       __syncwarp();
     }
     if (lane < ccnt && cpos < ef) W[cpos] = cand;
