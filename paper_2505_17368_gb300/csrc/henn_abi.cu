@@ -1339,13 +1339,17 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
     if (has_exact && sp.exact_method == HENN_EXACT_SORT)
       require(idx->layers[top_exact].size <= (1 << (hb_min - 1)),
               "exact_method SORT: the exact layer must have <= 2^(hash_bits - 1) points (512 by default)");
-    int warps = sp.warps_per_block > 0 ? sp.warps_per_block : kSearchWarps;
-    require(warps >= 1 && warps <= kSearchWarps, "warps_per_block must be in [1, 4]");
     const int team = sp.team_size > 0 ? sp.team_size : 1;
+    // warps per block of a launch of n queries with a beam capacity
+    auto block_warps = [&](int64_t n, int cap, int bits) {
+      if (sp.warps_per_block > 0) return (int)sp.warps_per_block;
+      return team > 1 ? kSearchWarps : search_block_warps(idx->device, n, search_warp_smem(cap, bits, idx->dpad));
+    };
+    const int warps = block_warps(nq, ef_cap, hb);
+    require(warps >= 1 && warps <= kSearchWarps, "warps_per_block must be in [1, 4]");
     require(team == 1 || team == 2 || team == 4, "team_size must be 1, 2 or 4");
     require(sp.tile_n == 0 || sp.tile_n == 128 || sp.tile_n == 256, "tile_n must be 0, 128 or 256");
     require(warps % team == 0, "team_size must divide warps_per_block");
-    const int teams = warps / team;  // queries in flight per block
 
     Scratch sc(st, idx->search_pool());
     const float* dQ = Q;
@@ -1532,6 +1536,7 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
     launches += groups;
     if (groups == 1) {
       a.order = d_order;
+      const int teams = warps / team;  // queries in flight per block
       size_t smem = search_team_smem(ef_cap, hb, idx->dpad, team) * teams;
       int64_t blocks_needed = (nq + teams - 1) / teams;
       int grid = (int)std::min<int64_t>(persistent_grid(idx->device, warps, smem), blocks_needed);
@@ -1555,10 +1560,11 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
         ag.ef_cap = caps[g];
         ag.hash_bits = pick_hash_bits(caps[g]);
         ag.counter = counter + g;
+        const int gwarps = block_warps(count[g], ag.ef_cap, ag.hash_bits), teams = gwarps / team;
         size_t smem = search_team_smem(ag.ef_cap, ag.hash_bits, idx->dpad, team) * teams;
         int64_t blocks_needed = (count[g] + teams - 1) / teams;
-        int grid = (int)std::min<int64_t>(persistent_grid(idx->device, warps, smem), blocks_needed);
-        CK(launch_search(ag, warps, grid, t));
+        int grid = (int)std::min<int64_t>(persistent_grid(idx->device, gwarps, smem), blocks_needed);
+        CK(launch_search(ag, gwarps, grid, t));
         cudaEvent_t join;
         CK(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
         CK(cudaEventRecord(join, t));

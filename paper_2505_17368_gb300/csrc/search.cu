@@ -1554,6 +1554,17 @@ int search_hash_bits(int ef_cap) {
   return hb;
 }
 
+int search_block_warps(int device, int64_t nq, size_t warp_smem) {
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms < 1)
+    return kSearchWarps;
+  const size_t room = 227 * 1024, fixed = 1024;  // shared memory of an SM; what each block takes besides
+  const int64_t most = 4 * SearchOcc<kFull>::kMinBlocks;
+  const int64_t r4 = std::min<int64_t>(most, 4 * (int64_t)(room / (4 * warp_smem + fixed)));
+  const int64_t r1 = std::min<int64_t>(most, (int64_t)(room / (warp_smem + fixed)));
+  return nq >= sms * r4 && r1 < r4 + 2 ? kSearchWarps : 1;
+}
+
 cudaError_t search_persistent_grid(int device, int warps, size_t smem, int* grid) {
   int sms = 0;
   const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
