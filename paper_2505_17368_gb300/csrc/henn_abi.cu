@@ -271,6 +271,11 @@ struct henn_index {
   // build, insertion or deletion in progress, which waits for it before it
   // returns, so that every stream may use the memory afterwards.
   cudaStream_t mem_stream = nullptr;
+  bool drained = false;  // the operation in progress has waited for the device
+  void begin(cudaStream_t st) {
+    mem_stream = st;
+    drained = false;
+  }
   template <typename T>
   T* alloc(size_t count) {
     void* p = nullptr;
@@ -284,14 +289,23 @@ struct henn_index {
     bytes += (int64_t)b;
     return static_cast<T*>(p);
   }
-  // frees one allocation made by alloc(), once the device is idle (searches
-  // on other streams may still read it)
+  // Waits for the device (searches on other streams may still read the
+  // index's memory) the way freeing a cudaMalloc'ed block does: also while
+  // another thread captures a stream, when cudaDeviceSynchronize is refused.
+  // cudaFree of pool memory does not wait.
+  static void drain() {
+    void* p = nullptr;
+    if (cudaMalloc(&p, 16) == cudaSuccess) cudaFree(p);
+  }
+  // frees one allocation made by alloc(): nothing may run on the index beside
+  // the operation in progress, so waiting once covers what ran before it
   void release(void* p) {
     if (!p) return;
     for (size_t i = 0; i < allocs.size(); ++i)
       if (allocs[i] == p) {
-        cudaDeviceSynchronize();
-        cudaFreeAsync(p, mem_stream);
+        if (!drained) drain();
+        drained = true;
+        cudaFree(p);
         allocs.erase(allocs.begin() + (long)i);
         return;
       }
@@ -359,19 +373,19 @@ struct henn_index {
     cudaGetDevice(&current);
     if (current != device) cudaSetDevice(device);
     drop_entry_ops();
-    cudaDeviceSynchronize();
-    if (pool) cudaMemPoolDestroy(pool);
+    if (pool) {
+      cudaDeviceSynchronize();
+      cudaMemPoolDestroy(pool);
+    }
+    drain();
     for (cudaEvent_t e : tev)
       if (e) cudaEventDestroy(e);
     for (cudaStream_t t : side) cudaStreamDestroy(t);
-    for (void* p : allocs) cudaFreeAsync(p, nullptr);
+    for (void* p : allocs) cudaFree(p);
     if (device < 64) {
       DevicePool& dp = device_pool(device);
       std::lock_guard<std::mutex> lk(dp.mu);
-      if (--dp.indexes == 0 && dp.pool) {
-        cudaStreamSynchronize(nullptr);
-        cudaMemPoolTrimTo(dp.pool, kPoolIdle);
-      }
+      if (--dp.indexes == 0 && dp.pool) cudaMemPoolTrimTo(dp.pool, kPoolIdle);
     }
     if (current != device) cudaSetDevice(current);
   }
@@ -785,7 +799,7 @@ extern "C" henn_status henn_build(const float* X, int64_t n, int32_t d, int32_t 
     BuildTrace tr(st);
 
     ix = new henn_index();
-    ix->mem_stream = st;
+    ix->begin(st);
     ix->params = p;
     ix->n = n;
     ix->d = d;
@@ -904,7 +918,7 @@ void rebuild_from(henn_index* ix, int32_t i, const std::vector<int32_t>& liveids
   } own;
   CK(cudaStreamCreateWithFlags(&own.s, cudaStreamNonBlocking));
   cudaStream_t st = own.s;
-  ix->mem_stream = st;
+  ix->begin(st);
   BuildTrace tr(st);
   ix->drop_entry_ops();
   for (int32_t li = ix->L; li >= i; --li) {
@@ -992,7 +1006,7 @@ extern "C" henn_status henn_delete(henn_index* ix, const int64_t* ids, int64_t n
     require(ids != nullptr, "ids is NULL");
     for (int64_t i = 0; i < n; ++i) require(ids[i] >= 0 && ids[i] < ix->n, "id out of range");
     cudaStream_t st = (cudaStream_t)stream;
-    ix->mem_stream = st;
+    ix->begin(st);
     if (!ix->dead) {
       ix->dead = ix->alloc<uint8_t>((size_t)ix->cap_n);
       CK(cudaMemsetAsync(ix->dead, 0, (size_t)ix->cap_n, st));
@@ -1057,7 +1071,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
     } own;
     CK(cudaStreamCreateWithFlags(&own.s, cudaStreamNonBlocking));
     cudaStream_t st = own.s;
-    ix->mem_stream = st;
+    ix->begin(st);
     const int64_t n0 = ix->n, n1 = n0 + n_new;
     const int32_t dpad = ix->dpad, d = ix->d, M = ix->M;
     const bool angular = ix->metric == HENN_ANGULAR;
