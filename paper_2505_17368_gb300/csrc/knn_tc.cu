@@ -17,9 +17,9 @@
 // product plus the FP32 accumulation, so the certified candidate pool of
 // the exact FP32 rerank stays small.
 //
-// Layout of one CTA (192 threads): warp 0 issues TMA loads, warp 1 owns
-// TMEM and issues the MMAs (one thread), warps 2-5 drain the accumulators
-// (TMEM lanes 32*(w%4)..+31 = rows of the 128-row block).  Rows of at most
+// Layout of one CTA (192 or 320 threads): warp 0 issues TMA loads, warp 1
+// owns TMEM and issues the MMAs (one thread), warps 2-5 or 2-9 drain the
+// accumulators (TMEM lanes 32*(w%4)..+31 = rows of the 128-row block).  Rows of at most
 // 128 values: the A block (128 rows, hi and lo planes) stays in shared
 // memory and B tiles (256 columns x 64 values of one plane) stream through
 // a 3-stage ring.  Wider rows (up to 1024 values): the A block no longer

@@ -104,12 +104,14 @@ int search_beam_cap(int k, int ef, int ef_upper, int ef_l1, bool rerank, int rer
 // entries without changing results, so it is sized for occupancy).
 int search_hash_bits(int ef_cap);
 // Warps (queries) per block of a launch of nq queries that use warp_smem
-// bytes each: 4 where such blocks fill every SM; 1 where there are too few
-// queries for that (single warps spread evenly over the SMs) or where whole
-// blocks of 4 leave shared memory unused that 2 or more warps would fit in.
-// 1,000 queries at ef 200: 771 us against 812 us in blocks of 4; 5,000 at ef
-// 32 - 512: 3.1 against 3.8 ms; 10,000 at ef 50 (full): 878 against 867 us.
-int search_block_warps(int device, int64_t nq, size_t warp_smem);
+// bytes each: 4, which share an SM's L1; 1 where blocks of 4 leave shared
+// memory unused that a quarter more warps would fit in (5,000 queries at ef
+// 32 - 512: 2.7 against 3.1 ms), and for launches of under 16 warps per SM
+// that run with more rows in flight, which single warps spread more evenly
+// (2,000 queries over 100,000 x 960 BF16: 1,287 against 1,344 us).  Where
+// they do not, blocks of 4 stay (100 queries over 50,000 x 100 FP32 at ef 16:
+// 100 against 123 us).
+int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad);
 // Blocks of `warps` warps using `smem` bytes of shared memory each that
 // stay resident together on every SM of `device` (a persistent launch).
 cudaError_t search_persistent_grid(int device, int warps, size_t smem, int* grid);
