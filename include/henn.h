@@ -25,6 +25,9 @@
  *    synchronise the stream before returning.
  *  - The caller owns every array it passes; the library copies what it
  *    keeps.  The index owns its device memory until henn_free().
+ *  - Device memory comes from one pool per device, which keeps up to 1 GiB
+ *    of unused memory between calls, and 256 MiB once the device's last
+ *    index has been freed.
  *  - No call throws.  Each returns a henn_status; on failure nothing is
  *    written to *out handles and henn_last_error() describes the failure.
  *  - A const index may be searched concurrently from several host threads
@@ -345,7 +348,8 @@ henn_status henn_greedy_probe(const henn_index* idx, int32_t layer, const float*
 
 /*
  * Exact k nearest neighbours of each query among the n base vectors (the
- * k-NN query of Sec. 2): tiled distances plus an exact FP32 rerank.  All
+ * k-NN query of Sec. 2): tiled distances plus an exact FP32 rerank of a
+ * candidate pool that is proven to hold the answer (else widened).  All
  * pointers device; out rows of k (int64 ids, float distances as in
  * henn_search).  1 <= k <= 112, 1 <= d <= 1024.
  */
