@@ -1071,12 +1071,14 @@ static cudaError_t launch_probe_vt(const GreedyProbeArgs& a, cudaStream_t st) {
 
 // ------------------------------------------------------------ launches
 
-// Rows of 32 chunks read by 8 lanes: four rows fill four chunks per lane
-// already, and more of them in flight gained nothing (50,000 x 100 FP32, 100
-// queries at ef 16: 117 us against 100; x 256 FP8 at ef 64 the same).
+// The most chunks in flight that a kernel gains from.  Rows of 32 chunks read
+// by 8 lanes hold four chunks per lane already: FP32 rows (65 - 128 values)
+// gain from kHalf only (50,000 x 100, ef 200: 600 queries 730 us, 777 with
+// kFew, 814 with kFull), FP8 rows (257 - 512 values) from neither.
 template <typename VT, int DMAX>
-constexpr bool has_more_in_flight() {
-  return RowShape<VT, DMAX>::G != 8 || RowShape<VT, DMAX>::CPL != 4;
+constexpr int most_in_flight() {
+  if (RowShape<VT, DMAX>::G != 8 || RowShape<VT, DMAX>::CPL != 4) return kFew;
+  return std::is_same<VT, float>::value ? kHalf : kFull;
 }
 
 // Chunks in flight for a launch of grid blocks: by the warps that can be
@@ -1097,11 +1099,12 @@ static int search_in_flight(int warps, int grid, size_t smem) {
 template <typename VT, int DMAX>
 static cudaError_t launch_t(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
   auto kern = a.team > 1 ? k_search<VT, DMAX, kFull, Team> : k_search<VT, DMAX, kFull, Solo>;
-  if constexpr (has_more_in_flight<VT, DMAX>()) {
+  constexpr int most = most_in_flight<VT, DMAX>();
+  if constexpr (most != kFull) {
     if (a.team <= 1) {
       const int f = search_in_flight(warps, grid, smem);
       if (f == kHalf) kern = k_search<VT, DMAX, kHalf, Solo>;
-      if (f == kFew) kern = k_search<VT, DMAX, kFew, Solo>;
+      if (f == kFew) kern = k_search<VT, DMAX, most, Solo>;
     }
   }
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1555,15 +1558,16 @@ size_t search_team_smem(int ef_cap, int hash_bits, int dpad, int team) {
   return team > 1 ? b + sizeof(TeamJob) : b;
 }
 
-// has_more_in_flight of the kernel that a storage type and row width run
+// whether the kernel of a storage type and row width has variants with more
+// chunks in flight
 static bool more_in_flight(int storage, int dpad) {
   auto of = [&](auto vt) {
     using VT = decltype(vt);
-    if (dpad <= 32) return has_more_in_flight<VT, 32>();
-    if (dpad <= 64) return has_more_in_flight<VT, 64>();
-    if (dpad <= 128) return has_more_in_flight<VT, 128>();
-    if (dpad <= 512) return has_more_in_flight<VT, 512>();
-    return has_more_in_flight<VT, 1024>();
+    if (dpad <= 32) return most_in_flight<VT, 32>() != kFull;
+    if (dpad <= 64) return most_in_flight<VT, 64>() != kFull;
+    if (dpad <= 128) return most_in_flight<VT, 128>() != kFull;
+    if (dpad <= 512) return most_in_flight<VT, 512>() != kFull;
+    return most_in_flight<VT, 1024>() != kFull;
   };
   if (storage == HENN_BF16) return of(__nv_bfloat16());
   if (storage == HENN_FP8E4M3) return of(__nv_fp8_e4m3());

@@ -109,8 +109,7 @@ int search_hash_bits(int ef_cap);
 // 32 - 512: 2.7 against 3.1 ms), and for launches of under 16 warps per SM
 // that run with more rows in flight, which single warps spread more evenly
 // (2,000 queries over 100,000 x 960 BF16: 1,287 against 1,344 us).  Where
-// they do not, blocks of 4 stay (100 queries over 50,000 x 100 FP32 at ef 16:
-// 100 against 123 us).
+// they do not, blocks of 4 stay.
 int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad);
 // Blocks of `warps` warps using `smem` bytes of shared memory each that
 // stay resident together on every SM of `device` (a persistent launch).
