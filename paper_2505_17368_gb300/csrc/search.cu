@@ -49,11 +49,11 @@ namespace henn {
 // few warps -- has registers to spare and waits for its rows in fewer round
 // trips: kHalf at up to 16 warps per SM (128 registers), kFew at up to 8
 // (255).  The arithmetic and its order are the same (rows_dist), so results
-// do not depend on the choice; search_in_flight has the rule.  Against kFull:
-// 2,000 queries over 100,000 x 960 BF16 rows 1.77 -> 1.35 ms (kHalf), 1,000
-// over 50,000 x 100 FP8 at ef 200 912 -> 735 us, one over 50,000 x 32 FP32
-// 172 -> 149 us (kFew), 64 over 1,000,000 x 128 BF16 (8 new rows an
-// expansion, one round trip either way) 421 -> 423 us.
+// do not depend on the choice; search_in_flight has the rule.  Against the
+// full launch's kernel in blocks of four: 2,000 queries over 100,000 x 960
+// BF16 rows 1.81 -> 1.20 ms (kHalf); 1,000 over 50,000 x 100 FP8 at ef 200 844
+// -> 516 us, 64 over 1,000,000 x 128 BF16 429 -> 361 us, one over 50,000 x 32
+// FP32 171 -> 148 us (kFew).
 constexpr int kFull = 4, kHalf = 16, kFew = 32;
 template <int IF>
 struct SearchOcc {
