@@ -349,9 +349,11 @@ henn_status henn_greedy_probe(const henn_index* idx, int32_t layer, const float*
 /*
  * Exact k nearest neighbours of each query among the n base vectors (the
  * k-NN query of Sec. 2): tiled distances plus an exact FP32 rerank of a
- * candidate pool that is proven to hold the answer (else widened).  All
- * pointers device; out rows of k (int64 ids, float distances as in
- * henn_search).  1 <= k <= 112, 1 <= d <= 1024.
+ * candidate pool that is proven to hold the answer; queries whose pool is
+ * not, and small calls, compare all base vectors in FP32.  So the answer is
+ * the first k in (FP32 distance, index) order, for a query alone as in a
+ * batch.  All pointers device; out rows of k (int64 ids, float distances as
+ * in henn_search).  1 <= k <= 112, 1 <= d <= 1024.
  */
 henn_status henn_exact_knn(const float* X, int64_t n, int32_t d, const float* Q, int64_t nq, int32_t k,
                            int32_t metric, int64_t* out_ids, float* out_dists, void* stream);

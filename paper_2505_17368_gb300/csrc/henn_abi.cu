@@ -641,7 +641,7 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
   if (use_tc) {
     hi = sc.get<uint16_t>((size_t)s * dk);
     lo = sc.get<uint16_t>((size_t)s * dk);
-    launch_order_split(ix->xw, Ly.ids, s, dpad, ix->seed, li, mode == 1, mean, dk, hi, lo, inv, norms, nullptr, nmax, st);
+    launch_order_split(ix->xw, Ly.ids, s, dpad, ix->seed, li, mode == 1, mean, dk, hi, lo, inv, norms, nmax, st);
   } else {
     xo = sc.get<float>((size_t)s * dpad);
     launch_order_gather(ix->xw, Ly.ids, s, dpad, ix->seed, li, ix->graph, mean, inv, xo, norms, st);
@@ -672,7 +672,7 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
     if (herr) throw Failure(HENN_ERR_TIMEOUT, "tensor-core tile pipeline wait timed out (code " + std::to_string(herr) + ")");
     tile_u = tc_tile_unit_error(dk);
   } else {
-    launch_tile_topk_simt(xo, norms, s, xo, norms, s, dpad, mode, KP, 1, cand, nullptr, nullptr, st);
+    launch_tile_topk_simt(xo, norms, s, xo, norms, s, dpad, mode, KP, 1, cand, st);
     CKL("distance tiles");
     tile_u = (dpad + 8.0) * std::ldexp(1.0, -24);
   }
@@ -1184,7 +1184,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
         uint16_t* lo = sc.get<uint16_t>((size_t)s1 * dk);
         float* norms = sc.get<float>(s1);
         float* nmax = sc.get<float>(1);
-        launch_order_split(ix->xw, lids, s1, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, norms, nullptr, nmax, st);
+        launch_order_split(ix->xw, lids, s1, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, norms, nmax, st);
         const int32_t splits = tile_list_splits(c, s1, false);
         uint64_t* lists = sc.get<uint64_t>((size_t)splits * c * KP);
         uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)c * KP) : lists;
@@ -1590,8 +1590,8 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
         const int32_t splits =
             (int32_t)std::max<int64_t>(1, std::min<int64_t>((2 * 152 + rb - 1) / rb, (s + 4095) / 4096));
         uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)splits * nq * 32) : pkeys;
-        launch_tile_topk_simt(qo, qn, nq, eo.xo, eo.norms, s, dpad, 2, 32, splits, cand, nullptr, nullptr, st);
-        if (splits > 1) launch_merge_splits(cand, nq, 32, splits, pkeys, nullptr, st);
+        launch_tile_topk_simt(qo, qn, nq, eo.xo, eo.norms, s, dpad, 2, 32, splits, cand, st);
+        if (splits > 1) launch_merge_splits(cand, nq, splits, pkeys, st);
         a.pre_tile_u = (dpad + 8.0) * std::ldexp(1.0, -24);
         launches += splits > 1 ? 3 : 2;
       }
@@ -1811,39 +1811,21 @@ extern "C" henn_status henn_index_get_layer(const henn_index* idx, int32_t layer
 
 namespace {
 
-// Pool width of the SIMT engine's candidates for k results.
-int32_t knn_pool(int32_t k) {
-  int32_t KP = 32;
-  while (KP < k + 16) KP <<= 1;
-  return KP;
-}
-
-// Exact k-NN by the SIMT FP32 tiles: a pool of at least k + 16 candidates,
-// reranked.  xp / qp: rows of dpad floats.
-void knn_simt(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t dpad, int32_t k, int32_t metric,
+// Exact k-NN by the scan alone.  xp / qp: rows of dpad floats.
+void knn_sweep(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t dpad, int32_t k, int32_t metric,
               int64_t* out_ids, float* out_dists, Scratch& sc, cudaStream_t st) {
-  float* xn = sc.get<float>(n);
-  float* qn = sc.get<float>(nq);
-  launch_sq_norms(xp, n, dpad, xn, st);
-  launch_sq_norms(qp, nq, dpad, qn, st);
-  const int32_t KP = knn_pool(k);
-  const int64_t rb = (nq + 63) / 64;
-  const int32_t splits = (int32_t)std::max<int64_t>(1, std::min<int64_t>((2 * 152 + rb - 1) / rb, (n + 4095) / 4096));
-  uint64_t* cand = sc.get<uint64_t>((size_t)splits * nq * KP);
-  launch_tile_topk_simt(qp, qn, nq, xp, xn, n, dpad, 2, KP, splits, cand, nullptr, nullptr, st);
-  uint64_t* merged = cand;
-  if (splits > 1) {
-    merged = sc.get<uint64_t>((size_t)nq * KP);
-    launch_merge_splits(cand, nq, KP, splits, merged, nullptr, st);
-  }
-  launch_rerank_queries(qp, nq, xp, dpad, metric, merged, KP, k, out_ids, out_dists, nullptr, nullptr, st);
+  const unsigned grid = sweep_grid();
+  uint64_t* lists = sc.get<uint64_t>(sweep_lists(grid, nq) * sweep_pool(k));
+  launch_sweep_knn(qp, nq, xp, n, dpad, metric, k, grid, lists, nullptr, nullptr, out_ids, out_dists, st);
 }
 
-// From this many (query, point) pairs on, the tensor-core path.  It takes
-// about 170 us at the least (14 launches); the SIMT path as long for one
-// query against 2,000 x 32 points (159 us) and more beyond: 8 queries 278 us,
-// 1 against 20,000 x 128 511 us, 1,000 against 1,000,000 x 128 11.9 ms (1.8
-// ms on the tensor cores).
+// From this many (query, point) pairs on, the tensor-core path: about 110 us
+// at the least (14 launches), where the sweep of a smaller call takes 32 - 99
+// us (one query against 2,000 x 32 to two against 2,000 x 960 points, k 10 and
+// 112).  The sweep stays ahead for a while beyond (8 queries against 2,000 x
+// 128 points: 32 against 111 us at k 10, 68 against 129 at k 100) and falls
+// behind with the columns (one against 20,000 x 128 at k 100: 250 against 196
+// us; 10,000 against 100,000 x 128: 18 ms against 1.8).
 constexpr int64_t kKnnTilesMin = 4096;
 // Queries that go through it together (its buffers are sized for them).
 constexpr int64_t kKnnBatch = 65536;
@@ -1853,8 +1835,10 @@ constexpr int64_t kKnnBatch = 65536;
 // column outside it is provably farther than the k-th), queries that fail
 // the certificate collect all columns that can matter in a second tile pass
 // over those queries alone, and those with too many (massive ties, values
-// that are no numbers) take the SIMT path.  Everything is enqueued without
-// a wait: the later passes read how many queries they have on the device.
+// that are no numbers) scan all columns.  So every answer is the exact one:
+// the first k in the order of (FP32 distance, index), whichever pass gave it.
+// Everything is enqueued without a wait: the later passes read how many
+// queries they have on the device.
 void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t dpad, int32_t k, int32_t metric,
                int64_t* out_ids, float* out_dists, Scratch& sc, cudaStream_t st) {
   const int32_t dk = round_up(dpad, 64);
@@ -1864,14 +1848,12 @@ void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t 
   void* hi = sc.get<uint16_t>((size_t)n * dk);
   void* lo = sc.get<uint16_t>((size_t)n * dk);
   float* xn = sc.get<float>(n);
-  float* xraw = sc.get<float>(n);
   float* nmax = sc.get<float>(2);  // of the points; of the queries (not used)
-  launch_order_split(xp, nullptr, n, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, xn, xraw, nmax, st);
+  launch_order_split(xp, nullptr, n, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, xn, nmax, st);
   const int64_t nb = std::min(nq, kKnnBatch);
   uint16_t* qhi = sc.get<uint16_t>((size_t)nb * dk);
   uint16_t* qlo = sc.get<uint16_t>((size_t)nb * dk);
   float* qn = sc.get<float>(nb);
-  float* qraw = sc.get<float>(nb);
   // the pool: 32, 64 or 128 candidates, at least 16 more than k; for more
   // than 16, lists enough that one (16 of half a split's columns) seldom
   // holds as many of the k as it is long: 6 on average
@@ -1897,12 +1879,8 @@ void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t 
   int32_t* over = sc.get<int32_t>((size_t)nb + 3);  // number, rows, flagged rows' number, tile error flag
   flagged.count = over + nb + 1;
   int32_t* err = over + nb + 2;
-  const int32_t KS = knn_pool(k);
-  // the SIMT path's lists: split over the points as far as 64 MB allow
-  const int32_t ssplits = (int32_t)std::max<int64_t>(
-      1, std::min<int64_t>({(int64_t)64, (n + 4095) / 4096, (int64_t)(64 << 20) / (nb * KS * 8)}));
-  uint64_t* scand = sc.get<uint64_t>((size_t)ssplits * nb * KS);
-  uint64_t* smerged = ssplits > 1 ? sc.get<uint64_t>((size_t)nb * KS) : scand;
+  const unsigned sgrid = sweep_grid();
+  uint64_t* slists = sc.get<uint64_t>(sweep_lists(sgrid, nb) * sweep_pool(k));
   const double tile_u = tc_tile_unit_error(dk);
   for (int64_t q0 = 0; q0 < nq; q0 += nb) {
     const int64_t c = std::min(nb, nq - q0);
@@ -1911,7 +1889,7 @@ void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t 
     float* od = out_dists + q0 * k;
     CK(cudaMemsetAsync(over, 0, sizeof(int32_t), st));
     CK(cudaMemsetAsync(flagged.count, 0, 2 * sizeof(int32_t), st));
-    launch_order_split(q, nullptr, c, dpad, 0, 0, true, mean, dk, qhi, qlo, nullptr, qn, qraw, nmax + 1, st);
+    launch_order_split(q, nullptr, c, dpad, 0, 0, true, mean, dk, qhi, qlo, nullptr, qn, nmax + 1, st);
     CK(launch_tile_lists_tc(qhi, qlo, qn, c, hi, lo, xn, n, dk, 2, nullptr, splits, lists, lthr, err, st));
     launch_merge_lists(lists, lthr, c, splits, KP, cand, thr, st);
     launch_rerank_knn(q, c, xp, n, dpad, metric, cand, thr, KP, k, qn, nmax, tile_u, err, oi, od, flagged, st);
@@ -1920,9 +1898,7 @@ void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t 
                               ncols, kCollectCap, err, st));
     launch_rerank_collected_knn(q, xp, flagged, c, dpad, metric, n, grid, cols, ncols, kCollectCap, k, oi, od, over,
                                 err, st);
-    launch_tile_topk_simt(q, qraw, c, xp, xraw, n, dpad, 2, KS, ssplits, scand, over + 1, over, st);
-    if (ssplits > 1) launch_merge_splits(scand, c, KS, ssplits, smerged, over, st);
-    launch_rerank_queries(q, c, xp, dpad, metric, smerged, KS, k, oi, od, over + 1, over, st);
+    launch_sweep_knn(q, c, xp, n, dpad, metric, k, sgrid, slists, over + 1, over, oi, od, st);
   }
 }
 
@@ -1964,7 +1940,7 @@ extern "C" henn_status henn_exact_knn(const float* X, int64_t n, int32_t d, cons
     if (nq * n >= kKnnTilesMin)
       knn_tiles(xp, n, qp, nq, dpad, k, metric, out_ids, out_dists, sc, st);
     else
-      knn_simt(xp, n, qp, nq, dpad, k, metric, out_ids, out_dists, sc, st);
+      knn_sweep(xp, n, qp, nq, dpad, k, metric, out_ids, out_dists, sc, st);
     CKL("exact knn");
     return HENN_OK;
   } catch (const Failure& f) {

@@ -64,12 +64,9 @@ void launch_order_gather(const float* xw, const int32_t* ids, int64_t s, int32_t
 // its mean at rank perm(j) (identity: j), as BF16 planes hi = bf16(x), lo =
 // bf16(x - hi), dk wide, with its squared norm; inv (nullable) as above;
 // *norm_max the largest norm (NaN if one is)
-// (raw_norms, nullable: the rows' squared norms without the mean taken off)
 void launch_order_split(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, uint64_t seed, int32_t layer,
                         bool identity, const float* mean, int32_t dk, void* hi, void* lo, int32_t* inv, float* norms,
-                        float* raw_norms, float* norm_max, cudaStream_t st);
-// squared norms of rows of dpad floats
-void launch_sq_norms(const float* x, int64_t s, int32_t dpad, float* norms, cudaStream_t st);
+                        float* norm_max, cudaStream_t st);
 void launch_gather_rows32(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, float* out,
                           cudaStream_t st);
 void launch_quantize(const float* x, int64_t n, int32_t d, int32_t dpad_in, int32_t dpad_out,
@@ -79,13 +76,11 @@ void launch_quantize(const float* x, int64_t n, int32_t d, int32_t dpad_in, int3
 //   mode 0: causal (column c valid iff c < row), A == B
 //   mode 1: all other rows (c != row), A == B
 //   mode 2: rows of A against all rows of B
-// rowsel / count (nullable): only the rows rowsel[0 .. *count - 1] of A; list
-// i is then row rowsel[i]'s
 void launch_tile_topk_simt(const float* A, const float* An, int64_t na, const float* B, const float* Bn,
                            int64_t nb, int32_t dpad, int32_t mode, int32_t KP, int32_t splits,
-                           uint64_t* out, const int32_t* rowsel, const int32_t* count, cudaStream_t st);
-void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t KP, int32_t splits, uint64_t* out,
-                         const int32_t* count, cudaStream_t st);
+                           uint64_t* out, cudaStream_t st);
+// lists of 32 keys per row and split (splits x rows x 32) -> the 32 smallest
+void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t splits, uint64_t* out, cudaStream_t st);
 // Sorted lists of 32 keys per row and split (splits x rows x 32, with their
 // bounds thr_in) -> the KP (32, 64 or 128) smallest of each row, and a bound
 // on what they leave out: every column of the row that is not among them has
@@ -191,20 +186,49 @@ void launch_rerank_knn(const float* Q, int64_t nq, const float* X, int64_t n, in
 void launch_exact_rows(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, int32_t metric,
                        const int32_t* inv, int32_t mode, const int32_t* rows, int32_t nrows, int32_t M,
                        int32_t* fwd, float* fwd_d, cudaStream_t st);
-// exact rerank of query candidates -> k results (rowsel / count as for the
-// SIMT tiles: list i is query rowsel[i]'s)
-void launch_rerank_queries(const float* Q, int64_t nq, const float* X, int32_t dpad, int32_t metric,
-                           const uint64_t* cand, int32_t KP, int32_t k, int64_t* out_ids, float* out_d,
-                           const int32_t* rowsel, const int32_t* count, cudaStream_t st);
+// Exact k results by a scan of all n columns (rowsel / count, nullable: of
+// the queries rowsel[0 .. *count - 1] only, their number on the device).
+// Each block of kSweepRows queries has sweep_runs runs of columns (at least 128
+// columns each), shared out over sweep_grid() CTAs; lists: sweep_lists(grid, nq)
+// lists of sweep_pool(k) keys.
+constexpr int kSweepRows = 32;
+constexpr int kSweepMaxRuns = 128;
+constexpr unsigned kSweepItems = 8;  // per CTA, unless the blocks alone are more
+// Runs per block: one wave of the CTAs while there are few blocks, else the
+// number of runs with the least time over all waves (10,000 queries are 313
+// blocks: one run each would leave the second wave of 304 CTAs empty).
+__host__ __device__ inline int32_t sweep_runs(unsigned grid, int64_t rows, int64_t n) {
+  const unsigned blocks = (unsigned)((rows + kSweepRows - 1) / kSweepRows);
+  const unsigned parts = (unsigned)((n + 127) / 128);
+  const unsigned most = parts < (unsigned)kSweepMaxRuns ? parts : (unsigned)kSweepMaxRuns;
+  unsigned pick = 1;
+  if (blocks * 16 <= grid) {
+    pick = grid / blocks;
+  } else {
+    unsigned best = ~0u;
+    for (unsigned k = 1; k <= 16 && (k == 1 || blocks * k <= kSweepItems * grid); ++k) {
+      const unsigned waves = (blocks * k + grid - 1) / grid;
+      const unsigned cost = waves * ((parts + k - 1) / k + 1);
+      if (cost < best) {
+        best = cost;
+        pick = k;
+      }
+    }
+  }
+  return (int32_t)(pick < most ? pick : most);
+}
+// for any number of rows up to nq
+inline size_t sweep_lists(unsigned grid, int64_t nq) {
+  const int64_t blocks = (nq + kSweepRows - 1) / kSweepRows;
+  const int64_t runs = (int64_t)kSweepItems * grid < blocks * kSweepMaxRuns ? (int64_t)kSweepItems * grid : blocks * kSweepMaxRuns;
+  return (size_t)kSweepRows * (size_t)(blocks > runs ? blocks : runs);
+}
+inline int32_t sweep_pool(int32_t k) { return k <= 32 ? 32 : (k <= 64 ? 64 : 128); }
+unsigned sweep_grid();
+void launch_sweep_knn(const float* Q, int64_t nq, const float* X, int64_t n, int32_t dpad, int32_t metric, int32_t k,
+                     unsigned grid, uint64_t* lists, const int32_t* rowsel, const int32_t* count, int64_t* out_ids,
+                     float* out_d, cudaStream_t st);
 void launch_max_nonneg(const float* v, int64_t n, float* out, cudaStream_t st);
-// exact recompute of the forward list of uncertified rows
-void launch_exact_rows(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, int32_t metric,
-                       const int32_t* inv, int32_t mode, const int32_t* rows, int32_t nrows, int32_t M,
-                       int32_t* fwd, float* fwd_d, cudaStream_t st);
-// exact rerank of query candidates -> k results
-void launch_rerank_queries(const float* Q, int64_t nq, const float* X, int32_t dpad, int32_t metric,
-                           const uint64_t* cand, int32_t KP, int32_t k, int64_t* out_ids, float* out_d,
-                           cudaStream_t st);
 
 // graph.cu: edge rule
 void launch_rev_count(const int32_t* fwd, int64_t s, int32_t M, int32_t* cnt, cudaStream_t st);

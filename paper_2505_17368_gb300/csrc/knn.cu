@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -21,9 +23,7 @@ template <int KP>
 __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict__ A, const float* __restrict__ An,
                                                         int64_t na, const float* __restrict__ B,
                                                         const float* __restrict__ Bn, int64_t nb, int32_t dpad,
-                                                        int32_t mode, int32_t splits, uint64_t* __restrict__ out,
-                                                        const int32_t* __restrict__ rowsel,
-                                                        const int32_t* __restrict__ count) {
+                                                        int32_t mode, int32_t splits, uint64_t* __restrict__ out) {
   __shared__ __align__(16) float As[kBK][kBM + 4];
   __shared__ __align__(16) float Bs[kBK][kBN + 4];
   __shared__ float S[kBM][kBN + 1];
@@ -31,11 +31,6 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   const int warp = tid >> 5;
-  const int64_t stride = na;  // rows between two splits' lists
-  if (count) {
-    na = min(na, (int64_t)*count);
-    if ((int64_t)blockIdx.x * kBM >= na) return;
-  }
   const int64_t nblocks = (na + kBM - 1) / kBM;
   // causal rows: heaviest row blocks first
   const int64_t rb = (mode == 0) ? (nblocks - 1 - blockIdx.x) : blockIdx.x;
@@ -68,7 +63,7 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
         int row = idx >> 3, kq = (idx & 7) * 4;
         int64_t gr = r0 + row;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (gr < na) v = *reinterpret_cast<const float4*>(A + (rowsel ? (int64_t)rowsel[gr] : gr) * dpad + k0 + kq);
+        if (gr < na) v = *reinterpret_cast<const float4*>(A + gr * dpad + k0 + kq);
         As[kq + 0][row] = v.x;
         As[kq + 1][row] = v.y;
         As[kq + 2][row] = v.z;
@@ -98,7 +93,7 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       int64_t gr = r0 + ty * 4 + i;
-      float an = gr < na ? An[rowsel ? (int64_t)rowsel[gr] : gr] : 0.f;
+      float an = gr < na ? An[gr] : 0.f;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         int64_t gc = c0 + tx * 4 + j;
@@ -145,7 +140,7 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
   for (int i = 0; i < 8; ++i) {
     int64_t gr = r0 + warp * 8 + i;
     if (gr < na) {
-      uint64_t* dst = out + ((int64_t)split * stride + gr) * KP;
+      uint64_t* dst = out + ((int64_t)split * na + gr) * KP;
 #pragma unroll
       for (int r = 0; r < KP / 32; ++r) dst[r * 32 + (tid & 31)] = lists[i].v[r];
     }
@@ -153,84 +148,54 @@ __global__ void __launch_bounds__(256) k_tile_topk_simt(const float* __restrict_
 }
 
 void launch_tile_topk_simt(const float* A, const float* An, int64_t na, const float* B, const float* Bn, int64_t nb,
-                           int32_t dpad, int32_t mode, int32_t KP, int32_t splits, uint64_t* out,
-                           const int32_t* rowsel, const int32_t* count, cudaStream_t st) {
+                           int32_t dpad, int32_t mode, int32_t KP, int32_t splits, uint64_t* out, cudaStream_t st) {
   dim3 grid((unsigned)((na + kBM - 1) / kBM), (unsigned)splits);
   switch (KP) {
-    case 32: k_tile_topk_simt<32><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
-    case 64: k_tile_topk_simt<64><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
-    case 128: k_tile_topk_simt<128><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
-    default: k_tile_topk_simt<256><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out, rowsel, count); break;
+    case 32: k_tile_topk_simt<32><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out); break;
+    case 64: k_tile_topk_simt<64><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out); break;
+    default: k_tile_topk_simt<128><<<grid, 256, 0, st>>>(A, An, na, B, Bn, nb, dpad, mode, splits, out); break;
   }
 }
 
-// merge per-split lists of one row into one list of KP
-template <int KP>
-__global__ void k_merge_splits(const uint64_t* __restrict__ in, int64_t rows, int32_t splits, uint64_t* __restrict__ out,
-                               const int32_t* __restrict__ count) {
+// merge per-split lists (32 keys) of one row into one
+__global__ void k_merge_splits(const uint64_t* __restrict__ in, int64_t rows, int32_t splits,
+                               uint64_t* __restrict__ out) {
   const int lane = threadIdx.x & 31;
-  const int64_t nr = count ? min(rows, (int64_t)*count) : rows;
-  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < nr;
+  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < rows;
        r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    WarpList<KP> list;
+    WarpList<32> list;
     list.clear();
     for (int s = 0; s < splits; ++s) {
-      const uint64_t* src = in + ((int64_t)s * rows + r) * KP;
-      for (int c = 0; c < KP; c += 32) {
-        uint64_t v = src[c + lane];
-        uint64_t thr = list.worst();
-        unsigned m = __ballot_sync(0xffffffffu, v < thr);
-        while (m) {
-          int sl = __ffs(m) - 1;
-          m &= m - 1;
-          uint64_t x = shfl64(v, sl);
-          if (x < list.worst()) list.insert(x);
-        }
+      const uint64_t v = in[((int64_t)s * rows + r) * 32 + lane];
+      unsigned m = __ballot_sync(0xffffffffu, v < list.worst());
+      while (m) {
+        const uint64_t x = shfl64(v, __ffs(m) - 1);
+        m &= m - 1;
+        if (x < list.worst()) list.insert(x);
       }
     }
-#pragma unroll
-    for (int q = 0; q < KP / 32; ++q) out[r * KP + q * 32 + lane] = list.v[q];
+    out[r * 32 + lane] = list.v[0];
   }
 }
 
-void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t KP, int32_t splits, uint64_t* out,
-                         const int32_t* count, cudaStream_t st) {
+void launch_merge_splits(const uint64_t* in, int64_t rows, int32_t splits, uint64_t* out, cudaStream_t st) {
   int grid = (int)((rows + 7) / 8);
   if (grid > 152 * 16) grid = 152 * 16;
-  switch (KP) {
-    case 32: k_merge_splits<32><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
-    case 64: k_merge_splits<64><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
-    case 128: k_merge_splits<128><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
-    default: k_merge_splits<256><<<grid, 256, 0, st>>>(in, rows, splits, out, count); break;
-  }
+  k_merge_splits<<<grid, 256, 0, st>>>(in, rows, splits, out);
 }
 
-// Exact FP32 distance, warp cooperative: lane k handles coordinates k, k+32,
-// ... (coalesced 128-byte lines), xor-tree reduction.  The operation order is
-// symmetric in (a, b), so dist(a,b) and dist(b,a) are bitwise equal.
-// L2: squared distance; angular (unit vectors): |a-b|^2 / 2 = 1 - cos.
-__device__ __forceinline__ float warp_exact_dist(const float* __restrict__ a, const float* __restrict__ b,
-                                                 int32_t dpad, int32_t metric) {
-  const int lane = threadIdx.x & 31;
-  float acc = 0.f;
-  for (int k = lane; k < dpad; k += 32) {
-    float t = a[k] - b[k];
-    acc = fmaf(t, t, acc);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  return metric == HENN_ANGULAR ? 0.5f * acc : acc;
-}
-
-// The same distance from row `a` to 32 rows at once: lane c gives row c's
-// index (count of them, lanes 0 .. count - 1) and gets its distance.  Eight
-// rows' loads are in flight together, and the 32 sums over the lanes are
-// formed by exchanging halves (31 shuffles for 32 rows instead of 160): lane
-// l ends with row l's sum, added up in the tree of the butterfly above
-// (offsets 16, 8, 4, 2, 1; addition commutes), so every distance has the bits
-// that warp_exact_dist gives it.  The rows come from L2 or HBM at random; one
-// row at a time left one load in flight per lane and a butterfly per row (the
-// rerank of 10,000 x 32 points' 32 candidates: 104 us, now 64 us).
+// Exact FP32 distance from row `a` to 32 rows at once: lane c gives row c's
+// index (count of them, lanes 0 .. count - 1) and gets its distance.  L2:
+// squared distance; angular (unit vectors): |a-b|^2 / 2 = 1 - cos.  Per row,
+// lane l sums the squared differences of elements l, l + 32, ... in order,
+// and the lanes' sums are added up in the tree of an xor butterfly (offsets
+// 16, 8, 4, 2, 1; addition commutes): symmetric in (a, b), so dist(a, b) and
+// dist(b, a) are bitwise equal.  Eight rows' loads are in flight together,
+// and the 32 sums over the lanes are formed by exchanging halves (31 shuffles
+// for 32 rows instead of 160): lane l ends with row l's sum.  The rows come
+// from L2 or HBM at random; one row at a time left one load in flight per
+// lane and a butterfly per row (the rerank of 10,000 x 32 points' 32
+// candidates: 104 us, now 64 us).
 __device__ __forceinline__ float warp_exact_dist32(const float* __restrict__ a, const float* __restrict__ X,
                                                    int64_t row, int count, int32_t dpad, int32_t metric) {
   const int lane = threadIdx.x & 31;
@@ -690,7 +655,7 @@ void launch_rerank_collected_knn(const float* Q, const float* X, const FlaggedRo
 // Exact forward lists of flagged rows, batched: a block takes RT flagged
 // rows (kept in shared memory) and streams every candidate column once for
 // all of them, so the columns are read once per RT rows instead of once per
-// row.  Each distance is formed exactly as warp_exact_dist forms it (lane
+// row.  Each distance is formed exactly as warp_exact_dist32 forms it (lane
 // l sums the squared differences of elements l, l+32, ... in order with
 // FMA, then the xor butterfly over the 32 lanes), so a flagged row gets the
 // list the certified path would give it.  Column validity: mode 0 (causal,
@@ -879,51 +844,229 @@ void launch_exact_rows(const float* xw, const int32_t* ids, int64_t s, int32_t d
   return launch_exact_rows_t<64, 0>(xw, ids, s, dpad, metric, inv, mode, rows, nrows, M, fwd, fwd_d, st);
 }
 
-// Query candidates -> exact k results (int64 ids, reported distances).
-template <int KP>
-__global__ void k_rerank_queries(const float* __restrict__ Q, int64_t nq, const float* __restrict__ X, int32_t dpad,
-                                 int32_t metric, const uint64_t* __restrict__ cand, int32_t k,
-                                 int64_t* __restrict__ out_ids, float* __restrict__ out_d,
-                                 const int32_t* __restrict__ rowsel, const int32_t* __restrict__ count) {
-  const int lane = threadIdx.x & 31;
-  const int64_t nl = count ? min(nq, (int64_t)*count) : nq;
-  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < nl;
-       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t q = rowsel ? (int64_t)rowsel[i] : i;
-    WarpList<KP> list;
-    list.clear();
-    for (int c = 0; c < KP; ++c) {
-      uint64_t key = cand[i * KP + c];
-      if (key == kEmpty) break;
-      uint32_t col = key_index(key);
-      float dv = warp_exact_dist(Q + q * dpad, X + (int64_t)col * dpad, dpad, metric);
-      list.insert(pack(dv, col));
-    }
+// Exact k-NN by a scan of all columns, for calls too small for the tiles and
+// for queries whose candidate lists and collected columns prove nothing.  An
+// item is 32 queries, four per warp, and one of sweep_runs runs of columns; a
+// block copies 32 KB of columns at a time to shared memory (double-buffered;
+// columns follow each other, so a chunk is one piece) and each warp forms the
+// differences of 8 columns and its 4 queries in registers, lane l the
+// elements l, l + 32, ..., summed over the lanes as warp_exact_dist32 does:
+// the same bits.  Bound by issue and by shared memory (a load of a column's 32
+// elements serves 4 queries): 10,000 queries x 100,000 x 128 all swept 18 ms;
+// a warp per query reading the columns from L2 took 62 ms.  KD = dpad / 32 up
+// to 4 (the queries in registers), else 0 (in shared memory).
+// rowsel / count (nullable): the queries rowsel[0 .. *count - 1] only.  List i
+// of run s (KP keys, ascending) is lists[(s * rows + i) * KP ..].
+constexpr int kSweepBytes = 32768;  // of columns per buffer
+
+// acc += (a - x, b - x) squared, each step rounded as a - x and fmaf round it
+__device__ __forceinline__ void add_sq_diff2(float2& acc, float a, float b, float x) {
+  asm("{\n\t.reg .b64 q, xx, t, s;\n\t"
+      "mov.b64 q, {%2, %3};\n\t"
+      "mov.b64 xx, {%4, %4};\n\t"
+      "mov.b64 s, {%0, %1};\n\t"
+      "sub.rn.f32x2 t, q, xx;\n\t"
+      "fma.rn.f32x2 s, t, t, s;\n\t"
+      "mov.b64 {%0, %1}, s;\n\t}"
+      : "+f"(acc.x), "+f"(acc.y)
+      : "f"(a), "f"(b), "f"(x));
+}
+
+template <int KP, int KD>
+__global__ void __launch_bounds__(256) k_sweep_knn(const float* __restrict__ Q, int64_t nq, const float* __restrict__ X,
+                                                  int64_t n, int32_t dpad, int32_t metric,
+                                                  const int32_t* __restrict__ rowsel,
+                                                  const int32_t* __restrict__ count, uint64_t* __restrict__ lists) {
+  constexpr int QW = kSweepRows / 8;  // queries per warp
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* buf = reinterpret_cast<float*>(smem_raw);  // 2 x kSweepBytes, then the queries (KD = 0)
+  float* qsm = buf + 2 * (kSweepBytes / 4);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t rows = count ? min(nq, (int64_t)*count) : nq;
+  if (rows <= 0) return;
+  const int kd = KD > 0 ? KD : dpad / 32;
+  // columns per chunk: as many 32s as the buffer holds, or 16 or 8 of wide rows
+  const int cb = kd <= 8 ? 256 / kd / 32 * 32 : (kd <= 16 ? 16 : 8);
+  const int64_t blocks = (rows + kSweepRows - 1) / kSweepRows;
+  const int32_t runs = sweep_runs(gridDim.x, rows, n);
+  const int64_t tiles = (n + 31) / 32, per = (tiles + runs - 1) / runs;  // of 32 columns
+  for (int64_t item = blockIdx.x; item < blocks * runs; item += gridDim.x) {
+    const int64_t s = item / blocks, i0 = (item - s * blocks) * kSweepRows + w * QW;
+    const int64_t c_end = min(n, (s + 1) * per * 32);
+    const int64_t c_first = s * per * 32;
+    const int64_t chunks = c_end > c_first ? (c_end - c_first + cb - 1) / cb : 0;
+    auto fetch = [&](int64_t ch) {  // columns c_first + ch * cb .. into buffer ch & 1
+      const int64_t c = c_first + ch * cb;
+      const int words = (int)min((int64_t)cb, c_end - c) * dpad;
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(buf + (ch & 1) * (kSweepBytes / 4));
+      for (int e = 4 * threadIdx.x; e < words; e += 4 * 256)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 4 * e), "l"(X + c * dpad + e) : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    __syncthreads();  // the last item's buffers are read
+    if (chunks > 0) fetch(0);
+    float qr[QW][KD > 0 ? KD : 1];
 #pragma unroll
-    for (int r = 0; r < KP / 32; ++r) {
-      int g = r * 32 + lane;
-      if (g < k) {
-        uint64_t key = list.v[r];
-        bool e = key == kEmpty;
-        float dv = e ? __int_as_float(0x7f800000) : key_dist(key);
-        out_ids[q * k + g] = e ? -1 : (int64_t)key_index(key);
-        out_d[q * k + g] = e ? dv : (metric == HENN_ANGULAR ? dv : sqrtf(dv));
+    for (int r = 0; r < QW; ++r) {
+      // past the last query: the last one again (its list is not written)
+      const int64_t i = min(i0 + r, rows - 1);
+      const float* q = Q + (rowsel ? (int64_t)rowsel[i] : i) * dpad;
+      if constexpr (KD > 0) {
+#pragma unroll
+        for (int k = 0; k < KD; ++k) qr[r][k] = __ldg(q + 32 * k + lane);
+      } else {
+        for (int k = 0; k < kd; ++k) qsm[(w * QW + r) * dpad + 32 * k + lane] = __ldg(q + 32 * k + lane);
       }
     }
+    uint64_t v[QW][KP / 32];
+    float dist[QW];  // lane: of column 8 (lane & 3) + (lane >> 2) of the 32
+#pragma unroll
+    for (int r = 0; r < QW; ++r) {
+      dist[r] = 0.f;
+#pragma unroll
+      for (int g = 0; g < KP / 32; ++g) v[r][g] = kEmpty;
+    }
+    for (int64_t ch = 0; ch < chunks; ++ch) {
+      if (ch + 1 < chunks) {
+        fetch(ch + 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      __syncthreads();
+      const int64_t c0 = c_first + ch * cb;
+      const int have = (int)min((int64_t)cb, c_end - c0);
+      const float* cols = buf + (ch & 1) * (kSweepBytes / 4) + lane;
+#pragma unroll 1
+      for (int g = 0; 8 * g < have && i0 < rows; ++g) {
+        float2 acc[QW / 2][8];  // queries 2 p and 2 p + 1
+#pragma unroll
+        for (int p = 0; p < QW / 2; ++p)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) acc[p][i] = make_float2(0.f, 0.f);
+        auto step = [&](int k, const float (&q)[QW]) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const float x = cols[(8 * g + i) * dpad + 32 * k];  // past the last column: not used
+#pragma unroll
+            for (int p = 0; p < QW / 2; ++p) add_sq_diff2(acc[p][i], q[2 * p], q[2 * p + 1], x);
+          }
+        };
+        if constexpr (KD > 0) {
+#pragma unroll
+          for (int k = 0; k < KD; ++k) {
+            float q[QW];
+#pragma unroll
+            for (int r = 0; r < QW; ++r) q[r] = qr[r][k];
+            step(k, q);
+          }
+        } else {
+#pragma unroll 2
+          for (int k = 0; k < kd; ++k) {
+            float q[QW];
+#pragma unroll
+            for (int r = 0; r < QW; ++r) q[r] = qsm[(w * QW + r) * dpad + 32 * k + lane];
+            step(k, q);
+          }
+        }
+        // these 8 are columns 8 * at .. of their 32
+        const int64_t c8 = c0 / 8 + g;
+        const int at = (int)(c8 & 3);
+#pragma unroll
+        for (int r = 0; r < QW; ++r) {
+          float sum[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) sum[i] = r & 1 ? acc[r / 2][i].y : acc[r / 2][i].x;
+#pragma unroll
+          for (int o = 16; o >= 4; o >>= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < o / 4; ++i) {
+              const float keep = up ? sum[i + o / 4] : sum[i];
+              const float send = up ? sum[i] : sum[i + o / 4];
+              sum[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+          }
+          sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], 2);
+          sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], 1);
+          if ((lane & 3) == at) dist[r] = sum[0];
+        }
+        if (at == 3 || 8 * (c8 + 1) >= c_end) {  // the 32 are complete
+          const int64_t col = (c8 - at) * 8 + 8 * (lane & 3) + (lane >> 2);
+#pragma unroll
+          for (int r = 0; r < QW; ++r) {
+            const float dv = metric == HENN_ANGULAR ? 0.5f * dist[r] : dist[r];
+            const uint64_t key = col < c_end ? pack(dv, (uint32_t)col) : kEmpty;
+            if (__any_sync(0xffffffffu, key < shfl64(v[r][KP / 32 - 1], 31))) merge_sorted32(v[r], warp_sort_asc(key));
+          }
+        }
+      }
+      __syncthreads();  // the buffer is read before the copy after next
+    }
+#pragma unroll
+    for (int r = 0; r < QW; ++r)
+      if (i0 + r < rows)  // warp-uniform
+#pragma unroll
+        for (int g = 0; g < KP / 32; ++g) lists[(s * rows + i0 + r) * KP + 32 * g + lane] = v[r][g];
   }
 }
 
-void launch_rerank_queries(const float* Q, int64_t nq, const float* X, int32_t dpad, int32_t metric, const uint64_t* cand,
-                           int32_t KP, int32_t k, int64_t* out_ids, float* out_d, const int32_t* rowsel,
-                           const int32_t* count, cudaStream_t st) {
-  int grid = (int)((nq + 7) / 8);
-  if (grid > 152 * 32) grid = 152 * 32;
-  if (grid < 1) grid = 1;
-  switch (KP) {
-    case 32: k_rerank_queries<32><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
-    case 64: k_rerank_queries<64><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
-    case 128: k_rerank_queries<128><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
-    default: k_rerank_queries<256><<<grid, 256, 0, st>>>(Q, nq, X, dpad, metric, cand, k, out_ids, out_d, rowsel, count); break;
+// the runs' lists of one query into its k results
+template <int KP>
+__global__ void __launch_bounds__(256) k_sweep_results(const uint64_t* __restrict__ lists, int64_t nq, int64_t n,
+                                                      int32_t metric, int32_t k, unsigned sweep_grid,
+                                                      const int32_t* __restrict__ rowsel,
+                                                      const int32_t* __restrict__ count,
+                                                      int64_t* __restrict__ out_ids, float* __restrict__ out_d) {
+  const int lane = threadIdx.x & 31;
+  const int64_t rows = count ? min(nq, (int64_t)*count) : nq;
+  if (rows <= 0) return;
+  const int32_t runs = sweep_runs(sweep_grid, rows, n);
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < rows;
+       i += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    uint64_t v[KP / 32];
+#pragma unroll
+    for (int r = 0; r < KP / 32; ++r) v[r] = kEmpty;
+    for (int32_t s = 0; s < runs; ++s)
+#pragma unroll
+      for (int r = 0; r < KP / 32; ++r) merge_sorted32(v, __ldg(lists + ((int64_t)s * rows + i) * KP + 32 * r + lane));
+    write_knn(v, rowsel ? (int64_t)rowsel[i] : i, k, metric, out_ids, out_d);
+  }
+}
+
+unsigned sweep_grid() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+    return 1;
+  return (unsigned)(2 * sms);
+}
+
+void launch_sweep_knn(const float* Q, int64_t nq, const float* X, int64_t n, int32_t dpad, int32_t metric, int32_t k,
+                     unsigned grid, uint64_t* lists, const int32_t* rowsel, const int32_t* count, int64_t* out_ids,
+                     float* out_d, cudaStream_t st) {
+  int g = (int)((nq + 7) / 8);
+  if (g > 152 * 16) g = 152 * 16;
+  const size_t smem = 2 * kSweepBytes + (dpad > 128 ? sizeof(float) * kSweepRows * (size_t)dpad : 0);
+  auto both = [&](auto scan, auto results) {
+    cudaFuncSetAttribute(scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    scan<<<grid, 256, smem, st>>>(Q, nq, X, n, dpad, metric, rowsel, count, lists);
+    results<<<g, 256, 0, st>>>(lists, nq, n, metric, k, grid, rowsel, count, out_ids, out_d);
+  };
+  auto width = [&](auto pool) {
+    constexpr int KP = decltype(pool)::value;
+    switch (dpad / 32) {
+      case 1: both(k_sweep_knn<KP, 1>, k_sweep_results<KP>); break;
+      case 2: both(k_sweep_knn<KP, 2>, k_sweep_results<KP>); break;
+      case 3: both(k_sweep_knn<KP, 3>, k_sweep_results<KP>); break;
+      case 4: both(k_sweep_knn<KP, 4>, k_sweep_results<KP>); break;
+      default: both(k_sweep_knn<KP, 0>, k_sweep_results<KP>); break;
+    }
+  };
+  switch (sweep_pool(k)) {
+    case 32: width(std::integral_constant<int, 32>()); break;
+    case 64: width(std::integral_constant<int, 64>()); break;
+    default: width(std::integral_constant<int, 128>()); break;
   }
 }
 

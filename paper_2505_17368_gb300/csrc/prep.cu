@@ -176,14 +176,14 @@ __global__ void __launch_bounds__(256) k_order_split(const float* __restrict__ x
                                                      const float* __restrict__ mean, int32_t dk,
                                                      __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                                      int32_t* __restrict__ inv, float* __restrict__ norms,
-                                                     float* __restrict__ raw_norms, float* __restrict__ norm_max) {
+                                                     float* __restrict__ norm_max) {
   const int lane = threadIdx.x & 31;
   int most = 0;  // bits of the largest norm (a NaN is above +inf)
   for (int64_t j = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; j < s;
        j += ((int64_t)gridDim.x * blockDim.x) >> 5) {
     const int64_t rank = identity ? j : (int64_t)f.perm((uint64_t)j);
     const float* src = xw + (ids ? (int64_t)ids[j] : j) * dpad;
-    float acc = 0.f, raw = 0.f;
+    float acc = 0.f;
     for (int k = 4 * lane; k < dk; k += 128) {
       float v[4] = {0.f, 0.f, 0.f, 0.f};
       if (k < dpad) {
@@ -193,7 +193,6 @@ __global__ void __launch_bounds__(256) k_order_split(const float* __restrict__ x
         v[1] = x.y - m.y;
         v[2] = x.z - m.z;
         v[3] = x.w - m.w;
-        raw = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, raw))));
       }
       uint32_t h[2], l[2];
 #pragma unroll
@@ -212,11 +211,6 @@ __global__ void __launch_bounds__(256) k_order_split(const float* __restrict__ x
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     most = max(most, __float_as_int(acc));
-    if (raw_norms) {  // uniform
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) raw += __shfl_xor_sync(0xffffffffu, raw, o);
-      if (lane == 0) raw_norms[rank] = raw;
-    }
     if (lane == 0) {
       if (inv) inv[rank] = (int32_t)j;
       norms[rank] = acc;
@@ -227,33 +221,14 @@ __global__ void __launch_bounds__(256) k_order_split(const float* __restrict__ x
 
 void launch_order_split(const float* xw, const int32_t* ids, int64_t s, int32_t dpad, uint64_t seed, int32_t layer,
                         bool identity, const float* mean, int32_t dk, void* hi, void* lo, int32_t* inv, float* norms,
-                        float* raw_norms, float* norm_max, cudaStream_t st) {
+                        float* norm_max, cudaStream_t st) {
   cudaMemsetAsync(norm_max, 0, sizeof(float), st);
   int grid = (int)((s + 7) / 8);
   if (grid > 152 * 8) grid = 152 * 8;
   const Feistel f = Feistel::make(seed, layer, (uint64_t)s);
   k_order_split<<<grid, 256, 0, st>>>(xw, ids, s, dpad, f, identity ? 1 : 0, mean, dk,
                                       static_cast<__nv_bfloat16*>(hi), static_cast<__nv_bfloat16*>(lo), inv, norms,
-                                      raw_norms, norm_max);
-}
-
-// one warp per row
-__global__ void k_sq_norms(const float* __restrict__ x, int64_t s, int32_t dpad, float* __restrict__ norms) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < s;
-       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    float acc = 0.f;
-    for (int k = lane; k < dpad; k += 32) acc = fmaf(x[r * dpad + k], x[r * dpad + k], acc);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) norms[r] = acc;
-  }
-}
-
-void launch_sq_norms(const float* x, int64_t s, int32_t dpad, float* norms, cudaStream_t st) {
-  int grid = (int)((s + 7) / 8);
-  if (grid > 152 * 8) grid = 152 * 8;
-  k_sq_norms<<<grid, 256, 0, st>>>(x, s, dpad, norms);
+                                      norm_max);
 }
 
 __global__ void k_gather_rows32(const float* __restrict__ xw, const int32_t* __restrict__ ids, int64_t s,
