@@ -692,7 +692,7 @@ void build_layer_graph(henn_index* ix, const henn_build_params& p, int32_t li, C
   flagged.rows = sc.get<int32_t>(s);
   flagged.thr = sc.get<float>(s);
   CK(cudaMemsetAsync(flagged.count, 0, sizeof(int32_t), st));
-  launch_rerank_fwd(ix->xw, Ly.ids, s, 0, dpad, ix->metric, inv, cand, thr, s, mode == 0, KP, M, norms, nmax, tile_u,
+  launch_rerank_fwd(ix->xw, Ly.ids, s, 0, dpad, ix->metric, inv, cand, thr, s, mode == 0, false, KP, M, norms, nmax, tile_u,
                     Ly.fwd, Ly.fwd_d, flagged, st);
   CKL("rerank");
   int32_t nunc = 0;
@@ -1199,7 +1199,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
         flagged.count = err + 1;
         flagged.rows = sc.get<int32_t>(c);
         flagged.thr = sc.get<float>(c);
-        launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, thr, s1, true, KP, M, norms + s0,
+        launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, thr, s1, true, true, KP, M, norms + s0,
                           nmax, tc_tile_unit_error(dk), Ly.fwd, Ly.fwd_d, flagged, st);
         CKL("rerank");
         int32_t host[2] = {0, 0};

@@ -154,10 +154,11 @@ struct FlaggedRows {
 // Row r is layer position inv[r], or row0 + r with inv == nullptr (columns
 // are then positions too).  thr: the pools' bounds (nullptr: a full pool's
 // last key).  nb: the columns; a row may take those before row0 + r (causal)
-// or all but itself.
+// or all but itself.  inserted: rows whose pool lacks columns at distances
+// that overflow are flagged too (a build's lists leave such columns out).
 void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
-                       const int32_t* inv, const uint64_t* cand, const float* thr, int64_t nb, bool causal, int32_t KP,
-                       int32_t M, const float* norms, const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d,
+                       const int32_t* inv, const uint64_t* cand, const float* thr, int64_t nb, bool causal, bool inserted,
+                       int32_t KP, int32_t M, const float* norms, const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d,
                        const FlaggedRows& flagged, cudaStream_t st);
 // The flagged rows' BF16 planes and norms, compact; lim[i]: causal the row's
 // own rank row0 + r, else nb; self[i]: r with skip_self, else -1.
@@ -165,7 +166,8 @@ void launch_gather_flagged(const FlaggedRows& f, int64_t max_rows, int64_t row0,
                            int64_t nb, const void* hi, const void* lo, const float* norms, int32_t dk, void* hi_out,
                            void* lo_out, float* norms_out, int32_t* lim, int32_t* self, cudaStream_t st);
 // exact FP32 rerank of collected columns -> forward lists of the flagged
-// rows; rows with more than cap columns in one CTA (or any, with *err set)
+// rows; rows with more than cap columns in one CTA or without a bound (or any,
+// with *err set)
 // go to over (over[0]: their number, then the rows, plus row0)
 void launch_rerank_collected_fwd(const float* xw, const int32_t* ids, const FlaggedRows& f, int64_t max_rows,
                                  int64_t row0, int32_t dpad, int32_t metric, const int32_t* inv, int64_t nb,

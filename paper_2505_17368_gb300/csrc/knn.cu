@@ -310,7 +310,10 @@ void launch_merge_lists(const uint64_t* in, const float* thr_in, int64_t rows, i
 // last exact distance dm, no outside column belongs to the list.  Else
 // *collect is the tile distance at or under which every column of the list
 // lies: their true distances are at most dm (the pool holds that many), so
-// their tile distances at most dm + beta.
+// their tile distances at most dm + beta.  *collect is +inf where no bound
+// holds: fewer than the wanted number in the pool, values that are no
+// numbers, or norms so large that a column of the list may overflow in the
+// tiles (its tile distance would be +inf or no number, and left out).
 __device__ __forceinline__ bool pool_certified(double thr, double dm, float norm_row, float norm_max, double tile_u,
                                                int32_t dpad, float* collect) {
   // relative error bound of the exact FP32 distances (dpad / 32 FMA
@@ -326,6 +329,11 @@ __device__ __forceinline__ bool pool_certified(double thr, double dm, float norm
   const double nc = norm_max != norm_max ? (double)norm_max : fmin((double)norm_max, rad * rad);
   const double beta = tile_u * 4.0 * (nr + nc) + 1e-30;
   *collect = __double2float_ru(dm * (1.0 + slack) + beta);
+  // norms and products of columns within reach add up to (2 rad)^2 at most
+  if (!(4.0 * rad * rad < 3.4e38)) {
+    *collect = __int_as_float(0x7f800000);
+    return false;
+  }
   return thr - beta > dm * (1.0 + slack);
 }
 
@@ -333,8 +341,7 @@ __device__ __forceinline__ void flag_row(const FlaggedRows& f, int32_t row, floa
   if ((threadIdx.x & 31) == 0) {
     const int at = atomicAdd(f.count, 1);
     f.rows[at] = row;
-    // not a number (a distance or a norm that is none): every column
-    f.thr[at] = thr != thr ? __int_as_float(0x7f800000) : thr;
+    f.thr[at] = thr != thr ? __int_as_float(0x7f800000) : thr;  // +inf: no bound
   }
 }
 
@@ -384,7 +391,7 @@ __global__ void __launch_bounds__(256) k_rerank_fwd(const float* __restrict__ xw
                                                     int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
                                                     const int32_t* __restrict__ inv, const uint64_t* __restrict__ cand,
                                                     const float* __restrict__ thr, int64_t nb, int32_t causal,
-                                                    int32_t M, const float* __restrict__ norms,
+                                                    int32_t inserted, int32_t M, const float* __restrict__ norms,
                                                     const float* __restrict__ norm_max, double tile_u,
                                                     int32_t* __restrict__ fwd, float* __restrict__ fwd_d,
                                                     FlaggedRows flagged) {
@@ -420,7 +427,9 @@ __global__ void __launch_bounds__(256) k_rerank_fwd(const float* __restrict__ xw
     // what bounds the columns left out (+inf: there are none)
     const float bound = all ? __int_as_float(0x7f800000)
                         : thr ? thr[r] : (last == kEmpty ? __int_as_float(0x7f800000) : key_dist(last));
-    if (!isinf(bound)) {
+    // (an insertion's lists are exact: a pool that is not full lacks the
+    // columns whose tile distances are no finite numbers)
+    if (!isinf(bound) || (inserted && !all)) {
       const uint64_t mkey = list_key(v, M - 1);
       double dm = (mkey == kEmpty) ? 1e300 : (double)key_dist(mkey);
       // exact distances here are of raw vectors; tile distances of centred
@@ -435,23 +444,26 @@ __global__ void __launch_bounds__(256) k_rerank_fwd(const float* __restrict__ xw
 }
 
 void launch_rerank_fwd(const float* xw, const int32_t* ids, int64_t nr, int64_t row0, int32_t dpad, int32_t metric,
-                       const int32_t* inv, const uint64_t* cand, const float* thr, int64_t nb, bool causal, int32_t KP,
-                       int32_t M, const float* norms, const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d,
+                       const int32_t* inv, const uint64_t* cand, const float* thr, int64_t nb, bool causal, bool inserted,
+                       int32_t KP, int32_t M, const float* norms, const float* norm_max, double tile_u, int32_t* fwd, float* fwd_d,
                        const FlaggedRows& flagged, cudaStream_t st) {
   int grid = (int)((nr + 7) / 8);
   if (grid > 152 * 32) grid = 152 * 32;
   if (grid < 1) grid = 1;
   switch (KP) {
     case 32:
-      k_rerank_fwd<32><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, M, norms, norm_max, tile_u, fwd,
+      k_rerank_fwd<32><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, inserted, M, norms,
+                                              norm_max, tile_u, fwd,
                                              fwd_d, flagged);
       break;
     case 64:
-      k_rerank_fwd<64><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, M, norms, norm_max, tile_u, fwd,
+      k_rerank_fwd<64><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, inserted, M, norms,
+                                              norm_max, tile_u, fwd,
                                              fwd_d, flagged);
       break;
     default:
-      k_rerank_fwd<128><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, M, norms, norm_max, tile_u,
+      k_rerank_fwd<128><<<grid, 256, 0, st>>>(xw, ids, nr, row0, dpad, metric, inv, cand, thr, nb, causal, inserted, M, norms,
+                                              norm_max, tile_u,
                                               fwd, fwd_d, flagged);
       break;
   }
@@ -553,12 +565,13 @@ template <int R, class RowOf, class KeyOf>
 __device__ __forceinline__ bool rerank_collected(const float* __restrict__ a, const float* __restrict__ X, int64_t i,
                                                  int32_t ns, const uint32_t* __restrict__ cols,
                                                  const int32_t* __restrict__ ncols, int32_t cap, int32_t dpad,
-                                                 int32_t metric, RowOf row_of, KeyOf key_of, uint64_t (&v)[R]) {
+                                                 int32_t metric, float thr, RowOf row_of, KeyOf key_of,
+                                                 uint64_t (&v)[R]) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int q = 0; q < R; ++q) v[q] = kEmpty;
   const int64_t seg0 = (i / kTileRows) * ns * kTileRows + i % kTileRows;
-  bool over = false;
+  bool over = isinf(thr);  // no bound: nothing says that the columns are all there
   for (int s = lane; s < ns; s += 32) over |= ncols[seg0 + (int64_t)s * kTileRows] > cap;
   if (__any_sync(0xffffffffu, over)) return false;
   for (int s = 0; s < ns; ++s) {
@@ -596,7 +609,7 @@ __global__ void __launch_bounds__(256) k_rerank_collected_fwd(const float* __res
     uint64_t v[1];  // M <= 32
     const bool ok = *err == 0 && rerank_collected(
                                      xw + (ids ? (int64_t)ids[j] : j) * dpad, xw, i, ns, cols, ncols, cap, dpad, metric,
-                                     [&](int64_t pos) { return ids ? (int64_t)ids[pos] : pos; },
+                                     f.thr[i], [&](int64_t pos) { return ids ? (int64_t)ids[pos] : pos; },
                                      [&](uint32_t c) { return inv ? (uint32_t)inv[c] : c; }, v);
     if (ok)
       write_fwd(v, j, M, fwd, fwd_d);
@@ -632,7 +645,7 @@ __global__ void __launch_bounds__(256) k_rerank_collected_knn(const float* __res
     uint64_t v[4];  // k <= 112
     const bool ok = *err == 0 &&
                     rerank_collected(
-                        Q + q * dpad, X, i, ns, cols, ncols, cap, dpad, metric, [](int64_t c) { return c; },
+                        Q + q * dpad, X, i, ns, cols, ncols, cap, dpad, metric, f.thr[i], [](int64_t c) { return c; },
                         [](uint32_t c) { return c; }, v) &&
                     list_key(v, k - 1) != kEmpty;
     if (ok)

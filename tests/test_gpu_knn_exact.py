@@ -1,5 +1,6 @@
 """Exact k-NN where the candidate lists prove nothing (GPU): batches whose near
-ties overflow the collecting pass, and calls too small for the tiles.  The
+ties overflow the collecting pass, calls too small for the tiles, and rows
+whose norms overflow.  The
 answer has to be the exact one there too, and the same for a query alone as
 in a batch.
 """
@@ -11,6 +12,15 @@ H = pytest.importorskip("paper_2505_17368_gb300")
 torch = pytest.importorskip("torch")
 
 from test_gpu_pools import check_dists, points, truth  # noqa: E402
+
+
+def huge(n, d, seed, lead):
+    """Finite rows on two sides of the origin, near ones 1e17 apart.  lead: "past" -- every squared norm overflows
+    FP32; "around" -- about half of them do (the largest FP32 value is 1.8447e19 squared)."""
+    x = 1e17 * points("spread", n, d, seed)
+    side = torch.where(torch.arange(n, device="cuda") % 2 == 0, 1.0, -1.0)
+    x[:, 0] = side * (2.2e19 if lead == "past" else 1.8447e19 + 0.1 * x[:, 0])
+    return x
 
 
 def near_rows(X, nq, seed):
@@ -53,3 +63,13 @@ def test_one_by_one_equals_batch(kind, n, d, k, metric):
     for q in (0, 127, 128, 511):
         i1, d1 = H.exact_knn(X, Q[q:q + 1], k, metric=metric)
         assert torch.equal(i1[0], ids[q]) and torch.equal(d1[0], dd[q])
+
+
+@pytest.mark.parametrize("lead", ["past", "around"])
+@pytest.mark.parametrize("n,d,nq,k", [(3000, 32, 500, 10), (2500, 200, 64, 100), (1200, 64, 2, 20)])
+def test_norms_that_overflow(lead, n, d, nq, k):
+    X = huge(n, d, 27, lead)
+    Q = X[torch.arange(nq, device="cuda") * 7919 % n] * 1.001
+    ids, dd = H.exact_knn(X, Q, k)
+    check_dists(dd, truth(X, Q, k, H.L2), d)
+    assert (ids >= 0).all() and (ids.sort(dim=1).values.diff(dim=1) > 0).all()
