@@ -89,7 +89,9 @@ typedef enum { HENN_SAMPLER_SAMPLING = 0, HENN_SAMPLER_HALVING = 1 } henn_sample
 
 /* Engine for the construction distance tiles: AUTO = tcgen05 where it
  * applies (M <= 16; rows of up to 128 values keep the row block resident in
- * shared memory, wider rows stream it slice by slice), else SIMT FP32. */
+ * shared memory, wider rows stream it slice by slice), else SIMT FP32.
+ * Insertions follow the index's choice: without tensor cores each new row
+ * is scanned exactly. */
 typedef enum { HENN_TILES_AUTO = 0, HENN_TILES_SIMT = 1, HENN_TILES_TCGEN05 = 2 } henn_tiles;
 
 /* ------------------------------------------------------------------ build */

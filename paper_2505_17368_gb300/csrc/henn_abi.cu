@@ -1171,7 +1171,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       CK(cudaMemcpyAsync(drows, rows.data(), sizeof(int32_t) * c, cudaMemcpyHostToDevice, st));
       const int32_t* lids = li >= 1 ? Ly.ids : nullptr;
       const int32_t KP = M <= 16 ? 32 : 64;
-      if (tc_tiles_supported(dpad, KP)) {
+      if (tc_tiles_supported(dpad, KP) && ix->params.tiles != HENN_TILES_SIMT) {
         // tiles of the new rows against the whole layer (row j takes the
         // columns before position s0 + j), reranked and settled as a build's.
         // The exact scan of every row that this replaces took 61.9 of the
