@@ -576,8 +576,9 @@ constexpr int32_t kCollectCap = 256;
 // them, listed in f): a second tile pass over those rows alone collects every
 // column that can belong to a list (its tile distance is at or under the
 // row's f.thr), and the exact FP32 rerank of these gives the list.  Rows with
-// too many such columns (massive ties) are scanned exactly.  Without this
-// pass the scan took them all: 52.9 of 74 ms of a 100,000 x 960 build.
+// too many such columns (massive ties), and all of them should the tile pass
+// time out, are scanned exactly.  Without this pass the scan took them all:
+// 52.9 of 74 ms of a 100,000 x 960 build.
 // hi / lo / norms: planes of the rows f refers to (nb: the columns, their
 // planes and norms b_*); row r may take columns below row0 + r (causal) or
 // all but itself.
@@ -604,11 +605,9 @@ void settle_flagged(henn_index* ix, const LayerDev& Ly, int64_t s, const Flagged
   launch_rerank_collected_fwd(ix->xw, ids, f, nf, row0, ix->dpad, ix->metric, inv, s, grid, cols, ncols, kCollectCap,
                               ix->M, Ly.fwd, Ly.fwd_d, over, err, st);
   CKL("collected rows");
-  int32_t nover = 0, herr = 0;
+  int32_t nover = 0;
   CK(cudaMemcpyAsync(&nover, over, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&herr, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (herr) throw Failure(HENN_ERR_TIMEOUT, "tensor-core tile pipeline wait timed out (code " + std::to_string(herr) + ")");
   if (nover > 0) {
     launch_exact_rows(ix->xw, ids, s, ix->dpad, ix->metric, inv, mode, over + 1, nover, ix->M, Ly.fwd, Ly.fwd_d, st);
     CKL("exact rows");
@@ -1171,11 +1170,14 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       CK(cudaMemcpyAsync(drows, rows.data(), sizeof(int32_t) * c, cudaMemcpyHostToDevice, st));
       const int32_t* lids = li >= 1 ? Ly.ids : nullptr;
       const int32_t KP = M <= 16 ? 32 : 64;
+      bool listed = false;
       if (tc_tiles_supported(dpad, KP) && ix->params.tiles != HENN_TILES_SIMT) {
         // tiles of the new rows against the whole layer (row j takes the
         // columns before position s0 + j), reranked and settled as a build's.
-        // The exact scan of every row that this replaces took 61.9 of the
-        // 72.9 ms that a 100,000 x 128 build and 20,000 insertions ran.
+        // Should they time out, the exact scan takes the rows: the arrays
+        // have grown, so the call has to go on.  The exact scan of every row
+        // that the tiles replace took 61.9 of the 72.9 ms that a 100,000 x
+        // 128 build and 20,000 insertions ran.
         const int32_t dk = round_up(dpad, 64);
         float* partial = sc.get<float>((size_t)mean_chunks(s1) * dpad);
         float* mean = sc.get<float>(dpad);
@@ -1205,14 +1207,13 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
         int32_t host[2] = {0, 0};
         CK(cudaMemcpyAsync(host, err, sizeof(host), cudaMemcpyDeviceToHost, st));
         CK(cudaStreamSynchronize(st));
-        if (host[0])
-          throw Failure(HENN_ERR_TIMEOUT, "tensor-core tile pipeline wait timed out (code " + std::to_string(host[0]) + ")");
-        if (host[1] > 0)
+        listed = host[0] == 0;
+        if (listed && host[1] > 0)
           settle_flagged(ix, Ly, s1, flagged, host[1], s0, 0, lids, nullptr, hi + (size_t)s0 * dk, lo + (size_t)s0 * dk,
                          norms + s0, hi, lo, norms, dk, sc, st);
-      } else {
-        launch_exact_rows(ix->xw, lids, s1, dpad, ix->metric, nullptr, 0, drows, (int32_t)c, M, Ly.fwd, Ly.fwd_d, st);
       }
+      if (!listed)
+        launch_exact_rows(ix->xw, lids, s1, dpad, ix->metric, nullptr, 0, drows, (int32_t)c, M, Ly.fwd, Ly.fwd_d, st);
       CKL("forward lists");
       // edge rule over the layer's updated forward lists
       int32_t* cnt = sc.get<int32_t>(s1);

@@ -899,18 +899,18 @@ __global__ void k_split_bf16(const float* __restrict__ x, int64_t s, int32_t dpa
 // Wait bound of the pipeline's mbarrier waits and the producer hold, from
 // the environment: HENN_TILE_SPIN_LIMIT (iterations of a try_wait that may
 // suspend up to 20 us; default and maximum kSpinLimit) and
-// HENN_TILE_HOLD_LOADS=1 (the producer issues no copy).  Together they make
-// the waits run out on purpose, with nothing in flight, so that tests can
-// check that a timeout comes back as an error status and leaves the
-// context usable.
-static void wait_policy(long long* spin_limit, int32_t* hold) {
+// HENN_TILE_HOLD_LOADS (1: the producer issues no copy, 2: only the
+// collecting pass's).  Together they make the waits run out on purpose, with
+// nothing in flight, so that tests can check what a timeout does and that it
+// leaves the context usable.
+static void wait_policy(bool collecting, long long* spin_limit, int32_t* hold) {
   *spin_limit = kSpinLimit;
   *hold = 0;
   if (const char* e = std::getenv("HENN_TILE_SPIN_LIMIT")) {
     const long long v = std::atoll(e);
     if (v >= 1 && v < kSpinLimit) *spin_limit = v;
   }
-  if (const char* e = std::getenv("HENN_TILE_HOLD_LOADS")) *hold = std::atoi(e) != 0;
+  if (const char* e = std::getenv("HENN_TILE_HOLD_LOADS")) *hold = std::atoi(e) == 2 ? collecting : std::atoi(e) != 0;
 }
 
 static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -1063,7 +1063,7 @@ cudaError_t launch_tile_lists_tc(const void* a_hi, const void* a_lo, const float
   rows.thr_out = thr;
   long long spin_limit;
   int32_t hold;
-  wait_policy(&spin_limit, &hold);
+  wait_policy(false, &spin_limit, &hold);
   v.fn<<<(unsigned)(nrb * splits), 64 + 32 * (eight ? 8 : 4), v.smem, st>>>(mah, mal, mbh, mbl, none, a_norms, b_norms, na, nb, dk / BK, mode,
                                                       out, nullptr, 0, nullptr, 0, splits, rows, err, spin_limit,
                                                       hold);
@@ -1101,7 +1101,7 @@ cudaError_t launch_tile_collect_tc(const void* a_hi, const void* a_lo, const flo
   rows.cap = cap;
   long long spin_limit;
   int32_t hold;
-  wait_policy(&spin_limit, &hold);
+  wait_policy(true, &spin_limit, &hold);
   v.fn<<<grid, 64 + 32 * 8, v.smem, st>>>(mah, mal, mbh, mbl, none, a_norms, b_norms, max_rows, nb, dk / BK, 4, nullptr,
                                           nullptr, 0, nullptr, 0, 1, rows, err, spin_limit, hold);
   return cudaGetLastError();
@@ -1163,7 +1163,7 @@ cudaError_t launch_tile_cross_tc(const void* a_hi, const void* a_lo, const float
   if (out_d && !make_store_map(&mo, out_d, na, ldo)) return cudaErrorInvalidValue;
   long long spin_limit;
   int32_t hold;
-  wait_policy(&spin_limit, &hold);
+  wait_policy(false, &spin_limit, &hold);
   // mode 3: eight epilogue warps (two per TMEM sub-partition); mode 2: four
   TileRows rows;
   std::memset(&rows, 0, sizeof(rows));

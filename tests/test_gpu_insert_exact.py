@@ -1,5 +1,6 @@
 """Insertions keep their exact lists where the tiles cannot give them (GPU):
-rows whose norms overflow FP32, and indexes made without tensor cores.
+rows whose norms overflow FP32, indexes made without tensor cores, and tile
+launches that time out; so do open rows of builds and exact k-NN.
 
 The tile pipeline is held by environment switches (its loads are not issued
 and its bounded waits run out), in a child process that no other test shares.
@@ -71,5 +72,57 @@ held("1")
 idx.insert(X[5000:])
 held("")
 same(idx, want)
+print("ok")
+""")
+
+
+def test_insertion_whose_tiles_time_out():
+    """The new rows are scanned; the index, whose arrays have grown, goes on."""
+    run_child("""
+want = H.Index(X[:5000], seed=2)
+want.insert(X[5000:])
+idx = H.Index(X[:5000], seed=2)
+held("1")
+idx.insert(X[5000:])
+held("")
+same(idx, want)
+assert idx.search(X[5000:], k=1, ef=64)[0][:, 0].tolist() == list(range(5000, 5200))
+idx.insert(X[:300])
+want.insert(X[:300])
+same(idx, want)
+print("ok")
+""")
+
+
+def test_collecting_passes_that_time_out():
+    """Tight groups far apart leave rows open; with only the collecting launches held these are scanned."""
+    run_child("""
+g = np.random.default_rng(3)
+X = (30.0 * g.standard_normal((90, 48)))[g.integers(90, size=6000)] + 0.02 * g.standard_normal((6000, 48))
+X = X.astype(np.float32)
+want = H.Index(X[:5800], seed=2)
+assert want.info()["uncertified_rows"] > 0
+held("2")
+idx = H.Index(X[:5800], seed=2)
+same(idx, want)
+idx.insert(X[5800:])
+held("")
+want.insert(X[5800:])
+same(idx, want)
+print("ok")
+""")
+
+
+def test_exact_knn_whose_tiles_time_out():
+    run_child("""
+import torch
+X = torch.from_numpy(X).cuda()
+for k in (10, 60):
+    want = H.exact_knn(X, X[:700] + 0.01, k)
+    for hold in "12":
+        held(hold)
+        got = H.exact_knn(X, X[:700] + 0.01, k)
+        held("")
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1]), (k, hold)
 print("ok")
 """)
