@@ -586,24 +586,32 @@ void settle_flagged(henn_index* ix, const LayerDev& Ly, int64_t s, const Flagged
                     int32_t mode, const int32_t* ids, const int32_t* inv, const void* hi, const void* lo,
                     const float* norms, const void* b_hi, const void* b_lo, const float* b_norms, int32_t dk,
                     Scratch& sc, cudaStream_t st) {
-  const int64_t nf = nflagged;
-  void* fhi = sc.get<uint16_t>((size_t)nf * dk);
-  void* flo = sc.get<uint16_t>((size_t)nf * dk);
-  float* fnorms = sc.get<float>(nf);
-  int32_t* lim = sc.get<int32_t>(nf);
-  int32_t* self = sc.get<int32_t>(nf);
-  const unsigned grid = tile_collect_grid(nf);
+  // a full wave of CTAs at a time: the buffers stay at 20 MiB of columns and
+  // 19,456 rows' planes (on 152 SMs) however many rows are open
+  const unsigned grid = tile_collect_grid(1);
+  const int64_t batch = std::min<int64_t>(nflagged, (int64_t)grid * kTileRows);
+  void* fhi = sc.get<uint16_t>((size_t)batch * dk);
+  void* flo = sc.get<uint16_t>((size_t)batch * dk);
+  float* fnorms = sc.get<float>(batch);
+  int32_t* lim = sc.get<int32_t>(batch);
+  int32_t* self = sc.get<int32_t>(batch);
   uint32_t* cols = sc.get<uint32_t>((size_t)grid * kTileRows * kCollectCap);
   int32_t* ncols = sc.get<int32_t>((size_t)grid * kTileRows);
-  int32_t* over = sc.get<int32_t>((size_t)nf + 2);  // their number, the rows, and the tile launch's error flag
-  int32_t* err = over + nf + 1;
+  int32_t* over = sc.get<int32_t>((size_t)nflagged + 2);  // their number, the rows, and the tile launches' error flag
+  int32_t* err = over + nflagged + 1;
   CK(cudaMemsetAsync(over, 0, sizeof(int32_t), st));
   CK(cudaMemsetAsync(err, 0, sizeof(int32_t), st));
-  launch_gather_flagged(f, nf, row0, mode == 0, mode == 1, s, hi, lo, norms, dk, fhi, flo, fnorms, lim, self, st);
-  CK(launch_tile_collect_tc(fhi, flo, fnorms, nf, b_hi, b_lo, b_norms, s, dk, lim, self, f.thr, f.count, grid, cols,
-                            ncols, kCollectCap, err, st));
-  launch_rerank_collected_fwd(ix->xw, ids, f, nf, row0, ix->dpad, ix->metric, inv, s, grid, cols, ncols, kCollectCap,
-                              ix->M, Ly.fwd, Ly.fwd_d, over, err, st);
+  for (int64_t at = 0; at < nflagged; at += batch) {
+    const int64_t nf = std::min<int64_t>(batch, nflagged - at);
+    FlaggedRows part = f;  // *count, all of them, is at least nf: each launch takes nf
+    part.rows += at;
+    part.thr += at;
+    launch_gather_flagged(part, nf, row0, mode == 0, mode == 1, s, hi, lo, norms, dk, fhi, flo, fnorms, lim, self, st);
+    CK(launch_tile_collect_tc(fhi, flo, fnorms, nf, b_hi, b_lo, b_norms, s, dk, lim, self, part.thr, part.count, grid,
+                              cols, ncols, kCollectCap, err, st));
+    launch_rerank_collected_fwd(ix->xw, ids, part, nf, row0, ix->dpad, ix->metric, inv, s, grid, cols, ncols,
+                                kCollectCap, ix->M, Ly.fwd, Ly.fwd_d, over, err, st);
+  }
   CKL("collected rows");
   int32_t nover = 0;
   CK(cudaMemcpyAsync(&nover, over, sizeof(int32_t), cudaMemcpyDeviceToHost, st));

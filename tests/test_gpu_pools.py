@@ -135,3 +135,14 @@ def test_inserted_forward_lists(kind, n, add, d, metric):
             dist = 0.5 * dist
         check_dists(fwd_d[r], dist.topk(16, largest=False, sorted=True).values, d, metric == H.ANGULAR)
         assert len(set(fwd[r].tolist())) == 16
+
+
+@pytest.mark.parametrize("graph", [H.GRAPH_NSW, H.GRAPH_KNN])
+def test_open_rows_in_several_batches(graph):
+    """More open rows than one collecting launch takes (128 per SM)."""
+    X = points("groups", 45_000, 40, 11)
+    a = H.Index(X, graph=graph, seed=3)
+    b = H.Index(X, graph=graph, seed=3, tiles=H.TILES_SIMT)
+    assert a.info()["uncertified_rows"] > 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    la, lb = a.layer(0), b.layer(0)
+    assert all(np.array_equal(la[key], lb[key]) for key in la)
