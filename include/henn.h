@@ -157,9 +157,11 @@ henn_status henn_build(const float* X, int64_t n, int32_t d, int32_t x_on_device
  * position), points of one call being inserted one after another; the
  * layer's adjacency is then the edge rule over the updated forward lists
  * (the rows of its forward neighbours gain it as a reverse link).  Device
- * arrays grow by doubling.  NSW graphs only (HENN_ERR_UNSUPPORTED for kNN
- * graphs, where earlier points' own lists would change).  Synchronises
- * `stream` before returning.  Not safe concurrently with searches on idx;
+ * arrays grow by doubling.  Scratch of 4 bytes a value of the layer is taken
+ * for the call where it fits (M <= 16); where it does not, the new rows are
+ * scanned without it, more slowly.  NSW graphs only (HENN_ERR_UNSUPPORTED
+ * for kNN graphs, where earlier points' own lists would change).
+ * Synchronises `stream` before returning.  Not safe concurrently with searches on idx;
  * servers made from idx before the call still point at the old arrays and
  * must be destroyed first.
  */

@@ -1054,6 +1054,60 @@ T* regrow(henn_index* ix, T* old, size_t used, size_t cap, cudaStream_t st) {
   return p;
 }
 
+// Forward lists of the rows s0 .. s0 + c - 1 of a layer (drows: their
+// numbers), each over the rows before it: tiles of the new rows against the
+// whole layer, reranked and settled as a build's.  The exact scan of every row
+// that they replace took 61.9 of the 72.9 ms that a 100,000 x 128 build and
+// 20,000 insertions ran.  False if the tiles timed out or their scratch (4
+// bytes a value of the layer and 256 a new row and split) does not fit: the
+// arrays have grown, so the insertion has to go on, with the scan, which needs
+// none.
+bool insert_lists(henn_index* ix, const LayerDev& Ly, const int32_t* lids, int64_t s0, int64_t c, const int32_t* drows,
+                  cudaStream_t st) {
+  const int64_t s1 = s0 + c;
+  const int32_t dpad = ix->dpad, M = ix->M, KP = 32, dk = round_up(dpad, 64);
+  Scratch sc(st, library_pool(ix->device));
+  try {
+    float* partial = sc.get<float>((size_t)mean_chunks(s1) * dpad);
+    float* mean = sc.get<float>(dpad);
+    uint16_t* hi = sc.get<uint16_t>((size_t)s1 * dk);
+    uint16_t* lo = sc.get<uint16_t>((size_t)s1 * dk);
+    float* norms = sc.get<float>(s1);
+    float* nmax = sc.get<float>(1);
+    const int32_t splits = tile_list_splits(c, s1, false);
+    uint64_t* lists = sc.get<uint64_t>((size_t)splits * c * KP);
+    uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)c * KP) : lists;
+    int32_t* err = sc.get<int32_t>(2);  // the tile launch's error flag, the flagged rows' number
+    float* thr = sc.get<float>(c);
+    float* lthr = splits > 1 ? sc.get<float>((size_t)splits * c) : thr;
+    FlaggedRows flagged;
+    flagged.count = err + 1;
+    flagged.rows = sc.get<int32_t>(c);
+    flagged.thr = sc.get<float>(c);
+    launch_layer_mean(ix->xw, lids, s1, dpad, partial, mean, st);
+    launch_order_split(ix->xw, lids, s1, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, norms, nmax, st);
+    CK(cudaMemsetAsync(err, 0, 2 * sizeof(int32_t), st));
+    CK(launch_tile_lists_tc(hi + (size_t)s0 * dk, lo + (size_t)s0 * dk, norms + s0, c, hi, lo, norms, s1, dk, 2, drows,
+                            splits, lists, lthr, err, st));
+    if (splits > 1) launch_merge_lists(lists, lthr, c, splits, KP, cand, thr, st);
+    launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, thr, s1, true, true, KP, M, norms + s0,
+                      nmax, tc_tile_unit_error(dk), Ly.fwd, Ly.fwd_d, flagged, st);
+    CKL("rerank");
+    int32_t host[2] = {0, 0};
+    CK(cudaMemcpyAsync(host, err, sizeof(host), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    if (host[0]) return false;
+    if (host[1] > 0)
+      settle_flagged(ix, Ly, s1, flagged, host[1], s0, 0, lids, nullptr, hi + (size_t)s0 * dk, lo + (size_t)s0 * dk,
+                     norms + s0, hi, lo, norms, dk, sc, st);
+    return true;
+  } catch (const Failure& f) {
+    if (f.status != HENN_ERR_OOM) throw;
+    cudaGetLastError();  // the failed allocation's
+    return false;
+  }
+}
+
 }  // namespace
 
 extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new, int32_t x_on_device, void* stream) {
@@ -1177,49 +1231,9 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       int32_t* drows = sc.get<int32_t>(c);
       CK(cudaMemcpyAsync(drows, rows.data(), sizeof(int32_t) * c, cudaMemcpyHostToDevice, st));
       const int32_t* lids = li >= 1 ? Ly.ids : nullptr;
-      const int32_t KP = M <= 16 ? 32 : 64;
-      bool listed = false;
-      if (tc_tiles_supported(dpad, KP) && ix->params.tiles != HENN_TILES_SIMT) {
-        // tiles of the new rows against the whole layer (row j takes the
-        // columns before position s0 + j), reranked and settled as a build's.
-        // Should they time out, the exact scan takes the rows: the arrays
-        // have grown, so the call has to go on.  The exact scan of every row
-        // that the tiles replace took 61.9 of the 72.9 ms that a 100,000 x
-        // 128 build and 20,000 insertions ran.
-        const int32_t dk = round_up(dpad, 64);
-        float* partial = sc.get<float>((size_t)mean_chunks(s1) * dpad);
-        float* mean = sc.get<float>(dpad);
-        launch_layer_mean(ix->xw, lids, s1, dpad, partial, mean, st);
-        uint16_t* hi = sc.get<uint16_t>((size_t)s1 * dk);
-        uint16_t* lo = sc.get<uint16_t>((size_t)s1 * dk);
-        float* norms = sc.get<float>(s1);
-        float* nmax = sc.get<float>(1);
-        launch_order_split(ix->xw, lids, s1, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, norms, nmax, st);
-        const int32_t splits = tile_list_splits(c, s1, false);
-        uint64_t* lists = sc.get<uint64_t>((size_t)splits * c * KP);
-        uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)c * KP) : lists;
-        int32_t* err = sc.get<int32_t>(2);  // the tile launch's error flag, the flagged rows' number
-        CK(cudaMemsetAsync(err, 0, 2 * sizeof(int32_t), st));
-        float* thr = sc.get<float>(c);
-        float* lthr = splits > 1 ? sc.get<float>((size_t)splits * c) : thr;
-        CK(launch_tile_lists_tc(hi + (size_t)s0 * dk, lo + (size_t)s0 * dk, norms + s0, c, hi, lo, norms, s1, dk, 2,
-                                drows, splits, lists, lthr, err, st));
-        if (splits > 1) launch_merge_lists(lists, lthr, c, splits, KP, cand, thr, st);
-        FlaggedRows flagged;
-        flagged.count = err + 1;
-        flagged.rows = sc.get<int32_t>(c);
-        flagged.thr = sc.get<float>(c);
-        launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, thr, s1, true, true, KP, M, norms + s0,
-                          nmax, tc_tile_unit_error(dk), Ly.fwd, Ly.fwd_d, flagged, st);
-        CKL("rerank");
-        int32_t host[2] = {0, 0};
-        CK(cudaMemcpyAsync(host, err, sizeof(host), cudaMemcpyDeviceToHost, st));
-        CK(cudaStreamSynchronize(st));
-        listed = host[0] == 0;
-        if (listed && host[1] > 0)
-          settle_flagged(ix, Ly, s1, flagged, host[1], s0, 0, lids, nullptr, hi + (size_t)s0 * dk, lo + (size_t)s0 * dk,
-                         norms + s0, hi, lo, norms, dk, sc, st);
-      }
+      // on the tiles where they apply, else (or should they not do) scanned
+      const bool listed = tc_tiles_supported(dpad, M <= 16 ? 32 : 64) && ix->params.tiles != HENN_TILES_SIMT &&
+                          insert_lists(ix, Ly, lids, s0, c, drows, st);
       if (!listed)
         launch_exact_rows(ix->xw, lids, s1, dpad, ix->metric, nullptr, 0, drows, (int32_t)c, M, Ly.fwd, Ly.fwd_d, st);
       CKL("forward lists");
