@@ -75,6 +75,7 @@ struct DevicePool {
   std::mutex mu;
   cudaMemPool_t pool = nullptr;
   int64_t indexes = 0;  // alive on this device
+  std::vector<void*> parked;  // blocks of freed indexes that could not be waited for yet
 };
 
 DevicePool& device_pool(int device) {
@@ -100,6 +101,15 @@ cudaMemPool_t library_pool(int device) {
   }
   return p.pool;
 }
+
+// Lets this thread's cudaMalloc and cudaFree through while a stream is being
+// captured, here or in another thread: in the default (global) capture mode
+// they are refused, and the attempt spoils the capture.
+struct BesideCaptures {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 
 // Stream-ordered scratch allocation, released when the owner goes out of
 // scope (also on failure).
@@ -272,9 +282,31 @@ struct henn_index {
   // returns, so that every stream may use the memory afterwards.
   cudaStream_t mem_stream = nullptr;
   bool drained = false;  // the operation in progress has waited for the device
+  // Blocks of the index go back to the pool by cudaFree, which does not wait
+  // for pool memory, and searches on any stream may still read them.  Freeing
+  // a cudaMalloc'ed block does wait for the device (cudaDeviceSynchronize does
+  // too, but spoils any capture in progress, a build's in another thread for
+  // instance), so an index holds two small ones, gates, and frees one before
+  // its blocks: the operation in progress may use one up (begin makes up for
+  // it), and one is left for the destructor.  No allocation is needed to free.
+  std::vector<void*> gates;
   void begin(cudaStream_t st) {
     mem_stream = st;
     drained = false;
+    BesideCaptures any;
+    while (gates.size() < 2) {
+      void* p = nullptr;
+      CK(cudaMalloc(&p, 16));
+      gates.push_back(p);
+    }
+  }
+  // Waits for the device; false if it could not.
+  bool drain() {
+    BesideCaptures any;
+    if (gates.empty()) return cudaDeviceSynchronize() == cudaSuccess;
+    if (cudaFree(gates.back()) != cudaSuccess) return cudaDeviceSynchronize() == cudaSuccess;
+    gates.pop_back();
+    return true;
   }
   template <typename T>
   T* alloc(size_t count) {
@@ -289,22 +321,16 @@ struct henn_index {
     bytes += (int64_t)b;
     return static_cast<T*>(p);
   }
-  // Waits for the device (searches on other streams may still read the
-  // index's memory) the way freeing a cudaMalloc'ed block does: also while
-  // another thread captures a stream, when cudaDeviceSynchronize is refused.
-  // cudaFree of pool memory does not wait.
-  static void drain() {
-    void* p = nullptr;
-    if (cudaMalloc(&p, 16) == cudaSuccess) cudaFree(p);
-  }
   // frees one allocation made by alloc(): nothing may run on the index beside
-  // the operation in progress, so waiting once covers what ran before it
+  // the operation in progress, so waiting once covers what ran before it; a
+  // block that cannot be waited for stays the index's until it is freed
   void release(void* p) {
     if (!p) return;
     for (size_t i = 0; i < allocs.size(); ++i)
       if (allocs[i] == p) {
-        if (!drained) drain();
-        drained = true;
+        if (!drained) drained = drain();
+        if (!drained) return;
+        BesideCaptures any;
         cudaFree(p);
         allocs.erase(allocs.begin() + (long)i);
         return;
@@ -372,21 +398,23 @@ struct henn_index {
     int current = device;  // the caller's device may be another
     cudaGetDevice(&current);
     if (current != device) cudaSetDevice(device);
+    BesideCaptures any;
+    const bool idle = drain();
     drop_entry_ops();
-    if (pool) {
-      cudaDeviceSynchronize();
-      cudaMemPoolDestroy(pool);
-    }
-    drain();
+    if (pool) cudaMemPoolDestroy(pool);  // (released once its last frees have run)
     for (cudaEvent_t e : tev)
       if (e) cudaEventDestroy(e);
     for (cudaStream_t t : side) cudaStreamDestroy(t);
-    for (void* p : allocs) cudaFree(p);
-    if (device < 64) {
-      DevicePool& dp = device_pool(device);
-      std::lock_guard<std::mutex> lk(dp.mu);
-      if (--dp.indexes == 0 && dp.pool) cudaMemPoolTrimTo(dp.pool, kPoolIdle);
+    for (void* p : gates) cudaFree(p);
+    DevicePool& dp = device_pool(device);
+    std::lock_guard<std::mutex> lk(dp.mu);
+    if (idle) {
+      allocs.insert(allocs.end(), dp.parked.begin(), dp.parked.end());
+      dp.parked.clear();
     }
+    for (void* p : allocs)
+      if (!idle || cudaFree(p) != cudaSuccess) dp.parked.push_back(p);
+    if (device < 64 && --dp.indexes == 0 && dp.pool) cudaMemPoolTrimTo(dp.pool, kPoolIdle);
     if (current != device) cudaSetDevice(current);
   }
 };

@@ -1,4 +1,8 @@
-"""Device memory of indexes (GPU): calls whose scratch does not fit."""
+"""Device memory of indexes (GPU): calls whose scratch does not fit, and freeing
+with searches in flight, on a full device and beside a capture."""
+import ctypes
+import threading
+
 import numpy as np
 import pytest
 
@@ -32,3 +36,104 @@ def test_insertion_into_a_full_device():
     assert all(np.array_equal(la[key], lb[key]) for key in la)
     for x, y in zip(a.search(new, k=10, ef=64), b.search(new, k=10, ef=64)):
         assert np.array_equal(x, y)
+
+
+def searches_in_flight(idx, Q, stream):
+    """Enough of them that the stream is still busy when this returns."""
+    with torch.cuda.stream(stream):
+        out = [idx.search(Q, k=10, ef=512, ef_upper=32, stream=stream)[:2] for _ in range(40)]
+    assert not stream.query()
+    return out
+
+
+def test_close_waits_for_searches_in_flight():
+    X, Q = rand(100_000, 64, 4), rand(10_000, 64, 5)
+    idx, other = H.Index(X, seed=1), H.Index(X[:1000], seed=1)
+    want = idx.search(Q, k=10, ef=512, ef_upper=32)[:2]
+    stream = torch.cuda.Stream()
+    out = searches_in_flight(idx, Q, stream)
+    idx.close()
+    assert stream.query()
+    other.close()
+    for ids, dd in out:
+        assert torch.equal(ids, want[0]) and torch.equal(dd, want[1])
+
+
+def test_close_on_a_full_device():
+    """Not a byte left to allocate: freeing waits all the same."""
+    X, Q = rand(100_000, 64, 4), rand(10_000, 64, 5)
+    idx = H.Index(X, seed=1)
+    want = idx.search(Q, k=10, ef=512, ef_upper=32)[:2]
+    stream = torch.cuda.Stream()
+    out = searches_in_flight(idx, Q, stream)  # (their buffers come first)
+    torch.cuda.synchronize()
+    del out
+    cudart = ctypes.CDLL("libcudart.so." + torch.version.cuda.split(".")[0])
+    held, size = [], 1 << 36
+    out = searches_in_flight(idx, Q, stream)
+    while size >= 512:
+        p = ctypes.c_void_p()
+        if cudart.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(size)) == 0:
+            held.append(p)
+        else:
+            size //= 2
+    cudart.cudaGetLastError()
+    try:
+        idx.close()
+        assert stream.query()
+    finally:
+        for p in held:
+            cudart.cudaFree(p)
+    for ids, dd in out:
+        assert torch.equal(ids, want[0]) and torch.equal(dd, want[1])
+
+
+@pytest.mark.parametrize("other_thread", [False, True])
+def test_close_beside_a_capture(other_thread):
+    """A capture in progress, in the default mode that other threads' calls can spoil, stays whole."""
+    X = rand(3000, 32, 6)
+    idx = H.Index(X, seed=1)
+    idx.search(X[:100], k=10)
+    g, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    y = torch.zeros_like(X)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=stream):
+        y.copy_(X)
+        y.mul_(2.0)
+        if other_thread:
+            t = threading.Thread(target=idx.close)
+            t.start()
+            t.join()
+        else:
+            idx.close()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, 2.0 * X)
+
+
+def test_threads_close_searched_indexes_beside_builds():
+    """Builds capture their steps; another thread's close must not spoil them."""
+    X = [rand(4000 + 300 * t, 48, 10 + t) for t in range(4)]
+    indexes = [H.Index(x, seed=2) for x in X]
+    want = [idx.search(x[:200], k=10)[0] for x, idx in zip(X, indexes)]
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(t):
+        try:
+            stream = torch.cuda.Stream()
+            for _ in range(8):
+                idx = H.Index(X[t], seed=2, stream=stream)
+                got = idx.search(X[t][:200], k=10, stream=stream)[0]
+                idx.close()
+                stream.synchronize()
+                assert torch.equal(got, want[t])
+        except Exception as e:  # reported below
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
