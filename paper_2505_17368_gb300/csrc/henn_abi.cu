@@ -1041,10 +1041,16 @@ extern "C" henn_status henn_delete(henn_index* ix, const int64_t* ids, int64_t n
     require(ids != nullptr, "ids is NULL");
     for (int64_t i = 0; i < n; ++i) require(ids[i] >= 0 && ids[i] < ix->n, "id out of range");
     cudaStream_t st = (cudaStream_t)stream;
+    // on a capturing stream an allocation would belong to the graph
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone)
+      throw Failure(HENN_ERR_CUDA, "henn_delete on a stream that is being captured");
     ix->begin(st);
     if (!ix->dead) {
-      ix->dead = ix->alloc<uint8_t>((size_t)ix->cap_n);
-      CK(cudaMemsetAsync(ix->dead, 0, (size_t)ix->cap_n, st));
+      uint8_t* flags = ix->alloc<uint8_t>((size_t)ix->cap_n);
+      CK(cudaMemsetAsync(flags, 0, (size_t)ix->cap_n, st));
+      ix->dead = flags;
     }
     Scratch sc(st);
     int64_t* d_ids = sc.get<int64_t>((size_t)n);

@@ -1,5 +1,6 @@
 """Device memory of indexes (GPU): calls whose scratch does not fit, and freeing
-with searches in flight, on a full device and beside a capture."""
+with searches in flight, on a full device and beside a capture, and deletion
+on a capturing stream."""
 import ctypes
 import threading
 
@@ -137,3 +138,22 @@ def test_threads_close_searched_indexes_beside_builds():
     for t in threads:
         t.join()
     assert not failed, failed
+
+
+def test_delete_on_a_capturing_stream_is_refused():
+    """Before anything has changed: the index searches on, and the capture stays whole."""
+    X = rand(3000, 32, 7)
+    idx = H.Index(X, seed=1)
+    want = idx.search(X[:100], k=10)[0]
+    g, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    y = torch.zeros_like(X)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=stream):
+        y.copy_(X)
+        with pytest.raises(H.HennError):
+            idx.delete([0, 1, 2], stream=stream)
+    g.replay()
+    assert torch.equal(idx.search(X[:100], k=10)[0], want)
+    idx.delete([0, 1, 2])
+    got = idx.search(X[:100], k=10)[0]
+    assert not torch.isin(got, torch.arange(3, device="cuda")).any() and torch.equal(y, X)
