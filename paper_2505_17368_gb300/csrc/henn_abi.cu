@@ -39,6 +39,7 @@ struct Failure : std::exception {
 
 void check(cudaError_t e, const char* what, int line) {
   if (e == cudaSuccess) return;
+  cudaGetLastError();  // reported here: a later call that asks for launch errors must not find it
   henn_status s = (e == cudaErrorMemoryAllocation) ? HENN_ERR_OOM : HENN_ERR_CUDA;
   throw Failure(s, std::string(what) + " (line " + std::to_string(line) + "): " + cudaGetErrorString(e));
 }
@@ -918,9 +919,8 @@ extern "C" void henn_free(henn_index* idx) { delete idx; }
 
 namespace {
 
-// The search-side layer table of ix (device), rewritten from ix->layers;
-// reallocated when the number of layers changed.
-void upload_layer_table(henn_index* ix, cudaStream_t st) {
+// The search-side layer table of ix (device) from ix->layers.
+void write_layer_table(henn_index* ix, cudaStream_t st) {
   std::vector<SearchLayer> h(ix->L + 1);
   for (int32_t li = 0; li <= ix->L; ++li) {
     h[li].adj = ix->layers[li].adj;
@@ -929,10 +929,15 @@ void upload_layer_table(henn_index* ix, cudaStream_t st) {
     h[li].down = ix->layers[li].down;
     h[li].size = ix->layers[li].size;
   }
-  ix->release(ix->d_layers);
-  ix->d_layers = ix->alloc<SearchLayer>(h.size());
   CK(cudaMemcpyAsync(ix->d_layers, h.data(), sizeof(SearchLayer) * h.size(), cudaMemcpyHostToDevice, st));
   CK(cudaStreamSynchronize(st));
+}
+
+// The same after the number of layers changed.
+void upload_layer_table(henn_index* ix, cudaStream_t st) {
+  ix->release(ix->d_layers);
+  ix->d_layers = ix->alloc<SearchLayer>((size_t)ix->L + 1);
+  write_layer_table(ix, st);
 }
 
 // Layer i resampled from the live points of layer i - 1 (global ids
@@ -1171,31 +1176,6 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
     const int32_t dpad = ix->dpad, d = ix->d, M = ix->M;
     const bool angular = ix->metric == HENN_ANGULAR;
 
-    // ---- vectors (FP32 master copy, unit rows for angular)
-    if (n1 > ix->cap_n) {
-      const int64_t cap = std::max(n1, 2 * ix->cap_n);
-      const bool aliased = ix->xw == ix->x32;
-      ix->x32 = regrow(ix, ix->x32, (size_t)n0 * dpad, (size_t)cap * dpad, st);
-      if (angular) {
-        ix->xw = regrow(ix, ix->xw, (size_t)n0 * dpad, (size_t)cap * dpad, st);
-        ix->inv_norm = regrow(ix, ix->inv_norm, (size_t)n0, (size_t)cap, st);
-      } else if (aliased) {
-        ix->xw = ix->x32;
-      }
-      if (ix->dead) ix->dead = regrow(ix, ix->dead, (size_t)n0, (size_t)cap, st);
-      ix->cap_n = cap;
-    }
-    if (ix->dead) CK(cudaMemsetAsync(ix->dead + n0, 0, (size_t)n_new, st));
-    float* xrow = ix->x32 + (size_t)n0 * dpad;
-    CK(cudaMemsetAsync(xrow, 0, sizeof(float) * (size_t)n_new * dpad, st));
-    CK(cudaMemcpy2DAsync(xrow, sizeof(float) * dpad, X, sizeof(float) * d, sizeof(float) * d, (size_t)n_new,
-                         x_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
-    if (angular) {
-      launch_inv_norms(xrow, n_new, dpad, ix->inv_norm + n0, st);
-      launch_normalise(xrow, ix->inv_norm + n0, n_new, dpad, ix->xw + (size_t)n0 * dpad, st);
-      CKL("normalise");
-    }
-
     // ---- layers each new point joins (App. C, Insert)
     std::vector<std::vector<int32_t>> add(ix->L + 1);
     for (int64_t j = 0; j < n_new; ++j) {
@@ -1207,14 +1187,30 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       }
     }
 
-    // ---- per layer: append members, their traversal rows, forward lists, edge rule
-    for (int32_t li = 0; li <= ix->L; ++li) {
-      LayerDev& Ly = ix->layers[li];
-      const int64_t s0 = Ly.size, c = (int64_t)add[li].size(), s1 = s0 + c;
-      if (c == 0) continue;
+    // ---- room for them: every array grows and the scratch is taken before
+    // anything else changes, so that a call that runs out of memory leaves the
+    // index as it was (the table on the device pointing at its arrays)
+    auto grow = [&] {
+      if (n1 > ix->cap_n) {
+        const int64_t cap = std::max(n1, 2 * ix->cap_n);
+        const bool aliased = ix->xw == ix->x32;
+        ix->x32 = regrow(ix, ix->x32, (size_t)n0 * dpad, (size_t)cap * dpad, st);
+        if (angular) {
+          ix->xw = regrow(ix, ix->xw, (size_t)n0 * dpad, (size_t)cap * dpad, st);
+          ix->inv_norm = regrow(ix, ix->inv_norm, (size_t)n0, (size_t)cap, st);
+        } else if (aliased) {
+          ix->xw = ix->x32;
+        }
+        if (ix->dead) ix->dead = regrow(ix, ix->dead, (size_t)n0, (size_t)cap, st);
+        ix->cap_n = cap;
+      }
       const size_t elem = ix->storage == HENN_BF16 ? 2 : (ix->storage == HENN_FP8E4M3 ? 1 : 4);
-      const bool vec_aliased = li == 0 && ix->storage == HENN_F32;
-      if (s1 > Ly.cap) {
+      for (int32_t li = 0; li <= ix->L; ++li) {
+        LayerDev& Ly = ix->layers[li];
+        const int64_t s0 = Ly.size, s1 = s0 + (int64_t)add[li].size();
+        const bool vec_aliased = li == 0 && ix->storage == HENN_F32;
+        if (vec_aliased) Ly.vec = ix->xw;
+        if (s1 <= Ly.cap) continue;
         const int64_t cap = std::max(s1, 2 * Ly.cap);
         if (li >= 1) {
           Ly.ids = regrow(ix, Ly.ids, (size_t)s0, (size_t)cap, st);
@@ -1228,8 +1224,43 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
         if (ix->storage == HENN_FP8E4M3) Ly.vscale = regrow(ix, Ly.vscale, (size_t)s0, (size_t)cap, st);
         Ly.cap = cap;
       }
-      if (vec_aliased) Ly.vec = ix->xw;
-      Scratch sc(st, library_pool(ix->device));
+    };
+    try {
+      grow();
+    } catch (...) {
+      if (ix->storage == HENN_F32) ix->layers[0].vec = ix->xw;
+      write_layer_table(ix, st);
+      throw;
+    }
+    write_layer_table(ix, st);
+    Scratch sc(st, library_pool(ix->device));
+    const int64_t s_max = ix->layers[0].size + n_new;  // layer 0 holds every point
+    const int64_t c_upper = ix->L >= 1 ? (int64_t)add[1].size() : 0;
+    float* gathered = ix->storage != HENN_F32 && c_upper > 0 ? sc.get<float>((size_t)c_upper * dpad) : nullptr;
+    int32_t* drows = sc.get<int32_t>(n_new);
+    int32_t* cnt = sc.get<int32_t>(s_max);
+    int32_t* fill = sc.get<int32_t>(s_max);
+    int64_t* off = sc.get<int64_t>((size_t)s_max + 1);
+    int64_t* tiles = sc.get<int64_t>((size_t)scan_tiles(s_max) + 1);
+    uint64_t* rev = sc.get<uint64_t>((size_t)s_max * M);
+
+    // ---- vectors (FP32 master copy, unit rows for angular)
+    if (ix->dead) CK(cudaMemsetAsync(ix->dead + n0, 0, (size_t)n_new, st));
+    float* xrow = ix->x32 + (size_t)n0 * dpad;
+    CK(cudaMemsetAsync(xrow, 0, sizeof(float) * (size_t)n_new * dpad, st));
+    CK(cudaMemcpy2DAsync(xrow, sizeof(float) * dpad, X, sizeof(float) * d, sizeof(float) * d, (size_t)n_new,
+                         x_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, st));
+    if (angular) {
+      launch_inv_norms(xrow, n_new, dpad, ix->inv_norm + n0, st);
+      launch_normalise(xrow, ix->inv_norm + n0, n_new, dpad, ix->xw + (size_t)n0 * dpad, st);
+      CKL("normalise");
+    }
+
+    // ---- per layer: append members, their traversal rows, forward lists, edge rule
+    for (int32_t li = 0; li <= ix->L; ++li) {
+      LayerDev& Ly = ix->layers[li];
+      const int64_t s0 = Ly.size, c = (int64_t)add[li].size(), s1 = s0 + c;
+      if (c == 0) continue;
       if (li >= 1) {
         // global ids, and positions in the layer below (appended there in this call)
         std::vector<int32_t> dn(c);
@@ -1247,8 +1278,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       // traversal rows of the new members
       const float* src = ix->xw + (size_t)n0 * dpad;  // layer 0: the appended rows in order
       if (li >= 1) {
-        float* g = ix->storage == HENN_F32 ? static_cast<float*>(Ly.vec) + (size_t)s0 * dpad
-                                           : sc.get<float>((size_t)c * dpad);
+        float* g = ix->storage == HENN_F32 ? static_cast<float*>(Ly.vec) + (size_t)s0 * dpad : gathered;
         launch_gather_rows32(ix->xw, Ly.ids + s0, c, dpad, g, st);
         src = g;
       }
@@ -1262,7 +1292,6 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       // forward lists: the new rows, inserted last in this order
       std::vector<int32_t> rows(c);
       for (int64_t j = 0; j < c; ++j) rows[j] = (int32_t)(s0 + j);
-      int32_t* drows = sc.get<int32_t>(c);
       CK(cudaMemcpyAsync(drows, rows.data(), sizeof(int32_t) * c, cudaMemcpyHostToDevice, st));
       const int32_t* lids = li >= 1 ? Ly.ids : nullptr;
       // on the tiles where they apply, else (or should they not do) scanned
@@ -1272,11 +1301,6 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
         launch_exact_rows(ix->xw, lids, s1, dpad, ix->metric, nullptr, 0, drows, (int32_t)c, M, Ly.fwd, Ly.fwd_d, st);
       CKL("forward lists");
       // edge rule over the layer's updated forward lists
-      int32_t* cnt = sc.get<int32_t>(s1);
-      int32_t* fill = sc.get<int32_t>(s1);
-      int64_t* off = sc.get<int64_t>((size_t)s1 + 1);
-      int64_t* tiles = sc.get<int64_t>((size_t)scan_tiles(s1) + 1);
-      uint64_t* rev = sc.get<uint64_t>((size_t)s1 * M);
       CK(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * s1, st));
       CK(cudaMemsetAsync(fill, 0, sizeof(int32_t) * s1, st));
       launch_rev_count(Ly.fwd, s1, M, cnt, st);
@@ -1288,18 +1312,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       Ly.size = s1;
     }
     ix->n = n1;
-
-    // ---- search-side layer table
-    std::vector<SearchLayer> h(ix->L + 1);
-    for (int32_t li = 0; li <= ix->L; ++li) {
-      h[li].adj = ix->layers[li].adj;
-      h[li].vec = ix->layers[li].vec;
-      h[li].scale = ix->layers[li].vscale;
-      h[li].down = ix->layers[li].down;
-      h[li].size = ix->layers[li].size;
-    }
-    CK(cudaMemcpyAsync(ix->d_layers, h.data(), sizeof(SearchLayer) * h.size(), cudaMemcpyHostToDevice, st));
-    CK(cudaStreamSynchronize(st));
+    write_layer_table(ix, st);
     return HENN_OK;
   } catch (const Failure& f) {
     g_error = f.msg;

@@ -157,3 +157,33 @@ def test_delete_on_a_capturing_stream_is_refused():
     idx.delete([0, 1, 2])
     got = idx.search(X[:100], k=10)[0]
     assert not torch.isin(got, torch.arange(3, device="cuda")).any() and torch.equal(y, X)
+
+
+def test_insertion_that_runs_out_of_memory():
+    """Whichever array does not fit any more, the index answers as before and takes the rows once there is room."""
+    X, new = rand(300_000, 512, 8), rand(20_000, 512, 9).cpu().numpy()
+    Q = X[:500] + 0.01
+    want = H.Index(X, storage=H.BF16, seed=3)
+    want.insert(new)
+    want = want.layer(0)
+    refused = 0
+    for left in (100, 1300, 1400, 1600, 2000, 2600):
+        idx = H.Index(X, storage=H.BF16, seed=3)
+        before = [t.clone() for t in idx.search(Q, k=10)[:2]]
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        full = torch.empty(torch.cuda.mem_get_info()[0] - (left << 20), dtype=torch.uint8, device="cuda")
+        try:
+            idx.insert(new)
+        except H.HennError as e:
+            assert e.status == 2
+            refused += 1
+        del full
+        torch.cuda.empty_cache()
+        if idx.n == 300_000:
+            assert all(torch.equal(a, b) for a, b in zip(idx.search(Q, k=10)[:2], before))
+            idx.insert(new)
+        got = idx.layer(0)
+        assert all(np.array_equal(got[key], want[key]) for key in want)
+        idx.close()
+    assert refused >= 1
