@@ -1496,8 +1496,9 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
     // warps per block of a launch of n queries with a beam capacity
     auto block_warps = [&](int64_t n, int cap, int bits) {
       if (sp.warps_per_block > 0) return (int)sp.warps_per_block;
-      return team > 1 ? kSearchWarps : search_block_warps(idx->device, n, search_warp_smem(cap, bits, idx->dpad),
-                                                              idx->storage, idx->dpad);
+      return team > 1 ? kSearchWarps
+                      : search_block_warps(idx->device, n, search_warp_smem(cap, bits, idx->dpad), idx->storage,
+                                           idx->dpad, search_is_brief(cap, sp.ef_upper));
     };
     const int warps = block_warps(nq, ef_cap, hb);
     require(warps >= 1 && warps <= kSearchWarps, "warps_per_block must be in [1, 4]");

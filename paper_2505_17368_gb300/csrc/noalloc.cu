@@ -125,7 +125,8 @@ extern "C" henn_status henn_search_host_noalloc(const henn_index* idx, const flo
   a.stats = nullptr;
   a.counter = counter;
 
-  const int warps = search_block_warps(device, nq, search_warp_smem(ef_cap, hb, a.dpad), a.storage, a.dpad);
+  const int warps = search_block_warps(device, nq, search_warp_smem(ef_cap, hb, a.dpad), a.storage, a.dpad,
+                                       search_is_brief(ef_cap, ef_upper));
   const size_t smem = search_warp_smem(ef_cap, hb, a.dpad) * warps;
   int grid = 0;
   cudaError_t e = search_persistent_grid(device, warps, smem, &grid);

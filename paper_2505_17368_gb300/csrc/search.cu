@@ -1081,11 +1081,22 @@ constexpr int most_in_flight() {
   return std::is_same<VT, float>::value ? kHalf : kFull;
 }
 
+// The warps per SM up to which kHalf serves: what its registers allow, less
+// for the shortest searches (greedy, a beam of at most 32) over those FP32
+// rows, which spill in it: over 50,000 x 100 at ef 16, 2,200 queries took 148
+// us with 15 warps per SM of kHalf and 134 in blocks of four of kFull, 1,800
+// (12 warps) 136 and 128; with fewer warps, walked or from ef 64 on kHalf is
+// as fast or faster (1,000 queries at ef 16 124 against 131).
+template <typename VT, int DMAX>
+constexpr int half_warps(bool brief) {
+  if (most_in_flight<VT, DMAX>() == kFull) return 0;  // no variants
+  return brief && most_in_flight<VT, DMAX>() == kHalf ? 10 : 16;
+}
+
 // Chunks in flight for a launch of grid blocks: by the warps that can be
 // resident together on an SM -- the launch's share of them, or what the
-// shared memory leaves room for.  The lines are the warps that the variants'
-// registers allow.
-static int search_in_flight(int warps, int grid, size_t smem) {
+// shared memory leaves room for.
+static int search_in_flight(int warps, int grid, size_t smem, int half) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
@@ -1093,7 +1104,7 @@ static int search_in_flight(int warps, int grid, size_t smem) {
   const int by_smem = (int)((size_t)(227 * 1024) / (smem + 1024));
   const int blocks = std::min((grid + sms - 1) / sms, by_smem);
   if (blocks * warps <= 8) return kFew;
-  return blocks * warps <= 16 ? kHalf : kFull;
+  return blocks * warps <= half ? kHalf : kFull;
 }
 
 template <typename VT, int DMAX>
@@ -1102,7 +1113,7 @@ static cudaError_t launch_t(const SearchArgs& a, int warps, int grid, size_t sme
   constexpr int most = most_in_flight<VT, DMAX>();
   if constexpr (most != kFull) {
     if (a.team <= 1) {
-      const int f = search_in_flight(warps, grid, smem);
+      const int f = search_in_flight(warps, grid, smem, half_warps<VT, DMAX>(search_is_brief(a.ef_cap, a.ef_upper)));
       if (f == kHalf) kern = k_search<VT, DMAX, kHalf, Solo>;
       if (f == kFew) kern = k_search<VT, DMAX, most, Solo>;
     }
@@ -1558,16 +1569,15 @@ size_t search_team_smem(int ef_cap, int hash_bits, int dpad, int team) {
   return team > 1 ? b + sizeof(TeamJob) : b;
 }
 
-// whether the kernel of a storage type and row width has variants with more
-// chunks in flight
-static bool more_in_flight(int storage, int dpad) {
+// half_warps by storage type and row width
+static int more_in_flight(int storage, int dpad, bool brief) {
   auto of = [&](auto vt) {
     using VT = decltype(vt);
-    if (dpad <= 32) return most_in_flight<VT, 32>() != kFull;
-    if (dpad <= 64) return most_in_flight<VT, 64>() != kFull;
-    if (dpad <= 128) return most_in_flight<VT, 128>() != kFull;
-    if (dpad <= 512) return most_in_flight<VT, 512>() != kFull;
-    return most_in_flight<VT, 1024>() != kFull;
+    if (dpad <= 32) return half_warps<VT, 32>(brief);
+    if (dpad <= 64) return half_warps<VT, 64>(brief);
+    if (dpad <= 128) return half_warps<VT, 128>(brief);
+    if (dpad <= 512) return half_warps<VT, 512>(brief);
+    return half_warps<VT, 1024>(brief);
   };
   if (storage == HENN_BF16) return of(__nv_bfloat16());
   if (storage == HENN_FP8E4M3) return of(__nv_fp8_e4m3());
@@ -1588,7 +1598,7 @@ int search_hash_bits(int ef_cap) {
   return hb;
 }
 
-int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad) {
+int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad, bool brief) {
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms < 1)
     return kSearchWarps;
@@ -1597,7 +1607,7 @@ int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, in
   const int64_t r4 = std::min<int64_t>(most, 4 * (int64_t)(room / (4 * warp_smem + fixed)));
   const int64_t r1 = std::min<int64_t>(most, (int64_t)(room / (warp_smem + fixed)));
   if (4 * r1 >= 5 * r4) return 1;
-  return more_in_flight(storage, dpad) && nq < sms * std::min<int64_t>(r4, 16) ? 1 : kSearchWarps;
+  return nq < sms * std::min<int64_t>(r4, more_in_flight(storage, dpad, brief)) ? 1 : kSearchWarps;
 }
 
 cudaError_t search_persistent_grid(int device, int warps, size_t smem, int* grid) {

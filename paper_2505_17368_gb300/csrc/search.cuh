@@ -110,7 +110,9 @@ int search_hash_bits(int ef_cap);
 // that run with more rows in flight, which single warps spread more evenly
 // (2,000 queries over 100,000 x 960 BF16: 1,287 against 1,344 us).  Where
 // they do not, blocks of 4 stay.
-int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad);
+int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad, bool brief);
+// the shortest searches: greedy above a layer-0 beam of at most 32 entries
+inline bool search_is_brief(int ef_cap, int ef_upper) { return ef_cap <= 32 && ef_upper <= 1; }
 // Blocks of `warps` warps using `smem` bytes of shared memory each that
 // stay resident together on every SM of `device` (a persistent launch).
 cudaError_t search_persistent_grid(int device, int warps, size_t smem, int* grid);
