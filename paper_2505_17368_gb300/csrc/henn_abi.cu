@@ -383,6 +383,57 @@ struct henn_index {
     }
     return pool;
   }
+  // The last search on each stream (at most kFlights of them), for the choice
+  // of the next one's kernel: launches side by side share the SMs.  A hint:
+  // results do not depend on it.  As long as one stream searches the index
+  // nothing is recorded.  Skipped on streams that are being captured.
+  static constexpr size_t kFlights = 32;
+  struct Flight {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t done = nullptr;  // recorded behind its last search
+    int64_t warps = 0;           // that search's; 0: it is known to have ended
+  };
+  mutable std::mutex flight_mu;
+  mutable std::vector<Flight> flights;
+  static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+  }
+  // warps of searches that may be running on other streams than st
+  int64_t searches_beside(cudaStream_t st) const {
+    std::lock_guard<std::mutex> lk(flight_mu);
+    if (flights.size() < 2) return 0;
+    int64_t sum = 0;
+    BesideCaptures any;
+    for (Flight& f : flights) {
+      if (f.stream == st || !f.done || f.warps == 0) continue;
+      if (cudaEventQuery(f.done) == cudaErrorNotReady)
+        sum += f.warps;
+      else
+        f.warps = 0;
+      cudaGetLastError();  // not ready is no error
+    }
+    return sum;
+  }
+  void note_search(cudaStream_t st, int64_t warps) const {
+    std::lock_guard<std::mutex> lk(flight_mu);
+    Flight* mine = nullptr;
+    for (Flight& f : flights)
+      if (f.stream == st) mine = &f;
+    if (!mine && flights.size() < kFlights) {
+      flights.push_back(Flight());
+      mine = &flights.back();
+    }
+    for (size_t i = 0; !mine && i < flights.size(); ++i)
+      if (flights[i].warps == 0) mine = &flights[i];
+    if (!mine) return;
+    mine->stream = st;
+    if (flights.size() == 1 || capturing(st)) return;
+    if (!mine->done && cudaEventCreateWithFlags(&mine->done, cudaEventDisableTiming) != cudaSuccess) mine->done = nullptr;
+    mine->warps = mine->done && cudaEventRecord(mine->done, st) == cudaSuccess ? warps : 0;
+  }
   // events of the last search with time_kernel = 1
   mutable std::mutex time_mu;
   mutable cudaEvent_t tev[2] = {nullptr, nullptr};
@@ -405,6 +456,8 @@ struct henn_index {
     if (pool) cudaMemPoolDestroy(pool);  // (released once its last frees have run)
     for (cudaEvent_t e : tev)
       if (e) cudaEventDestroy(e);
+    for (Flight& f : flights)
+      if (f.done) cudaEventDestroy(f.done);
     for (cudaStream_t t : side) cudaStreamDestroy(t);
     for (void* p : gates) cudaFree(p);
     DevicePool& dp = device_pool(device);
@@ -1493,12 +1546,13 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
       require(idx->layers[top_exact].size <= (1 << (hb_min - 1)),
               "exact_method SORT: the exact layer must have <= 2^(hash_bits - 1) points (512 by default)");
     const int team = sp.team_size > 0 ? sp.team_size : 1;
+    const int64_t beside = idx->searches_beside(st);
     // warps per block of a launch of n queries with a beam capacity
     auto block_warps = [&](int64_t n, int cap, int bits) {
       if (sp.warps_per_block > 0) return (int)sp.warps_per_block;
       return team > 1 ? kSearchWarps
                       : search_block_warps(idx->device, n, search_warp_smem(cap, bits, idx->dpad), idx->storage,
-                                           idx->dpad, search_is_brief(cap, sp.ef_upper));
+                                           idx->dpad, search_is_brief(cap, sp.ef_upper), beside);
     };
     const int warps = block_warps(nq, ef_cap, hb);
     require(warps >= 1 && warps <= kSearchWarps, "warps_per_block must be in [1, 4]");
@@ -1695,7 +1749,7 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
       size_t smem = search_team_smem(ef_cap, hb, idx->dpad, team) * teams;
       int64_t blocks_needed = (nq + teams - 1) / teams;
       int grid = (int)std::min<int64_t>(persistent_grid(idx->device, warps, smem), blocks_needed);
-      CK(launch_search(a, warps, grid, st));
+      CK(launch_search(a, warps, grid, beside, st));
     } else {
       std::lock_guard<std::mutex> lk(idx->side_mu);
       while ((int)idx->side.size() < groups) {
@@ -1719,7 +1773,7 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
         size_t smem = search_team_smem(ag.ef_cap, ag.hash_bits, idx->dpad, team) * teams;
         int64_t blocks_needed = (count[g] + teams - 1) / teams;
         int grid = (int)std::min<int64_t>(persistent_grid(idx->device, gwarps, smem), blocks_needed);
-        CK(launch_search(ag, gwarps, grid, t));
+        CK(launch_search(ag, gwarps, grid, beside, t));
         cudaEvent_t join;
         CK(cudaEventCreateWithFlags(&join, cudaEventDisableTiming));
         CK(cudaEventRecord(join, t));
@@ -1728,6 +1782,7 @@ extern "C" henn_status henn_search(const henn_index* idx, const float* Q, int64_
       }
       cudaEventDestroy(fork);
     }
+    idx->note_search(st, std::min<int64_t>(nq, 24 * 152));  // a full launch's warps at most
     if (sp.time_kernel) {
       CK(cudaEventRecord(idx->tev[1], st));
       idx->t_launches = launches;

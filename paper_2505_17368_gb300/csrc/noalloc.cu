@@ -126,7 +126,7 @@ extern "C" henn_status henn_search_host_noalloc(const henn_index* idx, const flo
   a.counter = counter;
 
   const int warps = search_block_warps(device, nq, search_warp_smem(ef_cap, hb, a.dpad), a.storage, a.dpad,
-                                       search_is_brief(ef_cap, ef_upper));
+                                       search_is_brief(ef_cap, ef_upper), 0);
   const size_t smem = search_warp_smem(ef_cap, hb, a.dpad) * warps;
   int grid = 0;
   cudaError_t e = search_persistent_grid(device, warps, smem, &grid);
@@ -138,7 +138,7 @@ extern "C" henn_status henn_search_host_noalloc(const henn_index* idx, const flo
   // overwritten before it is read
   if ((e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st)) != cudaSuccess ||
       (e = cudaMemcpyAsync(dq, Q, (size_t)nq * a.d * sizeof(float), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = launch_search(a, warps, grid, st)) != cudaSuccess ||
+      (e = launch_search(a, warps, grid, 0, st)) != cudaSuccess ||
       (e = cudaMemcpyAsync(out_ids, dids, (size_t)nq * out_stride * sizeof(int64_t), cudaMemcpyDeviceToHost, st)) !=
           cudaSuccess ||
       (e = cudaMemcpyAsync(out_dists, dd, (size_t)nq * out_stride * sizeof(float), cudaMemcpyDeviceToHost, st)) !=

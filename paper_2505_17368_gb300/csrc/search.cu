@@ -52,8 +52,11 @@ namespace henn {
 // do not depend on the choice; search_in_flight has the rule.  Against the
 // full launch's kernel in blocks of four: 2,000 queries over 100,000 x 960
 // BF16 rows 1.81 -> 1.20 ms (kHalf); 1,000 over 50,000 x 100 FP8 at ef 200 844
-// -> 516 us, 64 over 1,000,000 x 128 BF16 429 -> 361 us, one over 50,000 x 32
-// FP32 171 -> 148 us (kFew).
+// -> 516 us, 64 over 1,000,000 x 128 BF16 429 -> 353 us, one over 50,000 x 32
+// FP32 171 -> 148 us (kFew).  Launches running side by side share an SM's
+// registers, so the rule counts theirs: 16 streams of 512 queries over 200,000
+// x 128 BF16, each launch taken by itself, ran 3.48 ms a round with kFew and
+// 2.02 with kFull.
 constexpr int kFull = 4, kHalf = 16, kFew = 32;
 template <int IF>
 struct SearchOcc {
@@ -1093,27 +1096,39 @@ constexpr int half_warps(bool brief) {
   return brief && most_in_flight<VT, DMAX>() == kHalf ? 10 : 16;
 }
 
-// Chunks in flight for a launch of grid blocks: by the warps that can be
-// resident together on an SM -- the launch's share of them, or what the
-// shared memory leaves room for.
-static int search_in_flight(int warps, int grid, size_t smem, int half) {
+// Rows that gain from kHalf also where the SMs are full (8 streams of 2,000
+// queries over 50,000 points, ef 64, against kFull: FP32 x 400 1.33 times the
+// speed, FP32 x 960 1.58, BF16 x 960 1.05; narrower BF16 and FP8 rows and FP32
+// ones of up to 128 values 0.81 - 0.97).
+template <typename VT, int DMAX>
+constexpr bool half_when_full() {
+  return (std::is_same<VT, float>::value && DMAX > 128) || (std::is_same<VT, __nv_bfloat16>::value && DMAX > 512);
+}
+
+// Chunks in flight for a launch of grid blocks: by the warps that will be
+// resident together on an SM -- the launch's share of them and those of
+// launches beside it (in all beside warps), or what the shared memory leaves
+// room for.
+static int search_in_flight(int warps, int grid, size_t smem, int half, int64_t beside, bool when_full) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
     return kFull;
-  const int by_smem = (int)((size_t)(227 * 1024) / (smem + 1024));
-  const int blocks = std::min((grid + sms - 1) / sms, by_smem);
-  if (blocks * warps <= 8) return kFew;
-  return blocks * warps <= half ? kHalf : kFull;
+  const int by_smem = (int)((size_t)(227 * 1024) / (smem + 1024)) * warps;
+  const int share = (grid + sms - 1) / sms * warps;
+  const int64_t all = std::min<int64_t>(share + (beside + sms - 1) / sms, by_smem);
+  if (all <= 8) return kFew;
+  return (when_full ? std::min(share, by_smem) : all) <= half ? kHalf : kFull;
 }
 
 template <typename VT, int DMAX>
-static cudaError_t launch_t(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
+static cudaError_t launch_t(const SearchArgs& a, int warps, int grid, size_t smem, int64_t beside, cudaStream_t st) {
   auto kern = a.team > 1 ? k_search<VT, DMAX, kFull, Team> : k_search<VT, DMAX, kFull, Solo>;
   constexpr int most = most_in_flight<VT, DMAX>();
   if constexpr (most != kFull) {
     if (a.team <= 1) {
-      const int f = search_in_flight(warps, grid, smem, half_warps<VT, DMAX>(search_is_brief(a.ef_cap, a.ef_upper)));
+      const int f = search_in_flight(warps, grid, smem, half_warps<VT, DMAX>(search_is_brief(a.ef_cap, a.ef_upper)),
+                                     beside, half_when_full<VT, DMAX>());
       if (f == kHalf) kern = k_search<VT, DMAX, kHalf, Solo>;
       if (f == kFew) kern = k_search<VT, DMAX, most, Solo>;
     }
@@ -1125,12 +1140,12 @@ static cudaError_t launch_t(const SearchArgs& a, int warps, int grid, size_t sme
 }
 
 template <typename VT>
-static cudaError_t launch_vt(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st) {
-  if (a.dpad <= 32) return launch_t<VT, 32>(a, warps, grid, smem, st);
-  if (a.dpad <= 64) return launch_t<VT, 64>(a, warps, grid, smem, st);
-  if (a.dpad <= 128) return launch_t<VT, 128>(a, warps, grid, smem, st);
-  if (a.dpad <= 512) return launch_t<VT, 512>(a, warps, grid, smem, st);
-  return launch_t<VT, 1024>(a, warps, grid, smem, st);
+static cudaError_t launch_vt(const SearchArgs& a, int warps, int grid, size_t smem, int64_t beside, cudaStream_t st) {
+  if (a.dpad <= 32) return launch_t<VT, 32>(a, warps, grid, smem, beside, st);
+  if (a.dpad <= 64) return launch_t<VT, 64>(a, warps, grid, smem, beside, st);
+  if (a.dpad <= 128) return launch_t<VT, 128>(a, warps, grid, smem, beside, st);
+  if (a.dpad <= 512) return launch_t<VT, 512>(a, warps, grid, smem, beside, st);
+  return launch_t<VT, 1024>(a, warps, grid, smem, beside, st);
 }
 
 template <typename VT, int DMAX>
@@ -1154,7 +1169,8 @@ static cudaError_t launch_serve_vt(const ServeArgs& a, int warps, int grid, size
 #ifndef HENN_SEARCH_ROWS  // the rest once, not per storage type
 
 #define HENN_DECLARE(T)                                                                                       \
-  cudaError_t launch_search_##T(const SearchArgs& a, int warps, int grid, size_t smem, cudaStream_t st);      \
+  cudaError_t launch_search_##T(const SearchArgs& a, int warps, int grid, size_t smem, int64_t beside,          \
+                                cudaStream_t st);                                                               \
   cudaError_t launch_serve_##T(const ServeArgs& a, int warps, int grid, size_t smem, cudaStream_t st);        \
   cudaError_t launch_probe_##T(const GreedyProbeArgs& a, cudaStream_t st);
 HENN_DECLARE(bf16)
@@ -1598,7 +1614,7 @@ int search_hash_bits(int ef_cap) {
   return hb;
 }
 
-int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad, bool brief) {
+int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad, bool brief, int64_t beside) {
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms < 1)
     return kSearchWarps;
@@ -1607,7 +1623,7 @@ int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, in
   const int64_t r4 = std::min<int64_t>(most, 4 * (int64_t)(room / (4 * warp_smem + fixed)));
   const int64_t r1 = std::min<int64_t>(most, (int64_t)(room / (warp_smem + fixed)));
   if (4 * r1 >= 5 * r4) return 1;
-  return nq < sms * std::min<int64_t>(r4, more_in_flight(storage, dpad, brief)) ? 1 : kSearchWarps;
+  return nq + beside < sms * std::min<int64_t>(r4, more_in_flight(storage, dpad, brief)) ? 1 : kSearchWarps;
 }
 
 cudaError_t search_persistent_grid(int device, int warps, size_t smem, int* grid) {
@@ -1630,16 +1646,16 @@ cudaError_t launch_serve(const ServeArgs& a, int warps_per_block, int grid, cuda
   return launch_serve_vt<float>(b, warps_per_block, grid, smem, st);
 }
 
-cudaError_t launch_search(const SearchArgs& a, int warps_per_block, int grid, cudaStream_t st) {
+cudaError_t launch_search(const SearchArgs& a, int warps_per_block, int grid, int64_t beside, cudaStream_t st) {
   SearchArgs b = a;
   const int team = a.team > 1 ? a.team : 1;
   if (warps_per_block % team != 0) return cudaErrorInvalidValue;
   b.team = team;
   b.warp_smem = (int32_t)search_team_smem(a.ef_cap, a.hash_bits, a.dpad, team);
   size_t smem = (size_t)b.warp_smem * (warps_per_block / team);
-  if (a.storage == HENN_BF16) return launch_search_bf16(b, warps_per_block, grid, smem, st);
-  if (a.storage == HENN_FP8E4M3) return launch_search_fp8(b, warps_per_block, grid, smem, st);
-  return launch_vt<float>(b, warps_per_block, grid, smem, st);
+  if (a.storage == HENN_BF16) return launch_search_bf16(b, warps_per_block, grid, smem, beside, st);
+  if (a.storage == HENN_FP8E4M3) return launch_search_fp8(b, warps_per_block, grid, smem, beside, st);
+  return launch_vt<float>(b, warps_per_block, grid, smem, beside, st);
 }
 
 #endif  // HENN_SEARCH_ROWS

@@ -110,7 +110,8 @@ int search_hash_bits(int ef_cap);
 // that run with more rows in flight, which single warps spread more evenly
 // (2,000 queries over 100,000 x 960 BF16: 1,287 against 1,344 us).  Where
 // they do not, blocks of 4 stay.
-int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad, bool brief);
+// (beside: warps of searches that run beside the launch, on other streams)
+int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad, bool brief, int64_t beside);
 // the shortest searches: greedy above a layer-0 beam of at most 32 entries
 inline bool search_is_brief(int ef_cap, int ef_upper) { return ef_cap <= 32 && ef_upper <= 1; }
 // Blocks of `warps` warps using `smem` bytes of shared memory each that
@@ -136,6 +137,6 @@ void launch_select_top32(const uint16_t* D, const float* cmin, int64_t nq, int64
                          uint64_t* out, bool discard, cudaStream_t st);
 cudaError_t launch_greedy_probe(const GreedyProbeArgs& a, int storage, cudaStream_t st);
 cudaError_t launch_serve(const ServeArgs& a, int warps_per_block, int grid, cudaStream_t st);
-cudaError_t launch_search(const SearchArgs& a, int warps_per_block, int grid, cudaStream_t st);
+cudaError_t launch_search(const SearchArgs& a, int warps_per_block, int grid, int64_t beside, cudaStream_t st);
 
 }  // namespace henn

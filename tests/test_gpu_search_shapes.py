@@ -117,3 +117,32 @@ def test_freed_indexes_give_their_memory_back():
     idx.close()
     # all but what the pool keeps once the last index is gone
     assert torch.cuda.mem_get_info()[0] - before >= held - (256 << 20) - (32 << 20)
+
+
+@pytest.mark.parametrize("storage,d", [(H.F32, 100), (H.BF16, 64), (H.FP8E4M3, 400)])
+def test_searches_side_by_side(storage, d):
+    """The launches of several streams choose their kernels by one another; the answers are those of one stream."""
+    X, Q = rand(8000, d, 21), rand(6 * 700, d, 22)
+    idx = H.Index(X, storage=storage, seed=9)
+    keys = torch.arange(len(Q), device="cuda", dtype=torch.int64)
+    want = idx.search(Q, k=10, ef=64, keys=keys)[:2]
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(t):
+        try:
+            stream = torch.cuda.Stream()
+            part = slice(700 * t, 700 * (t + 1))
+            out = [idx.search(Q[part], k=10, ef=64, keys=keys[part], stream=stream) for _ in range(12)]
+            stream.synchronize()
+            for ids, dd, _ in out:
+                assert torch.equal(ids, want[0][part]) and torch.equal(dd, want[1][part])
+        except Exception as e:  # reported below
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(6)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
