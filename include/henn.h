@@ -26,8 +26,9 @@
  *  - The caller owns every array it passes; the library copies what it
  *    keeps.  The index owns its device memory until henn_free().
  *  - Device memory comes from one pool per device, which keeps up to 1 GiB
- *    of unused memory between calls, and 256 MiB once the device's last
- *    index has been freed.
+ *    of unused memory between calls beside the indexes' arrays, and 256 MiB
+ *    once the device's last index has been freed (an exact k-NN call after
+ *    that may leave 1 GiB again).
  *  - No call throws.  Each returns a henn_status; on failure nothing is
  *    written to *out handles and henn_last_error() describes the failure.
  *  - A const index may be searched concurrently from several host threads

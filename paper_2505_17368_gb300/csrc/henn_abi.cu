@@ -69,14 +69,31 @@ static void* mapped_host(const void* p) {
 // mapped its gigabytes anew (of a 10,000 x 32 build, 2.4 ms, the kernels ran
 // 0.75 ms).  This pool keeps up to kPoolKeep of unused memory between calls
 // and gives all but kPoolIdle back when the device's last index is freed.
+// (A pool's release threshold counts what it has in use too, so it moves with
+// the size of the indexes' arrays.)
 constexpr uint64_t kPoolKeep = 1ull << 30;
 constexpr uint64_t kPoolIdle = 256ull << 20;
+
+struct Block {
+  void* p;
+  size_t bytes;
+};
 
 struct DevicePool {
   std::mutex mu;
   cudaMemPool_t pool = nullptr;
-  int64_t indexes = 0;  // alive on this device
-  std::vector<void*> parked;  // blocks of freed indexes that could not be waited for yet
+  int64_t indexes = 0;        // alive on this device
+  uint64_t held = 0;          // bytes of their arrays
+  uint64_t keep = 0;          // the release threshold set
+  std::vector<Block> parked;  // blocks of freed indexes that could not be waited for yet
+
+  // with mu held: the arrays' bytes have changed
+  void hold(int64_t bytes) {
+    held += (uint64_t)bytes;
+    uint64_t now = kPoolKeep + (held & ~((64ull << 20) - 1));  // in steps: small indexes leave it alone
+    if (!pool || now == keep) return;
+    if (cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &now) == cudaSuccess) keep = now;
+  }
 };
 
 DevicePool& device_pool(int device) {
@@ -96,9 +113,8 @@ cudaMemPool_t library_pool(int device) {
     props.location.id = device;
     cudaMemPool_t made = nullptr;
     CK(cudaMemPoolCreate(&made, &props));
-    uint64_t keep = kPoolKeep;
-    CK(cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep));
     p.pool = made;
+    p.hold(0);
   }
   return p.pool;
 }
@@ -268,7 +284,7 @@ struct henn_index {
   uint8_t* dead = nullptr;  // 1 per deleted point (allocated at the first delete)
   int64_t n_dead = 0;
   SearchLayer* d_layers = nullptr;
-  std::vector<void*> allocs;
+  std::vector<Block> allocs;
   int64_t bytes = 0;
   int64_t uncertified = 0;
   double build_seconds = 0.0;
@@ -318,8 +334,11 @@ struct henn_index {
       CK(cudaMallocFromPoolAsync(&p, b, lib, mem_stream));
     else
       CK(cudaMallocAsync(&p, b, mem_stream));
-    allocs.push_back(p);
+    allocs.push_back({p, b});
     bytes += (int64_t)b;
+    DevicePool& dp = device_pool(device);
+    std::lock_guard<std::mutex> lk(dp.mu);
+    dp.hold((int64_t)b);
     return static_cast<T*>(p);
   }
   // frees one allocation made by alloc(): nothing may run on the index beside
@@ -328,11 +347,14 @@ struct henn_index {
   void release(void* p) {
     if (!p) return;
     for (size_t i = 0; i < allocs.size(); ++i)
-      if (allocs[i] == p) {
+      if (allocs[i].p == p) {
         if (!drained) drained = drain();
         if (!drained) return;
         BesideCaptures any;
         cudaFree(p);
+        DevicePool& dp = device_pool(device);
+        std::lock_guard<std::mutex> lk(dp.mu);
+        dp.hold(-(int64_t)allocs[i].bytes);
         allocs.erase(allocs.begin() + (long)i);
         return;
       }
@@ -466,8 +488,14 @@ struct henn_index {
       allocs.insert(allocs.end(), dp.parked.begin(), dp.parked.end());
       dp.parked.clear();
     }
-    for (void* p : allocs)
-      if (!idle || cudaFree(p) != cudaSuccess) dp.parked.push_back(p);
+    int64_t freed = 0;
+    for (const Block& b : allocs) {
+      if (idle && cudaFree(b.p) == cudaSuccess)
+        freed += (int64_t)b.bytes;
+      else
+        dp.parked.push_back(b);
+    }
+    dp.hold(-freed);
     if (device < 64 && --dp.indexes == 0 && dp.pool) cudaMemPoolTrimTo(dp.pool, kPoolIdle);
     if (current != device) cudaSetDevice(current);
   }

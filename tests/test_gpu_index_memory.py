@@ -187,3 +187,18 @@ def test_insertion_that_runs_out_of_memory():
         assert all(np.array_equal(got[key], want[key]) for key in want)
         idx.close()
     assert refused >= 1
+
+
+def test_scratch_is_kept_beside_large_indexes():
+    """An index of over 1 GiB: its insertions' scratch (0.9 GB) stays in the pool between calls, and goes with it."""
+    idx = H.Index(rand(440_000, 512, 1), storage=H.BF16, seed=3)
+    new = rand(100, 512, 2).cpu().numpy()
+    idx.insert(new)  # the arrays have doubled: 880,000 rows
+    arrays = 880_000 * (512 * 6 + 32 * 4 + 16 * 8)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = torch.cuda.mem_get_info()[0]
+    idx.close()
+    back = torch.cuda.mem_get_info()[0] - before
+    # all but what the pool keeps once the last index is gone; the upper layers' arrays come on top
+    assert arrays + 850e6 - (256 << 20) <= back <= 1.1 * arrays + (1 << 30)
