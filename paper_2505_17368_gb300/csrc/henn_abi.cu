@@ -303,15 +303,15 @@ struct henn_index {
   // for pool memory, and searches on any stream may still read them.  Freeing
   // a cudaMalloc'ed block does wait for the device (cudaDeviceSynchronize does
   // too, but spoils any capture in progress, a build's in another thread for
-  // instance), so an index holds two small ones, gates, and frees one before
-  // its blocks: the operation in progress may use one up (begin makes up for
-  // it), and one is left for the destructor.  No allocation is needed to free.
+  // instance), so an index holds a small one, a gate, for its destructor to
+  // free before the blocks, and another for an operation that frees some.  No
+  // allocation is needed to free.
   std::vector<void*> gates;
-  void begin(cudaStream_t st) {
+  void begin(cudaStream_t st, size_t frees = 1) {  // frees: whether the operation may
     mem_stream = st;
     drained = false;
     BesideCaptures any;
-    while (gates.size() < 2) {
+    while (gates.size() < 1 + frees) {
       void* p = nullptr;
       CK(cudaMalloc(&p, 16));
       gates.push_back(p);
@@ -916,7 +916,7 @@ extern "C" henn_status henn_build(const float* X, int64_t n, int32_t d, int32_t 
     BuildTrace tr(st);
 
     ix = new henn_index();
-    ix->begin(st);
+    ix->begin(st, 0);
     ix->params = p;
     ix->n = n;
     ix->d = d;
