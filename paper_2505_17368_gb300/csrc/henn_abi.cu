@@ -1969,7 +1969,7 @@ namespace {
 void knn_sweep(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t dpad, int32_t k, int32_t metric,
               int64_t* out_ids, float* out_dists, Scratch& sc, cudaStream_t st) {
   const unsigned grid = sweep_grid();
-  uint64_t* lists = sc.get<uint64_t>(sweep_lists(grid, nq) * sweep_pool(k));
+  uint64_t* lists = sc.get<uint64_t>(sweep_lists(grid, nq, n) * sweep_pool(k));
   launch_sweep_knn(qp, nq, xp, n, dpad, metric, k, grid, lists, nullptr, nullptr, out_ids, out_dists, st);
 }
 
@@ -2034,7 +2034,7 @@ void knn_tiles(const float* xp, int64_t n, const float* qp, int64_t nq, int32_t 
   flagged.count = over + nb + 1;
   int32_t* err = over + nb + 2;
   const unsigned sgrid = sweep_grid();
-  uint64_t* slists = sc.get<uint64_t>(sweep_lists(sgrid, nb) * sweep_pool(k));
+  uint64_t* slists = sc.get<uint64_t>(sweep_lists(sgrid, nb, n) * sweep_pool(k));
   const double tile_u = tc_tile_unit_error(dk);
   for (int64_t q0 = 0; q0 < nq; q0 += nb) {
     const int64_t c = std::min(nb, nq - q0);

@@ -191,7 +191,7 @@ void launch_exact_rows(const float* xw, const int32_t* ids, int64_t s, int32_t d
 // Exact k results by a scan of all n columns (rowsel / count, nullable: of
 // the queries rowsel[0 .. *count - 1] only, their number on the device).
 // Each block of kSweepRows queries has sweep_runs runs of columns (at least 128
-// columns each), shared out over sweep_grid() CTAs; lists: sweep_lists(grid, nq)
+// columns each), shared out over sweep_grid() CTAs; lists: sweep_lists(grid, nq, n)
 // lists of sweep_pool(k) keys.
 constexpr int kSweepRows = 32;
 constexpr int kSweepMaxRuns = 128;
@@ -220,9 +220,10 @@ __host__ __device__ inline int32_t sweep_runs(unsigned grid, int64_t rows, int64
   return (int32_t)(pick < most ? pick : most);
 }
 // for any number of rows up to nq
-inline size_t sweep_lists(unsigned grid, int64_t nq) {
-  const int64_t blocks = (nq + kSweepRows - 1) / kSweepRows;
-  const int64_t runs = (int64_t)kSweepItems * grid < blocks * kSweepMaxRuns ? (int64_t)kSweepItems * grid : blocks * kSweepMaxRuns;
+inline size_t sweep_lists(unsigned grid, int64_t nq, int64_t n) {
+  const int64_t blocks = (nq + kSweepRows - 1) / kSweepRows, parts = (n + 127) / 128;
+  const int64_t most = blocks * (parts < kSweepMaxRuns ? parts : kSweepMaxRuns);
+  const int64_t runs = (int64_t)kSweepItems * grid < most ? (int64_t)kSweepItems * grid : most;
   return (size_t)kSweepRows * (size_t)(blocks > runs ? blocks : runs);
 }
 inline int32_t sweep_pool(int32_t k) { return k <= 32 ? 32 : (k <= 64 ? 64 : 128); }

@@ -109,7 +109,9 @@ int search_hash_bits(int ef_cap);
 // 32 - 512: 2.7 against 3.1 ms), and for launches of under 16 warps per SM
 // that run with more rows in flight, which single warps spread more evenly
 // (2,000 queries over 100,000 x 960 BF16: 1,287 against 1,344 us).  Where
-// they do not, blocks of 4 stay.
+// they do not, blocks of 4 stay.  (Counted against the whole 227 KB; the grid
+// below stops at 200 KB, so that beams of 256 and 512 entries run up to a
+// fifth fewer warps than this rule weighs.)
 // (beside: warps of searches that run beside the launch, on other streams)
 int search_block_warps(int device, int64_t nq, size_t warp_smem, int storage, int dpad, bool brief, int64_t beside);
 // the shortest searches: greedy above a layer-0 beam of at most 32 entries
