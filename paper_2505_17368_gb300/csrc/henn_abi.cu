@@ -1271,8 +1271,10 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
     // ---- room for them: every array grows and the scratch is taken before
     // anything else changes, so that a call that runs out of memory leaves the
     // index as it was (the table on the device pointing at its arrays)
+    bool grown = false;
     auto grow = [&] {
       if (n1 > ix->cap_n) {
+        grown = true;
         const int64_t cap = std::max(n1, 2 * ix->cap_n);
         const bool aliased = ix->xw == ix->x32;
         ix->x32 = regrow(ix, ix->x32, (size_t)n0 * dpad, (size_t)cap * dpad, st);
@@ -1292,6 +1294,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
         const bool vec_aliased = li == 0 && ix->storage == HENN_F32;
         if (vec_aliased) Ly.vec = ix->xw;
         if (s1 <= Ly.cap) continue;
+        grown = true;
         const int64_t cap = std::max(s1, 2 * Ly.cap);
         if (li >= 1) {
           Ly.ids = regrow(ix, Ly.ids, (size_t)s0, (size_t)cap, st);
@@ -1313,7 +1316,7 @@ extern "C" henn_status henn_insert(henn_index* ix, const float* X, int64_t n_new
       write_layer_table(ix, st);
       throw;
     }
-    write_layer_table(ix, st);
+    if (grown) write_layer_table(ix, st);
     Scratch sc(st, library_pool(ix->device));
     const int64_t s_max = ix->layers[0].size + n_new;  // layer 0 holds every point
     const int64_t c_upper = ix->L >= 1 ? (int64_t)add[1].size() : 0;
