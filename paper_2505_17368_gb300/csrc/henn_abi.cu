@@ -1198,28 +1198,29 @@ bool insert_lists(henn_index* ix, const LayerDev& Ly, const int32_t* lids, int64
   const int32_t dpad = ix->dpad, M = ix->M, KP = 32, dk = round_up(dpad, 64);
   Scratch sc(st, library_pool(ix->device));
   try {
+    // (each launch before the next one's buffers: the device does not wait for them)
     float* partial = sc.get<float>((size_t)mean_chunks(s1) * dpad);
     float* mean = sc.get<float>(dpad);
+    launch_layer_mean(ix->xw, lids, s1, dpad, partial, mean, st);
     uint16_t* hi = sc.get<uint16_t>((size_t)s1 * dk);
     uint16_t* lo = sc.get<uint16_t>((size_t)s1 * dk);
     float* norms = sc.get<float>(s1);
     float* nmax = sc.get<float>(1);
+    launch_order_split(ix->xw, lids, s1, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, norms, nmax, st);
     const int32_t splits = tile_list_splits(c, s1, false);
     uint64_t* lists = sc.get<uint64_t>((size_t)splits * c * KP);
     uint64_t* cand = splits > 1 ? sc.get<uint64_t>((size_t)c * KP) : lists;
     int32_t* err = sc.get<int32_t>(2);  // the tile launch's error flag, the flagged rows' number
+    CK(cudaMemsetAsync(err, 0, 2 * sizeof(int32_t), st));
     float* thr = sc.get<float>(c);
     float* lthr = splits > 1 ? sc.get<float>((size_t)splits * c) : thr;
+    CK(launch_tile_lists_tc(hi + (size_t)s0 * dk, lo + (size_t)s0 * dk, norms + s0, c, hi, lo, norms, s1, dk, 2, drows,
+                            splits, lists, lthr, err, st));
+    if (splits > 1) launch_merge_lists(lists, lthr, c, splits, KP, cand, thr, st);
     FlaggedRows flagged;
     flagged.count = err + 1;
     flagged.rows = sc.get<int32_t>(c);
     flagged.thr = sc.get<float>(c);
-    launch_layer_mean(ix->xw, lids, s1, dpad, partial, mean, st);
-    launch_order_split(ix->xw, lids, s1, dpad, 0, 0, true, mean, dk, hi, lo, nullptr, norms, nmax, st);
-    CK(cudaMemsetAsync(err, 0, 2 * sizeof(int32_t), st));
-    CK(launch_tile_lists_tc(hi + (size_t)s0 * dk, lo + (size_t)s0 * dk, norms + s0, c, hi, lo, norms, s1, dk, 2, drows,
-                            splits, lists, lthr, err, st));
-    if (splits > 1) launch_merge_lists(lists, lthr, c, splits, KP, cand, thr, st);
     launch_rerank_fwd(ix->xw, lids, c, s0, dpad, ix->metric, nullptr, cand, thr, s1, true, true, KP, M, norms + s0,
                       nmax, tc_tile_unit_error(dk), Ly.fwd, Ly.fwd_d, flagged, st);
     CKL("rerank");
