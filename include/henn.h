@@ -162,6 +162,7 @@ henn_status henn_build(const float* X, int64_t n, int32_t d, int32_t x_on_device
  * for the call where it fits (M <= 16); where it does not, the new rows are
  * scanned without it, more slowly.  NSW graphs only (HENN_ERR_UNSUPPORTED
  * for kNN graphs, where earlier points' own lists would change).
+ * HENN_ERR_OOM leaves the index as it was.
  * Synchronises `stream` before returning.  Not safe concurrently with searches on idx;
  * servers made from idx before the call still point at the old arrays and
  * must be destroyed first.
@@ -182,7 +183,10 @@ henn_status henn_insert(henn_index* idx, const float* X, int64_t n_new, int32_t 
  * 0 keeps every point.  Servers made from idx before the call do not see
  * it and must be destroyed first.  Not safe concurrently with searches on
  * idx.  Synchronises `stream`.  Errors: HENN_ERR_INVALID_ARG for an id out
- * of range; a failed resampling as henn_build (HENN_ERR_EPSNET_NOT_FOUND).
+ * of range; HENN_ERR_CUDA on a stream that is being captured; a failed
+ * resampling as henn_build (HENN_ERR_EPSNET_NOT_FOUND, HENN_ERR_OOM): the
+ * points are deleted then, and the index goes on without the layers that
+ * were to be rebuilt.
  */
 henn_status henn_delete(henn_index* idx, const int64_t* ids, int64_t n, void* stream);
 

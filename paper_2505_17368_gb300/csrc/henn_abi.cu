@@ -1026,8 +1026,9 @@ void write_layer_table(henn_index* ix, cudaStream_t st) {
 
 // The same after the number of layers changed.
 void upload_layer_table(henn_index* ix, cudaStream_t st) {
+  SearchLayer* table = ix->alloc<SearchLayer>((size_t)ix->L + 1);
   ix->release(ix->d_layers);
-  ix->d_layers = ix->alloc<SearchLayer>((size_t)ix->L + 1);
+  ix->d_layers = table;
   write_layer_table(ix, st);
 }
 
@@ -1035,7 +1036,8 @@ void upload_layer_table(henn_index* ix, cudaStream_t st) {
 // liveids, at positions livepos of layer i - 1) and every layer above it
 // rebuilt: membership (Alg. 1 + Alg. 2 or Alg. 3, the build's seed and
 // layer numbers), down pointers into layer i - 1's arrays (which keep
-// their dead entries), graphs and traversal copies.
+// their dead entries), graphs and traversal copies.  Should that fail (no
+// memory), the index goes on with the layers below i.
 void rebuild_from(henn_index* ix, int32_t i, const std::vector<int32_t>& liveids, const std::vector<int32_t>& livepos) {
   const henn_build_params& p = ix->params;
   struct OwnStream {
@@ -1052,43 +1054,54 @@ void rebuild_from(henn_index* ix, int32_t i, const std::vector<int32_t>& liveids
   ix->begin(st);
   BuildTrace tr(st);
   ix->drop_entry_ops();
-  for (int32_t li = ix->L; li >= i; --li) {
-    LayerDev& Ly = ix->layers[li];
-    for (void* q : {(void*)Ly.ids, (void*)Ly.down, (void*)Ly.adj, (void*)Ly.fwd, (void*)Ly.fwd_d, Ly.vec,
-                    (void*)Ly.vscale})
-      ix->release(q);
+  auto drop = [&] {  // the layers from i on
+    for (int32_t li = (int32_t)ix->layers.size() - 1; li >= i; --li) {
+      LayerDev& Ly = ix->layers[li];
+      for (void* q : {(void*)Ly.ids, (void*)Ly.down, (void*)Ly.adj, (void*)Ly.fwd, (void*)Ly.fwd_d, Ly.vec,
+                      (void*)Ly.vscale})
+        ix->release(q);
+    }
+    ix->layers.resize(i);
+    ix->attempts.resize(i);
+    ix->ambiguous.resize(i);
+    ix->L = i - 1;
+  };
+  drop();
+  try {
+    {
+      Scratch sc(st, library_pool(ix->device));
+      int32_t* prev = sc.get<int32_t>(liveids.size());
+      CK(cudaMemcpyAsync(prev, liveids.data(), sizeof(int32_t) * liveids.size(), cudaMemcpyHostToDevice, st));
+      CapturedGraph attempt_graph;
+      build_membership(ix, p, i, prev, (int64_t)liveids.size(), attempt_graph, tr, st);
+    }
+    if ((int32_t)ix->layers.size() > i) {
+      // the first new layer's down pointers: positions in the live list -> in layer i - 1
+      LayerDev& F = ix->layers[i];
+      std::vector<int32_t> dn((size_t)F.size);
+      CK(cudaMemcpyAsync(dn.data(), F.down, sizeof(int32_t) * dn.size(), cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      for (int32_t& v : dn) v = livepos[(size_t)v];
+      CK(cudaMemcpyAsync(F.down, dn.data(), sizeof(int32_t) * dn.size(), cudaMemcpyHostToDevice, st));
+      CK(cudaStreamSynchronize(st));
+    }
+    ix->L = (int32_t)ix->layers.size() - 1;
+    CapturedGraph layer_graph;
+    for (int32_t li = i; li <= ix->L; ++li) {
+      LayerDev& Ly = ix->layers[li];
+      Ly.cap = Ly.size;
+      Ly.adj = ix->alloc<int32_t>((size_t)Ly.size * kMmax);
+      Ly.fwd = ix->alloc<int32_t>((size_t)Ly.size * ix->M);
+      Ly.fwd_d = ix->alloc<float>((size_t)Ly.size * ix->M);
+      build_layer_graph(ix, p, li, layer_graph, st, tr);
+    }
+    upload_layer_table(ix, st);
+  } catch (...) {
+    cudaStreamSynchronize(st);  // what was enqueued for the layers to be dropped
+    drop();
+    write_layer_table(ix, st);
+    throw;
   }
-  ix->layers.resize(i);
-  ix->attempts.resize(i);
-  ix->ambiguous.resize(i);
-  {
-    Scratch sc(st, library_pool(ix->device));
-    int32_t* prev = sc.get<int32_t>(liveids.size());
-    CK(cudaMemcpyAsync(prev, liveids.data(), sizeof(int32_t) * liveids.size(), cudaMemcpyHostToDevice, st));
-    CapturedGraph attempt_graph;
-    build_membership(ix, p, i, prev, (int64_t)liveids.size(), attempt_graph, tr, st);
-  }
-  if ((int32_t)ix->layers.size() > i) {
-    // the first new layer's down pointers: positions in the live list -> in layer i - 1
-    LayerDev& F = ix->layers[i];
-    std::vector<int32_t> dn((size_t)F.size);
-    CK(cudaMemcpyAsync(dn.data(), F.down, sizeof(int32_t) * dn.size(), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-    for (int32_t& v : dn) v = livepos[(size_t)v];
-    CK(cudaMemcpyAsync(F.down, dn.data(), sizeof(int32_t) * dn.size(), cudaMemcpyHostToDevice, st));
-    CK(cudaStreamSynchronize(st));
-  }
-  ix->L = (int32_t)ix->layers.size() - 1;
-  CapturedGraph layer_graph;
-  for (int32_t li = i; li <= ix->L; ++li) {
-    LayerDev& Ly = ix->layers[li];
-    Ly.cap = Ly.size;
-    Ly.adj = ix->alloc<int32_t>((size_t)Ly.size * kMmax);
-    Ly.fwd = ix->alloc<int32_t>((size_t)Ly.size * ix->M);
-    Ly.fwd_d = ix->alloc<float>((size_t)Ly.size * ix->M);
-    build_layer_graph(ix, p, li, layer_graph, st, tr);
-  }
-  upload_layer_table(ix, st);
 }
 
 // Delete of App. C after the tombstones are set: the lowest upper layer i

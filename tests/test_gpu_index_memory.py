@@ -202,3 +202,30 @@ def test_scratch_is_kept_beside_large_indexes():
     back = torch.cuda.mem_get_info()[0] - before
     # all but what the pool keeps once the last index is gone; the upper layers' arrays come on top
     assert arrays + 850e6 - (256 << 20) <= back <= 1.1 * arrays + (1 << 30)
+
+
+def test_deletion_whose_rebuild_runs_out_of_memory():
+    """The upper layers go, the index answers from what is left, without the deleted points."""
+    X = rand(3_000_000, 16, 12)
+    idx = H.Index(X, storage=H.BF16, seed=5)
+    upper = idx.layer(1)["ids"]
+    gone = np.concatenate([upper[: 2 * len(upper) // 3], np.arange(0, 3_000_000, 1000)])
+    Q = X[:300].cpu().numpy()
+    idx.search(Q, k=10, ef=128)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    # the rings of layer 1 want 1.2 GB, the pool keeps 1 GiB at most
+    full = torch.empty(torch.cuda.mem_get_info()[0] - (64 << 20), dtype=torch.uint8, device="cuda")
+    with pytest.raises(H.HennError) as e:
+        idx.delete(gone)
+    assert e.value.status == 2
+    assert len(idx.info()["sizes"]) == 1 and idx.info()["L"] == 0
+    ids = idx.search(Q, k=10, ef=128)[0]
+    del full
+    dead = np.zeros(3_000_000, bool)
+    dead[gone] = True
+    assert (ids >= 0).all() and not dead[ids].any()
+    assert np.array_equal(idx.search(Q, k=10, ef=128)[0], ids)
+    idx.delete(np.arange(5, 100_000, 7))
+    again = idx.search(Q, k=10, ef=128)[0]
+    assert (again >= 0).all() and not (again % 7 == 5)[again < 100_000].any()
